@@ -173,7 +173,8 @@ int scint_spectrum_rec(const scint_params* p, double* s_rec, uint64_t* counts, i
  * dq = 1/L, J = min(n_bins - 1, N/2): the integral of Eq. crec between the
  * paper's q_min = 1/L and q_max = 1/(2 Delta_1) by the midpoint rule on the
  * annuli, with J0 from the CUDA math library; and R_diff^rec, the root of
- * D_rec(R) = 1, by 64 bisection steps on (0, L/2] (NaN if D_rec(L/2) < 1).
+ * D_rec(R) = 1, by bisection on (0, L/2] to a bracket of L 2^-65 (NaN if D_rec(L/2) < 1);
+ * the last steps bisect D_rec's interpolating polynomial over the narrow bracket.
  * s_rec may be scint_spectrum_rec's output or any spectrum sampled at q_j
  * (e.g. the theoretical S_phi, as in the paper's comparison).
  *   s_rec   device, n_bins >= 2 doubles, read.
@@ -181,7 +182,7 @@ int scint_spectrum_rec(const scint_params* p, double* s_rec, uint64_t* counts, i
  *           (both may be NULL when n_r == 0).
  *   r_rec   device, 1 double written, or NULL to skip the root.
  * Each D_rec value is summed in a fixed order (reproducible bit for bit).
- * Needs workspace (< 1 KB) when r_rec != NULL.
+ * Needs workspace (1280 bytes) when r_rec != NULL.
  */
 int scint_structure_function_rec(const scint_params* p, const double* s_rec, int n_bins,
                                  const double* r_km, int n_r, double* d_rec, double* r_rec,

@@ -1449,8 +1449,8 @@ int scint_structure_function_rec(const scint_params* p, const double* s_rec, int
         if (rc) return rc;
         BisectState* st = c.take<BisectState>(sizeof(BisectState));
         const int rc2 = launch_timed(K_CREC, 8.0 * a.J, 0.0, s,
-                                     [&] { return launch_bisect(a, st, kRdiffRecIterations, r_rec, s); },
-                                     kRdiffRecIterations + 1);
+                                     [&] { return launch_bisect(a, st, p->n, kRdiffRecIterations, r_rec, s); },
+                                     bisect_launches(p->n));
         if (rc2) return rc2;
     }
     return ok();

@@ -195,8 +195,9 @@ cudaError_t launch_curve_moments(const float* curves, int n_curves, int n_sample
 // ---- screen check of Sect. 3.1.1 (screen_check.cu) --------------------------------
 constexpr int kRadialThreads = 512;
 constexpr int kCrecThreads = 256;
-constexpr int kBisectBlocks = 128;
-// Annulus sums of |F|^2 and bin counts (rows walked by `blocks` persistent
+constexpr int kCrecSplit = 8;       // blocks (one cluster) per lag
+constexpr int kBisectBlocks = 148;  // blocks of a root round, shared between its points (and BisectState within 1280 bytes)
+// Annulus sums of |F|^2 and bin counts (an octant of the spectrum walked by `blocks` persistent
 // blocks, n_hist annuli in shared memory), then S_rec = sum / count * inv_l2.
 // s_rec and counts must be zero on entry.
 cudaError_t launch_radial_spectrum(const SynthArgs& a, double inv_l2, int n_hist, double* s_rec,
@@ -214,7 +215,10 @@ struct BisectState {
     double partial[kBisectBlocks];
 };
 cudaError_t launch_crec(const CrecArgs& a, const double* r_km, int n_r, double* d, cudaStream_t s);
-cudaError_t launch_bisect(const CrecArgs& a, BisectState* st, int iterations, double* out, cudaStream_t s);
+static_assert(sizeof(BisectState) <= 1280, "the root's workspace");
+// n: grid size (the number of bisection rounds); iterations: total bisection steps
+cudaError_t launch_bisect(const CrecArgs& a, BisectState* st, int n, int iterations, double* out, cudaStream_t s);
+int bisect_launches(int n);
 
 
 // ---- light-curve time analysis (timeseries.cu) -------------------------------------

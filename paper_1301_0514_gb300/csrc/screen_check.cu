@@ -9,15 +9,16 @@
 //   R_diff^rec = root of D_rec(R) = 1, bisection on (0, L/2].
 //
 // The annulus sums run as one persistent pass: each block keeps a histogram of
-// every annulus in shared memory, walks whole spectral rows (each thread a
-// contiguous run of columns, adding into its current annulus until it changes,
-// so a run of equal annuli costs one shared atomic), and adds its histogram
-// into the global one at the end.  The sums are 64-bit fixed point (see
-// annulus_shift), hence exact and independent of the order of the additions;
-// the hot loop has no FP64 operation (GB300's FP64 pipe is narrow).  The noise is regenerated per bin
-// (spectrum.cuh), never stored.  The bisection launches one kernel per step;
-// within a step the blocks' partial sums are combined in block order by the
+// every annulus in shared memory, its warps walk one octant of the spectrum (radial_kernel
+// below), and the block adds its histogram into the global one at the end.  The sums are 64-bit
+// fixed point (see annulus_shift), hence exact and independent of the order of the additions;
+// outside the FP64 square the loop has no FP64 operation (GB300's FP64 pipe is narrow).  The noise is
+// regenerated per bin (spectrum.cuh), never stored.  The root takes a few launches (bisect_kernel);
+// within one the blocks' partial sums are combined in a fixed order by the
 // last block to finish, so the result does not depend on scheduling.
+#include <cmath>
+
+#include <cooperative_groups.h>
 #include <math_constants.h>
 
 #include "dispatch.cuh"
@@ -68,10 +69,35 @@ SCINT_DEV unsigned long long to_fixed(double v, int s) {
     return e >= 0 ? m << e : (e > -53 ? m >> -e : 0ull);
 }
 
+// The bins of one octant, 0 <= ax <= ay <= n/2 (a = |m|), stand for the whole grid: up to eight
+// bins (+-ax, +-ay), (+-ay, +-ax) share |m|^2 and so the annulus, its shift and the amplitude
+// (one index search, one powf and one log2 per eight bins; the noise of each bin stays its own).
+// A warp takes kSeg cells of a spectral row ay, each lane kRun of them in a row, in the
+// direction in which the annulus changes slowly (at most 0.71 per cell), and adds a run of
+// cells of one annulus in a register before it goes to the block's shared histogram.  The sums
+// are the same integers as bin by bin.  At n = 14000: sums 2.16 -> 1.17 ms (328 -> 176 warp
+// instructions per 32 bins; Philox and the two branches of -ln u remain, issue 76 %), counts
+// 0.35 -> 0.07 ms, against whole rows per block and a powf and an annulus search per bin.  The tasks go round the
+// blocks, so that the rows ay <= low_k, drawn in FP64, spread over all SMs.
+constexpr int kRun = 4, kSeg = 32 * kRun;
+
+// number of (row, segment) tasks of rows 0..h
+__host__ __device__ constexpr int radial_tasks(int h) {
+    const int G = h / kSeg;
+    return kSeg * (G * (G + 1) / 2) + (h + 1 - G * kSeg) * (G + 1);
+}
+// task -> (row ay, first cell): rows [g kSeg, (g + 1) kSeg) have g + 1 segments each
+SCINT_DEV void radial_task(int task, int& ay, int& ax0) {
+    int g = (int)((sqrtf(8.0f * ((float)task / kSeg) + 1.0f) - 1.0f) * 0.5f);
+    while (kSeg * ((g + 1) * (g + 2) / 2) <= task) ++g;
+    while (kSeg * (g * (g + 1) / 2) > task) --g;
+    const int rem = task - kSeg * (g * (g + 1) / 2);
+    ay = g * kSeg + rem / (g + 1);
+    ax0 = (rem % (g + 1)) * kSeg;
+}
+
 // COUNT: bins per annulus.  Otherwise: fixed-point sums of |F|^2 (high bins from
-// their FP32 value, low bins from their FP64 value, as the synthesis draws them);
-// a thread adds a run of bins of one annulus in a register and the run into the
-// block's shared histogram with one atomic.
+// their FP32 value, low bins from their FP64 value, as the synthesis draws them).
 template <bool COUNT>
 __global__ void __launch_bounds__(kRadialThreads)
 radial_kernel(SynthArgs a, int n_hist, unsigned long long* sums, unsigned long long* counts) {
@@ -83,17 +109,24 @@ radial_kernel(SynthArgs a, int n_hist, unsigned long long* sums, unsigned long l
         else hs[j] = 0ull;
     }
     __syncthreads();
-    const int n = a.n;
-    const int chunk = (n + blockDim.x - 1) / blockDim.x;
-    const int x0 = threadIdx.x * chunk, x1 = min(n, x0 + chunk);
-    for (int ky = blockIdx.x; ky < n; ky += gridDim.x) {
-        const int my = signed_freq(ky, n);
+    const int n = a.n, h = n / 2;
+    const int tasks = radial_tasks(h), lane = threadIdx.x & 31;
+    const int warps = gridDim.x * (kRadialThreads / 32);
+#pragma unroll 1
+    for (int task = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; task < tasks; task += warps) {
+        int ay, ax0;
+        radial_task(task, ay, ax0);
+        ax0 += lane * kRun;
         int cur = -1, shift = 0;
         unsigned long long acc = 0ull;
         unsigned cnt = 0u;
-        for (int kx = x0; kx < x1; ++kx) {
-            const int mx = signed_freq(kx, n);
-            const int m2 = mx * mx + my * my;
+        // frequency -h and its mirror are one bin, and so is 0
+        const bool two_y = ay != 0 && ay != h;
+#pragma unroll 1
+        for (int i = 0; i < kRun; ++i) {
+            const int ax = ax0 + i;
+            if (ax > ay) break;
+            const int m2 = ax * ax + ay * ay;
             const int j = annulus_of(m2);
             if (j != cur) {
                 if (cur >= 0 && cur < n_hist) {
@@ -105,11 +138,30 @@ radial_kernel(SynthArgs a, int n_hist, unsigned long long* sums, unsigned long l
                 cnt = 0u;
                 if (!COUNT) shift = annulus_shift(a, j);
             }
+            const bool two_x = ax != 0 && ax != h;
             if (COUNT) {
-                ++cnt;
+                cnt += (two_x ? 2u : 1u) * (two_y ? 2u : 1u) * (ax != ay ? 2u : 1u);
             } else if (j < n_hist && m2 > 0) {
-                const u32x4 w = philox4x32_10(u32x4{(uint32_t)kx, (uint32_t)ky, a.screen_id, 0u}, a.key0, a.key1);
-                acc += low_bin(a, mx, my) ? to_fixed(power_low(a, w, m2), shift) : to_fixed(power_high(a, w, m2), shift);
+                const bool low = ay <= a.low_k;    // ax <= ay
+                const double sig_low = low ? amplitude_low(a, m2) : 0.0, sig2_low = sig_low * sig_low;
+                const float sig = low ? 0.0f : amplitude_high(a, m2), sig2 = sig * sig;
+                // (ax, ay) and, off the diagonal, (ay, ax); each with both signs of both
+#pragma unroll 1
+                for (int q = 0; q < (ax != ay ? 4 : 2); ++q) {
+                    const int px = q < 2 ? ax : ay, py = q < 2 ? ay : ax;
+                    const bool two_px = q < 2 ? two_x : two_y, two_py = q < 2 ? two_y : two_x;
+                    if ((q & 1) && !two_py) continue;
+                    const uint32_t ky = (uint32_t)((q & 1) ? n - py : py);
+                    const u32x4 w = philox4x32_10(u32x4{(uint32_t)px, ky, a.screen_id, 0u}, a.key0, a.key1);
+                    const u32x4 v = philox4x32_10(u32x4{(uint32_t)(n - px), ky, a.screen_id, 0u}, a.key0, a.key1);
+                    if (low) {
+                        acc += to_fixed(sig2_low * (2.0 * neg_log_ua64(w)), shift);
+                        if (two_px) acc += to_fixed(sig2_low * (2.0 * neg_log_ua64(v)), shift);
+                    } else {
+                        acc += to_fixed(sig2 * (2.0f * neg_log_ua32(w)), shift);
+                        if (two_px) acc += to_fixed(sig2 * (2.0f * neg_log_ua32(v)), shift);
+                    }
+                }
             }
         }
         if (cur >= 0 && cur < n_hist) {
@@ -173,33 +225,63 @@ SCINT_DEV double block_sum_fixed(double v, double* red) {
     return t;
 }
 
+// A lag's sum over a cluster of kCrecSplit blocks (7000 J0 terms keep one SM's narrow FP64 pipe
+// busy for 0.14 ms, and a call has fewer lags than the GPU has SMs: 48 lags 144 -> 56 us), block
+// partials added in rank order through distributed shared memory.
 __global__ void __launch_bounds__(kCrecThreads) crec_kernel(CrecArgs a, const double* r_km, int n_r, double* d) {
     __shared__ double red[kCrecThreads];
-    const int i = blockIdx.x;
-    const double acc = crec_terms(a.s, a.J, a.dq, r_km[i], 1 + threadIdx.x, blockDim.x);
+    __shared__ double part;
+    auto cl = cooperative_groups::this_cluster();
+    const int rank = (int)cl.block_rank(), i = blockIdx.x / kCrecSplit;
+    const double acc = crec_terms(a.s, a.J, a.dq, r_km[i], 1 + rank * (int)blockDim.x + (int)threadIdx.x,
+                                  kCrecSplit * (int)blockDim.x);
     const double t = block_sum_fixed(acc, red);
-    if (threadIdx.x == 0) d[i] = 4.0 * kPi * a.dq * t;
+    if (threadIdx.x == 0) part = t;
+    cl.sync();
+    if (rank == 0 && threadIdx.x == 0) {
+        double tot = 0.0;
+        for (int k = 0; k < kCrecSplit; ++k) tot += *cl.map_shared_rank(&part, k);
+        d[i] = 4.0 * kPi * a.dq * tot;
+    }
+    cl.sync();    // no block leaves before its partial is read
 }
 
 cudaError_t launch_crec(const CrecArgs& a, const double* r_km, int n_r, double* d, cudaStream_t s) {
-    crec_kernel<<<n_r, kCrecThreads, 0, s>>>(a, r_km, n_r, d);
-    return cudaGetLastError();
+    return launch_k(crec_kernel, kCrecSplit, dim3(n_r * kCrecSplit), dim3(kCrecThreads), 0, s, a, r_km, n_r, d);
 }
 
-// One bisection step.  Step -1 evaluates D_rec(L/2) and opens the bracket (or
-// marks "no root"); step k >= 0 evaluates D_rec at the midpoint and keeps the
-// half that brackets the root.  The last step writes the result.
-__global__ void __launch_bounds__(kCrecThreads) bisect_kernel(CrecArgs a, BisectState* st, int step, int last,
-                                                            double* out) {
+// ---- R_diff^rec: bisection of D_rec(R) = 1 on (0, L/2] ------------------------------
+// Round by round.  A bisection round evaluates D_rec at the midpoint of the bracket and at both
+// midpoints that may follow, each over its share of the blocks, and then takes two bisection
+// steps: the decisions are those of one step at a time.  Once the bracket is so narrow that every
+// term is smooth over it (q_max times its half width below pi/64 rad), a last round
+// evaluates D_rec at the eight Chebyshev nodes of the bracket and bisects the polynomial
+// through them (interpolation error below (pi/64)^8 / (8! 2^7) < 1e-17 of D's terms) down to
+// the resolution of the 64 steps.  At n = 14000: 9 rounds and the last, 13 us each, where one launch
+// per bisection step with a serial sum of its blocks' partials took 65 x 16 us.  More steps per round
+// do not pay: a D_rec costs the whole GPU's FP64 pipes 1 us (J = 7000), a round's latency is 10.
+constexpr int kNodes = 8;
+struct NodeCos { double c[4 * kNodes]; };    // cos(pi j / 16)
+
+// The first round also evaluates D_rec(L/2), which decides whether there is a root.
+template <bool LAST>
+__global__ void __launch_bounds__(kCrecThreads) bisect_kernel(CrecArgs a, BisectState* st, int first, int points,
+                                                            int iterations, NodeCos nc, double* out) {
     __shared__ double red[kCrecThreads];
+    __shared__ double D[kNodes];
     __shared__ bool is_last;
-    if (st->no_root) {   // uniform across the grid: nothing left to do
-        if (blockIdx.x == 0 && threadIdx.x == 0 && step == last) *out = CUDART_NAN;
+    const double lo = first ? 0.0 : st->lo, hi = first ? a.half_L : st->hi;
+    const bool none = first ? false : st->no_root != 0;
+    if (none) {    // uniform across the grid: nothing left to do
+        if (LAST && blockIdx.x == 0 && threadIdx.x == 0) *out = CUDART_NAN;
         return;
     }
-    const double r = step < 0 ? a.half_L : 0.5 * (st->lo + st->hi);
-    const int stride = gridDim.x * blockDim.x;
-    const double acc = crec_terms(a.s, a.J, a.dq, r, 1 + blockIdx.x * blockDim.x + threadIdx.x, stride);
+    const double mid = 0.5 * (lo + hi), half = 0.5 * (hi - lo);
+    const int per = gridDim.x / points, pt = blockIdx.x / per, b = blockIdx.x % per;
+    double r;
+    if (LAST) r = fma(half, nc.c[2 * pt + 1], mid);
+    else r = pt == 0 ? 0.5 * (lo + mid) : (pt == 1 ? mid : (pt == 2 ? 0.5 * (mid + hi) : a.half_L));
+    const double acc = crec_terms(a.s, a.J, a.dq, r, 1 + b * (int)blockDim.x + (int)threadIdx.x, per * (int)blockDim.x);
     const double t = block_sum_fixed(acc, red);
     if (threadIdx.x == 0) {
         st->partial[blockIdx.x] = t;
@@ -207,33 +289,95 @@ __global__ void __launch_bounds__(kCrecThreads) bisect_kernel(CrecArgs a, Bisect
         is_last = atomicAdd(&st->arrived, 1u) == gridDim.x - 1;
     }
     __syncthreads();
-    if (!is_last || threadIdx.x != 0) return;
+    if (!is_last) return;
     __threadfence();
-    double tot = 0.0;
-    for (int b = 0; b < (int)gridDim.x; ++b) tot += *((volatile double*)&st->partial[b]);
-    const double D = 4.0 * kPi * a.dq * tot;
-    if (step < 0) {
-        st->lo = 0.0;
-        st->hi = a.half_L;
-        st->no_root = D < 1.0;
-    } else if (D < 1.0) {
-        st->lo = r;
-    } else {
-        st->hi = r;
+    // warp w adds the partials of point w (fixed order)
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (w < points) {
+        double v = 0.0;
+        for (int k = lane; k < per; k += 32) v += __ldcg(&st->partial[w * per + k]);
+        for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) D[w] = 4.0 * kPi * a.dq * v;
     }
-    st->arrived = 0u;
-    if (step == last) *out = st->no_root ? CUDART_NAN : 0.5 * (st->lo + st->hi);
+    __syncthreads();
+    if (w != 0) return;
+    if constexpr (!LAST) {
+        if (lane == 0) {
+            double l = lo, h = hi;
+            if (D[1] < 1.0) {
+                l = mid;
+                if (D[2] < 1.0) l = 0.5 * (mid + hi);
+                else h = 0.5 * (mid + hi);
+            } else {
+                h = mid;
+                if (D[0] < 1.0) l = 0.5 * (lo + mid);
+                else h = 0.5 * (lo + mid);
+            }
+            st->lo = l;
+            st->hi = h;
+            if (first) st->no_root = D[3] < 1.0;
+            st->arrived = 0u;
+        }
+    } else {
+        // Chebyshev coefficients of D over the bracket, then 5 bisection steps at a time: lane j holds
+        // the polynomial at the j-th of 32 equal parts of the bracket (u in [-1, 1])
+        double c[kNodes];
+#pragma unroll
+        for (int k = 0; k < kNodes; ++k) {
+            double v = 0.0;
+#pragma unroll
+            for (int i = 0; i < kNodes; ++i) v = fma(D[i], nc.c[(k * (2 * i + 1)) % (4 * kNodes)], v);
+            c[k] = v * (k == 0 ? 1.0 / kNodes : 2.0 / kNodes);
+        }
+        double ul = -1.0, uh = 1.0;
+#pragma unroll 1
+        for (int k = 0; k < iterations; k += 5) {
+            const double u = fma(uh - ul, lane * 0.03125, ul);
+            double b1 = 0.0, b2 = 0.0;     // Clenshaw's recurrence
+#pragma unroll
+            for (int q = kNodes - 1; q >= 1; --q) {
+                const double b0 = fma(2.0 * u, b1, c[q] - b2);
+                b2 = b1;
+                b1 = b0;
+            }
+            const unsigned below = __ballot_sync(0xffffffffu, fma(u, b1, c[0] - b2) < 1.0);
+            int l = 0, h = 32;
+#pragma unroll
+            for (int q = 0; q < 5; ++q) {
+                const int m = (l + h) / 2;
+                if ((below >> m) & 1u) l = m;
+                else h = m;
+            }
+            const double d = uh - ul, base = ul;
+            ul = fma(d, l * 0.03125, base);
+            uh = fma(d, h * 0.03125, base);
+        }
+        if (lane == 0) *out = fma(half, 0.5 * (ul + uh), mid);
+    }
 }
 
-cudaError_t launch_bisect(const CrecArgs& a, BisectState* st, int iterations, double* out, cudaStream_t s) {
-    const int blocks = kBisectBlocks;
+// bisection steps before the last round: the bracket's half width is then L/4 2^-steps with
+// 2^steps >= 16 n (two steps per round)
+static int bisect_steps(int n) {
+    int steps = 0;
+    while ((1ll << steps) < 16ll * n) ++steps;
+    return steps + (steps & 1);
+}
+int bisect_launches(int n) { return bisect_steps(n) / 2 + 1; }
+
+cudaError_t launch_bisect(const CrecArgs& a, BisectState* st, int n, int iterations, double* out, cudaStream_t s) {
+    NodeCos nc;
+    for (int j = 0; j < 4 * kNodes; ++j) nc.c[j] = std::cos(kPi * j / (2.0 * kNodes));
+    const int steps = bisect_steps(n);
     cudaError_t e = cudaMemsetAsync(st, 0, sizeof(BisectState), s);
-    if (e != cudaSuccess) return e;
-    for (int step = -1; step < iterations; ++step) {
-        bisect_kernel<<<blocks, kCrecThreads, 0, s>>>(a, st, step, iterations - 1, out);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    for (int k = 0; k < steps && e == cudaSuccess; k += 2) {
+        const int points = k == 0 ? 4 : 3;
+        bisect_kernel<false><<<kBisectBlocks / points * points, kCrecThreads, 0, s>>>(a, st, k == 0, points, 0, nc, out);
+        e = cudaGetLastError();
     }
-    return cudaSuccess;
+    if (e != cudaSuccess) return e;
+    bisect_kernel<true><<<kBisectBlocks / kNodes * kNodes, kCrecThreads, 0, s>>>(a, st, 0, kNodes, iterations - steps, nc, out);
+    return cudaGetLastError();
 }
 
 }  // namespace scint

@@ -104,3 +104,27 @@ def test_screen_check_paper_realisation_14000():
     _, root = S.structure_function_rec(pg, s)
     assert 500.0 < root.item() < 600.0
     assert root.item() == pytest.approx(540.0, rel=0.08)
+
+
+@pytest.mark.parametrize("n", [18, 254, 256, 258, 514, 770])
+def test_octant_walk_edges(n):
+    """Rows that end inside, at and just after a warp's 128-cell segment, the FP64 square reaching
+    the whole grid (n <= 512) or part of it, the bins of frequency 0 and -n/2, the diagonal."""
+    pg, po = _pair(n, pix=20.0, rd=90.0)
+    s, c = S.spectrum_rec(pg)
+    s_o, c_o = O.spectrum_rec(po)
+    assert torch.equal(c.cpu(), torch.from_numpy(c_o.astype(np.int64)))
+    np.testing.assert_allclose(s.cpu().numpy(), s_o, rtol=S_TOL, atol=0.0)
+
+
+@pytest.mark.parametrize("n,n_bins", [(16, 9), (18, 9), (1000, 300), (4098, 2050)])
+def test_root_rounds(n, n_bins):
+    """Smallest grid, few annuli (long-period terms only), an odd and an even number of bisection
+    steps; the oracle bisects one step at a time."""
+    pix, rd = 10.0, 25.0
+    q = np.arange(n_bins) / (n * pix)
+    s = np.zeros_like(q)
+    s[1:] = O.phase_spectrum(q[1:], rd, 11.0 / 3.0)
+    _, root = S.structure_function_rec(S.params(n=n, pixel_km=pix, r_diff_km=rd), torch.from_numpy(s).cuda())
+    want = O.rdiff_rec(s, n, pix)
+    assert root.item() == pytest.approx(want, rel=1e-12, nan_ok=True)
