@@ -215,7 +215,7 @@ int resolve_ws(void* ws, size_t bytes, size_t need, cudaStream_t s, Carver* c) {
 // A table is computed once, outside stream capture, synchronously (so every stream
 // may read it at once), and kept until scint_release.  A call that is capturing and
 // finds no table, or that must not allocate, computes one in its own workspace.
-enum TwKind { kTw32 = 0, kTwDf = 1 };
+enum TwKind { kTw32 = 0, kTwDf = 1, kTw64 = 2 };
 struct TwCache {
     std::mutex mu;
     std::map<std::tuple<int, int, int>, void*> tab;
@@ -239,12 +239,13 @@ int cached_twiddles(int n, int kind, cudaStream_t s, const void** out) {
     SCINT_CUDA(cudaStreamIsCapturing(s, &cs));
     if (cs != cudaStreamCaptureStatusNone) return SCINT_OK;
     void* p = nullptr;
-    if (cudaMalloc(&p, (size_t)n * (kind == kTwDf ? 16 : 8)) != cudaSuccess) {
+    if (cudaMalloc(&p, (size_t)n * (kind == kTw32 ? 8 : 16)) != cudaSuccess) {
         cudaGetLastError();
         return SCINT_OK;   // no room: the caller uses its workspace
     }
-    cudaError_t e = kind == kTwDf ? launch_twiddles_df(static_cast<dfc*>(p), n, s)
-                                  : launch_twiddles32(static_cast<float2*>(p), n, s);
+    cudaError_t e = kind == kTwDf   ? launch_twiddles_df(static_cast<dfc*>(p), n, s)
+                    : kind == kTw64 ? launch_twiddles64(static_cast<double2*>(p), n, s)
+                                    : launch_twiddles32(static_cast<float2*>(p), n, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
         cudaFree(p);
@@ -944,8 +945,11 @@ int scint_propagate64(const scint_params* p, const double* phi, double* intensit
     Prop64Args a{};
     a.n = p->n;
     a.phi = phi;
-    double2* tw = c.take<double2>((size_t)p->n * 16);
-    a.tw = tw;
+    double2* slot = c.take<double2>((size_t)p->n * 16);    // tables, or twiddles when none are kept
+    const void* kept = nullptr;
+    rc = cached_twiddles(p->n, kTw64, s, &kept);
+    if (rc) return rc;
+    a.tw = kept ? static_cast<const double2*>(kept) : slot;
     a.field = c.take<double2>((size_t)p->n * p->n * 16);
     a.intensity = intensity;
     a.scale = p->lambda_ref_nm / lam;
@@ -956,10 +960,10 @@ int scint_propagate64(const scint_params* p, const double* phi, double* intensit
     a.c_hi = std::ldexp(std::nearbyint(std::ldexp(cf, 31)), -31);
     a.c_lo = cf - a.c_hi;
     const double nn = (double)p->n * p->n;
-    SCINT_LAUNCH(K_TWIDDLES, 16.0 * p->n, 0.0, s, launch_twiddles64(tw, p->n, s));
+    if (!kept) SCINT_LAUNCH(K_TWIDDLES, 16.0 * p->n, 0.0, s, launch_twiddles64(slot, p->n, s));
     // rows: phi read, complex128 field written; columns: field read, FP64 map written
     SCINT_LAUNCH(K_PROP64, 8.0 * nn + 16.0 * nn + 16.0 * nn + 8.0 * nn, 4.0 * p->n * fft_flops(p->n), s,
-                 launch_prop64(a, s));
+                 launch_prop64(a, kept ? slot : nullptr, s));
     return ok();
 }
 

@@ -1,14 +1,14 @@
 // Shared-memory Stockham FFT for one line of N points held by a team of
 // threads (FP32 float2, FP64 double2 or double-float dfc).
 //
-// A team of T = N/E threads (E = 8, 16 or 32) transforms one line; thread t holds the E values at
+// A team of T = N/E threads (E = 4, 8, 16 or 32) transforms one line; thread t holds the E values at
 // positions t + m*T (m = 0..E-1) in registers, both on entry and on exit (the
 // Stockham autosort keeps that distribution, so a forward transform, a pointwise
 // multiply and an inverse transform chain with no extra data movement).
 //
 // Radix plan: the first stage is radix 16 (or N for N < 16), then radix-16
-// stages, then one radix 2/4/8 stage for the remaining bits (with 8 values per
-// thread: radix-8 stages and a radix 2/4 tail).  Between stages the
+// stages, then one radix 2/4/8 stage for the remaining bits (with 8 or 4 values per
+// thread: radix-8 or radix-4 stages and a smaller tail).  Between stages the
 // line goes through the team's shared-memory buffer, padded by one element per
 // 16 so that the stride-16 stores of the first stage are bank-conflict free.
 //
@@ -233,19 +233,19 @@ SCINT_DEV void dft16_fused(float2* x, const float2* w) {
 }
 
 // ---- plan ----------------------------------------------------------------
-// EPT = values held per thread (8, 16 or 32); each stage's butterflies are spread
+// EPT = values held per thread (4, 8, 16 or 32); each stage's butterflies are spread
 // over the T = N/E threads of the line, E/R butterflies per thread.  The stages
-// are radix 16 (EPT 16 or 32) or radix 8 (EPT 8), then one smaller tail stage.
-// With EPT 8 every stage after the first must have N/R >= 16 (the padded
-// addressing of the loads below), i.e. N >= 128.
+// are radix 16 (EPT 16 or 32), radix 8 (EPT 8) or radix 4 (EPT 4), then one smaller tail stage.
+// With EPT 8 and 4 every stage after the first must have N/R >= 16 (the padded
+// addressing of the loads below), i.e. N >= 128 and N >= 64.
 template <int N, int EPT = 16>
 struct FftPlan {
     static_assert(N >= 2 && (N & (N - 1)) == 0, "N must be a power of two");
-    static_assert(EPT == 8 || EPT == 16 || EPT == 32, "8, 16 or 32 values per thread");
+    static_assert(EPT == 4 || EPT == 8 || EPT == 16 || EPT == 32, "4, 8, 16 or 32 values per thread");
     static constexpr int LOG2N = ilog2(N);
     static constexpr int E = N < EPT ? N : EPT;          // values per thread
     static constexpr int T = N / E;                      // threads per line
-    static constexpr int RB = EPT == 8 ? 8 : 16;         // radix of the full stages
+    static constexpr int RB = EPT < 16 ? EPT : 16;        // radix of the full stages
     static constexpr int LB = ilog2(RB);
     static constexpr int R0 = N < RB ? N : RB;           // radix of the first stage
     static constexpr int REST = LOG2N - ilog2(R0);

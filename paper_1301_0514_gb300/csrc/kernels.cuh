@@ -126,8 +126,12 @@ struct Prop64Args {
     double c_hi, c_lo;       // frac(lambda z / (2 L^2)) = c_hi + c_lo, c_hi with 31 bits after the point
     double2* field;          // n*n complex128 scratch
     double* intensity;       // n*n
+    const double2* h;        // H(m)/n, m = 0..n/2, and
+    const double* sf;        // the taper, i = 0..n/2 - 1 (set by launch_prop64)
 };
-cudaError_t launch_prop64(const Prop64Args& a, cudaStream_t s);
+// tables: n * 16 bytes for H and the taper, or NULL (then every element computes its own: a call
+// under capture that has no kept twiddle table keeps its twiddles in that room)
+cudaError_t launch_prop64(const Prop64Args& a, void* tables, cudaStream_t s);
 
 // -------- source smoothing ---------------------------------------------------
 struct SmoothArgs {

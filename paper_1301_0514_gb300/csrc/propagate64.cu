@@ -39,37 +39,60 @@ SCINT_DEV double2 transfer64(const Prop64Args& a, int i) {
     return make_double2(cs / n, sn / n);
 }
 
-template <int N> __host__ __device__ constexpr size_t p64_smem() { return (size_t)FftPlan<N>::BUF * sizeof(double2); }
-// values per thread: 8 up to N = 1024, so that a line has N/8 threads (at 256^2 sixteen values
-// per thread left less than one warp per SM on the FP64 pipe's latency)
-template <int N> __host__ __device__ constexpr int p64_ept() { return N <= 1024 ? 8 : 16; }
+// H(m)/n for m = 0..n/2 and the taper of one half of a line (both are even), one value per thread:
+// in the passes themselves they had been a sincospi per element of every line, and in the margin a
+// sinpi too.  With the tables, twiddles kept between calls and four values per thread at 256^2 both
+// passes took 83 -> 37 us there (FP64 pipe 33 -> 63 % busy), 168 -> 101 us at 512^2, 587 -> 346 us at 1024^2.
+__global__ void prop64_tables_kernel(Prop64Args a, double2* h, double* sf) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, half = a.n / 2;
+    if (i <= half) h[i] = transfer64(a, i);
+    if (i < half) sf[i] = taper64(i, a.n, a.margin_px);
+}
+template <int N, bool TAB>
+SCINT_DEV double2 transfer_of(const Prop64Args& a, int i) {
+    if constexpr (TAB) return __ldg(a.h + (i <= N / 2 ? i : N - i));
+    else return transfer64(a, i);
+}
+template <int N, bool TAB>
+SCINT_DEV double taper_of(const Prop64Args& a, int i) {
+    if constexpr (TAB) return __ldg(a.sf + (i < N / 2 ? i : N - 1 - i));
+    else return taper64(i, N, a.margin_px);
+}
 
-template <int N>
+template <int N> __host__ __device__ constexpr size_t p64_smem() { return (size_t)FftPlan<N>::BUF * sizeof(double2); }
+// values per thread: 4 at N = 128 and 256 (a line has two warps or one; with eight values per thread
+// and 256 lines the SMs had one or two warps each, and the FP64 pipe was 33 % busy), 8 up to
+// N = 1024 (four were 4 % slower at 512: more FP64 operations, and the lines fill the SMs)
+template <int N> __host__ __device__ constexpr int p64_ept() {
+    return N == 128 || N == 256 ? 4 : (N <= 1024 ? 8 : 16);
+}
+
+template <int N, bool TAB>
 __global__ void __launch_bounds__(FftPlan<N, p64_ept<N>()>::T) prop64_rows_kernel(Prop64Args a) {
     constexpr int EPT = p64_ept<N>();
     using Pl = FftPlan<N, EPT>;
     constexpr int T = Pl::T, E = Pl::E;
     extern __shared__ double2 smem64[];
     const int y = blockIdx.x, t = threadIdx.x;
-    const double sfy = taper64(y, N, a.margin_px);
+    const double sfy = taper_of<N, TAB>(a, y);
     double2 v[E];
 #pragma unroll
     for (int m = 0; m < E; ++m) {
         const int x = t + m * T;
         double sn, cs;
         sincos(a.phi[(size_t)y * N + x] * a.scale, &sn, &cs);
-        const double w = sfy * taper64(x, N, a.margin_px);
+        const double w = sfy * taper_of<N, TAB>(a, x);
         v[m] = make_double2(w * cs, w * sn);
     }
     fft_line<double2, N, -1, EPT, 1, 0>(v, smem64, t, a.tw);
 #pragma unroll
-    for (int m = 0; m < E; ++m) v[m] = cmul(v[m], transfer64(a, t + m * T));
+    for (int m = 0; m < E; ++m) v[m] = cmul(v[m], transfer_of<N, TAB>(a, t + m * T));
     fft_line<double2, N, +1, EPT, 1, 0>(v, smem64, t, a.tw);
 #pragma unroll
     for (int m = 0; m < E; ++m) a.field[(size_t)y * N + t + m * T] = v[m];
 }
 
-template <int N>
+template <int N, bool TAB>
 __global__ void __launch_bounds__(FftPlan<N, p64_ept<N>()>::T) prop64_cols_kernel(Prop64Args a) {
     constexpr int EPT = p64_ept<N>();
     using Pl = FftPlan<N, EPT>;
@@ -81,26 +104,41 @@ __global__ void __launch_bounds__(FftPlan<N, p64_ept<N>()>::T) prop64_cols_kerne
     for (int m = 0; m < E; ++m) v[m] = a.field[(size_t)(t + m * T) * N + x];
     fft_line<double2, N, -1, EPT, 1, 0>(v, smem64, t, a.tw);
 #pragma unroll
-    for (int m = 0; m < E; ++m) v[m] = cmul(v[m], transfer64(a, t + m * T));
+    for (int m = 0; m < E; ++m) v[m] = cmul(v[m], transfer_of<N, TAB>(a, t + m * T));
     fft_line<double2, N, +1, EPT, 1, 0>(v, smem64, t, a.tw);
 #pragma unroll
     for (int m = 0; m < E; ++m) a.intensity[(size_t)(t + m * T) * N + x] = v[m].x * v[m].x + v[m].y * v[m].y;
 }
 
-cudaError_t launch_prop64(const Prop64Args& a, cudaStream_t s) {
-    return dispatch_n(a.n, [&](auto nc) -> cudaError_t {
+template <int N, bool TAB>
+cudaError_t launch_passes64(const Prop64Args& a, cudaStream_t s) {
+    cudaError_t e = set_smem(prop64_rows_kernel<N, TAB>, p64_smem<N>());
+    if (e == cudaSuccess) e = set_smem(prop64_cols_kernel<N, TAB>, p64_smem<N>());
+    if (e != cudaSuccess) return e;
+    constexpr int T = FftPlan<N, p64_ept<N>()>::T;
+    prop64_rows_kernel<N, TAB><<<N, T, p64_smem<N>(), s>>>(a);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    prop64_cols_kernel<N, TAB><<<N, T, p64_smem<N>(), s>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_prop64(const Prop64Args& args, void* tables, cudaStream_t s) {
+    return dispatch_n(args.n, [&](auto nc) -> cudaError_t {
         constexpr int N = decltype(nc)::value;
         if constexpr (N > kMax64N) {
             return cudaErrorNotSupported;
         } else {
-            cudaError_t e = set_smem(prop64_rows_kernel<N>, p64_smem<N>());
-            if (e == cudaSuccess) e = set_smem(prop64_cols_kernel<N>, p64_smem<N>());
+            Prop64Args a = args;
+            if (!tables) return launch_passes64<N, false>(a, s);
+            double2* h = static_cast<double2*>(tables);
+            double* sf = reinterpret_cast<double*>(h + N / 2 + 1);
+            static_assert((N / 2 + 1) * sizeof(double2) + N / 2 * sizeof(double) <= N * sizeof(double2), "tables fit");
+            prop64_tables_kernel<<<(N / 2 + 32) / 32, 32, 0, s>>>(a, h, sf);
+            const cudaError_t e = cudaGetLastError();
             if (e != cudaSuccess) return e;
-            constexpr int T = FftPlan<N, p64_ept<N>()>::T;
-            prop64_rows_kernel<N><<<N, T, p64_smem<N>(), s>>>(a);
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            prop64_cols_kernel<N><<<N, T, p64_smem<N>(), s>>>(a);
-            return cudaGetLastError();
+            a.h = h;
+            a.sf = sf;
+            return launch_passes64<N, true>(a, s);
         }
     });
 }

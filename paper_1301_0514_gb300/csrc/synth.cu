@@ -78,13 +78,21 @@ template <int N> __host__ __device__ constexpr int synth_lines() {
     constexpr int spread = (N / 2 + 1) / 304 > 1 ? (N / 2 + 1) / 304 : 1;
     return synth_tile_lines<N>() < spread ? synth_tile_lines<N>() : spread;
 }
-template <int N> __host__ __device__ constexpr int synth_threads() { return synth_lines<N>() * FftPlan<N>::T / synth_cs<N>(); }
-// column pass: complex lines (each two real output columns) per block, at most N/2
-// (two at N = 4096, 139 KB of shared memory: 0.236 -> 0.201 ms per 4096^2 pass against one)
+// Values per thread: 4 from N = 64 to 512, where a pass has one warp or less per SM with sixteen
+// and runs straight through its code once: at 256^2 the row pass had waited on instruction
+// fetches (8.8 of its 10.8 cycles per instruction) and the column pass had used eight SMs
+// (by events: draw and rows 38 -> 28 us, columns 16 -> 8 us; at 512^2 95 -> 64 and 19 -> 9 us).
+template <int N> __host__ __device__ constexpr int synth_ept() { return N >= 64 && N <= kDrawN ? 4 : 16; }
+template <int N> using SynthPlan = FftPlan<N, synth_ept<N>()>;
+template <int N> __host__ __device__ constexpr int synth_threads() { return synth_lines<N>() * SynthPlan<N>::T / synth_cs<N>(); }
+// column pass: complex lines (each two real output columns) per block, the tile but no more than
+// leaves 128 blocks (two at N = 4096, 139 KB of shared memory: 0.236 -> 0.201 ms per 4096^2 pass
+// against one)
 template <int N> __host__ __device__ constexpr int synth_col_lines() {
-    return N == 4096 ? 2 : (synth_tile_lines<N>() < N / 2 ? synth_tile_lines<N>() : N / 2);
+    constexpr int spread = N / 256 > 1 ? N / 256 : 1;
+    return N == 4096 ? 2 : (synth_tile_lines<N>() < spread ? synth_tile_lines<N>() : spread);
 }
-template <int N> __host__ __device__ constexpr int synth_col_threads() { return synth_col_lines<N>() * FftPlan<N>::T / synth_cs<N>(); }
+template <int N> __host__ __device__ constexpr int synth_col_threads() { return synth_col_lines<N>() * SynthPlan<N>::T / synth_cs<N>(); }
 template <int N> constexpr size_t synth_smem() { return (size_t)synth_lines<N>() * FftPlan<N>::BUF * sizeof(dfc) / synth_cs<N>(); }
 template <int N> constexpr size_t synth_col_smem() { return (size_t)synth_col_lines<N>() * FftPlan<N>::BUF * sizeof(dfc) / synth_cs<N>(); }
 
@@ -98,11 +106,6 @@ template <int N> SCINT_DEV size_t synth_idx(int ky, int x) {
     const size_t strip = (size_t)(x >> 1) * synth_strip<N>() + (x & 1);
     if constexpr (N >= kSplitN) return strip + (size_t)(ky & 1) * (synth_strip<N>() / 2) + (size_t)(ky >> 1) * 2;
     else return strip + (size_t)ky * 2;
-}
-
-template <int CS> SCINT_DEV int synth_rank() {
-    if constexpr (CS == 1) return 0;
-    else return (int)cooperative_groups::this_cluster().block_rank();
 }
 
 // F_h(ky, kx) = (F(ky, kx) + conj F(-ky, -kx)) / 2 (the halving is exact)
@@ -147,73 +150,83 @@ SCINT_DEV void synth_row32(const SynthArgs& a, int ky, bool live, int t, float2*
 }
 
 // Up to N = 512 every bin is drawn in FP64 on the narrow FP64 pipe; a row's team there has
-// only N/16 threads, so the Hermitian bins of rows 0..N/2 are drawn first, one per thread of
-// this kernel, into a.drawn (row-major), and the row pass reads them.
-__global__ void __launch_bounds__(256) synth_draw_kernel(SynthArgs a) {
-    const int n = a.n;
-    const int i = blockIdx.x * 256 + threadIdx.x;
-    if (i >= (n / 2 + 1) * n) return;
-    a.drawn[i] = hermitian_bin(a, i % n, i / n);
+// few threads, so the Hermitian bins of rows 0..N/2 are drawn first, by a kernel of their own, into
+// a.drawn (row-major), and the row pass reads them.  A thread draws the bins at (kx, ky) and
+// (-kx, ky) from the four bins (+-kx, +-ky), which share |k| and so one FP64 power law (the FP64
+// pipe is the bound at 256^2, 83 % busy); one warp per block, so that the warps spread evenly.
+constexpr int kDrawThreads = 32;
+__host__ __device__ constexpr int draw_bins(int n) { return (n / 2 + 1) * (n / 2 + 1); }
+__global__ void __launch_bounds__(kDrawThreads) synth_draw_kernel(SynthArgs a) {
+    const int n = a.n, half_n = n / 2;
+    const int i = blockIdx.x * kDrawThreads + threadIdx.x;
+    if (i >= draw_bins(n)) return;
+    const int kx = i % (half_n + 1), ky = i / (half_n + 1);
+    const int nx = (n - kx) & (n - 1), ny = (n - ky) & (n - 1);
+    dfc* row = a.drawn + (size_t)ky * n;
+    const int m2 = kx * kx + ky * ky;
+    if (m2 == 0) {
+        row[0] = make_c<dfc>(0.0, 0.0);
+        return;
+    }
+    const double sig = amplitude_low(a, m2);
+    // F_h = (F(k) + conj F(-k)) / 2 at k = (kx, ky) and at k = (-kx, ky)
+    auto fh = [&](int x, int xm) {
+        const double2 f = shaped_low(bin_words(a, x, ky), sig), g = shaped_low(bin_words(a, xm, ny), sig);
+        return dfc{half(dfl(f.x) + dfl(g.x)), half(dfl(f.y) - dfl(g.y))};
+    };
+    row[kx] = fh(kx, nx);
+    if (nx != kx) row[nx] = fh(nx, kx);
 }
 
 template <int N>
 __global__ void __launch_bounds__(synth_threads<N>())
 synth_rows_kernel(SynthArgs a) {
-    using Pl = FftPlan<N>;
-    constexpr int CS = synth_cs<N>();
-    constexpr int T = Pl::T, E = Pl::E, B = synth_lines<N>(), TL = T / CS;
+    using Pl = SynthPlan<N>;
+    static_assert(synth_cs<N>() == 1, "unsplit rows");
+    constexpr int T = Pl::T, E = Pl::E, B = synth_lines<N>();
     extern __shared__ dfc smem_df[];
-    const int team = threadIdx.x / TL;
-    const int t = synth_rank<CS>() * TL + threadIdx.x % TL;
-    const int ky = (blockIdx.x / CS) * B + team;
+    const int team = threadIdx.x / T, t = threadIdx.x % T;
+    const int ky = blockIdx.x * B + team;
     const bool live = ky <= N / 2;                 // rows above N/2 are the conjugates of rows below
-    if constexpr (CS == 1) {
+    dfc v[E];
+    dfc* buf = smem_df + team * Pl::BUF;
+    if constexpr (N <= kDrawN) {
+#pragma unroll
+        for (int m = 0; m < E; ++m) v[m] = live ? a.drawn[(size_t)ky * N + t + m * T] : make_c<dfc>(0.0, 0.0);
+    } else {
         // every row of the block outside the square (the choice is uniform over the block)
-        if ((blockIdx.x / CS) * B > a.low_k) {
+        if ((int)blockIdx.x * B > a.low_k) {
             synth_row32<N>(a, ky, live, t, reinterpret_cast<float2*>(smem_df) + team * Pl::BUF);
             return;
         }
-    }
-    dfc v[E];
-    dfc* buf = smem_df + team * (Pl::BUF / CS);
-    if constexpr (CS == 1) {
-        if (a.drawn) {
-#pragma unroll
-            for (int m = 0; m < E; ++m) v[m] = live ? a.drawn[(size_t)ky * N + t + m * T] : make_c<dfc>(0.0, 0.0);
-        } else {
-            // the bins are drawn in a loop that is not unrolled (one copy of the Philox and
-            // Box-Muller code: unrolled sixteen times it overflowed the instruction cache) and
-            // staged in the line buffer, where each thread reads back its own entries
+        // the bins are drawn in a loop that is not unrolled (one copy of the Philox and
+        // Box-Muller code: unrolled sixteen times it overflowed the instruction cache) and
+        // staged in the line buffer, where each thread reads back its own entries
 #pragma unroll 1
-            for (int m = 0; m < E; ++m)
-                buf[pad16(t + m * T)] = live ? hermitian_bin(a, t + m * T, ky) : make_c<dfc>(0.0, 0.0);
+        for (int m = 0; m < E; ++m)
+            buf[pad16(t + m * T)] = live ? hermitian_bin(a, t + m * T, ky) : make_c<dfc>(0.0, 0.0);
 #pragma unroll
-            for (int m = 0; m < E; ++m) v[m] = buf[pad16(t + m * T)];
-        }
-    } else {
-#pragma unroll
-        for (int m = 0; m < E; ++m) v[m] = live ? hermitian_bin(a, t + m * T, ky) : make_c<dfc>(0.0, 0.0);
+        for (int m = 0; m < E; ++m) v[m] = buf[pad16(t + m * T)];
+        __syncthreads();
     }
-    line_sync<CS>();
-    fft_line<dfc, N, +1, 16, 1, 0, CS>(v, buf, t, a.tw);
+    fft_line<dfc, N, +1, synth_ept<N>(), 1, 0>(v, buf, t, a.tw);
     if (live) {
 #pragma unroll
         for (int m = 0; m < E; ++m) a.work[synth_idx<N>(ky, t + m * T)] = v[m];
     }
-    if constexpr (CS == 2) line_sync<CS>();
 }
 
 // two real output columns (xa, xa + 1) per complex line
 template <int N>
 __global__ void __launch_bounds__(synth_col_threads<N>())
 synth_cols_kernel(SynthArgs a) {
-    using Pl = FftPlan<N>;
-    constexpr int CS = synth_cs<N>();
-    constexpr int T = Pl::T, E = Pl::E, W = synth_col_lines<N>(), TL = T / CS;
+    using Pl = SynthPlan<N>;
+    static_assert(synth_cs<N>() == 1, "unsplit columns");
+    constexpr int T = Pl::T, E = Pl::E, W = synth_col_lines<N>();
     extern __shared__ dfc smem_df[];
     const int w = threadIdx.x % W;
-    const int t = synth_rank<CS>() * TL + threadIdx.x / W;
-    const int xa = ((blockIdx.x / CS) * W + w) * 2;
+    const int t = threadIdx.x / W;
+    const int xa = ((int)blockIdx.x * W + w) * 2;
     dfc v[E];
 #pragma unroll
     for (int m = 0; m < E; ++m) {
@@ -225,14 +238,12 @@ synth_cols_kernel(SynthArgs a) {
         const dfc za = lo ? ga : conjc(ga), zb = lo ? gb : conjc(gb);
         v[m] = dfc{za.x - zb.y, za.y + zb.x};
     }
-    line_sync<CS>();
-    fft_line<dfc, N, +1, 16, W, 0, CS>(v, smem_df + w, t, a.tw);     // W lines interleaved
+    fft_line<dfc, N, +1, synth_ept<N>(), W, 0>(v, smem_df + w, t, a.tw);     // W lines interleaved
     // columns xa, xa + 1 of a row are adjacent (xa even): one 16-byte store per row
 #pragma unroll
     for (int m = 0; m < E; ++m)
         *reinterpret_cast<double2*>(a.phi + (size_t)(t + m * T) * N + xa) =
             make_double2(scaled_to_double(v[m].x, a.out_scale_df), scaled_to_double(v[m].y, a.out_scale_df));
-    if constexpr (CS == 2) line_sync<CS>();
 }
 
 // ---- N = 16384: lines split by one radix-2 step over a two-block cluster --------------
@@ -352,9 +363,9 @@ cudaError_t launch_synth_pass(const SynthArgs& a, cudaStream_t s) {
                 return launch_pairs_to_rows(a.pairs, a.phi, N, s);
             } else if (ROWS) {
                 if ((e = set_smem(synth_rows_kernel<N>, synth_smem<N>())) != cudaSuccess) return e;
-                if (a.drawn) {
-                    const int bins = (N / 2 + 1) * N;
-                    synth_draw_kernel<<<(bins + 255) / 256, 256, 0, s>>>(a);
+                if constexpr (N <= kDrawN) {
+                    if (!a.drawn) return cudaErrorInvalidValue;
+                    synth_draw_kernel<<<(draw_bins(N) + kDrawThreads - 1) / kDrawThreads, kDrawThreads, 0, s>>>(a);
                     if ((e = cudaGetLastError()) != cudaSuccess) return e;
                 }
                 const int rows = N / 2 + 1;

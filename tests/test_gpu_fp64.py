@@ -88,3 +88,31 @@ def test_fp64_path_rejects_grids_above_4096():
     rc = S.lib().scint_propagate64(ctypes.byref(p), ctypes.c_void_p(phi.data_ptr()), ctypes.c_void_p(out.data_ptr()),
                                    None, 0, None)
     assert rc == 5 and "4096" in S.lib().scint_last_error().decode()
+
+
+@pytest.mark.parametrize("n", [128, 256, 512])
+def test_fp64_passes_inside_a_capture_before_any_call(n):
+    """A capture that finds no kept twiddle table fills the workspace slot with the twiddles and
+    computes H and the taper in the passes: the same bits as with the tables (both forms
+    evaluate the same expressions)."""
+    p = S.params(n=n, pixel_km=20.0, r_diff_km=100.0, seed=7)
+    phi = S.make_screen(p)
+    ws = torch.empty(S.workspace_bytes(p, 1), dtype=torch.uint8, device="cuda")
+    out = torch.zeros((n, n), dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    S.release()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        S.propagate64(p, phi, out=out, workspace=ws)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, S.propagate64(p, phi, workspace=ws))
+
+
+@pytest.mark.parametrize("n", [16, 32, 64, 128, 256, 512])
+def test_small_screens_in_fp64_draws(n):
+    """Screens whose every bin is drawn in FP64 (rows of 1 to 128 threads, one to two column pairs
+    per block): 1e-11 rad, the double-float transform's bound above."""
+    it = W._item(n, 20.0, 60.0, seed=W.SEED_BASE + 64 + n, screen_id=5)
+    err = np.abs(S.make_screen(gpu_params(it)).cpu().numpy() - O.make_screen(oracle_params(it))).max()
+    assert err <= 1e-11
