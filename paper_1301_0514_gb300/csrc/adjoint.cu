@@ -119,10 +119,8 @@ adj_rows_kernel(AdjArgs a) {
     TwiddleRegs<float2, N, 16> tr;
     tr.load(a.tw, t);
 #pragma unroll
-    for (int m = 0; m < E; ++m) {
-        P[m * T] = phase_fixed(a.phi[(size_t)y * N + t + m * T]);
-        acc[m] = 0.0f;
-    }
+    for (int m = 0; m < E; ++m) acc[m] = 0.0f;
+    phases_fixed<E>([&](int m) { return a.phi[(size_t)y * N + t + m * T]; }, [&](int m, long long p) { P[m * T] = p; });
     __syncthreads();
 #pragma unroll 1
     for (int l = 0; l < a.lam.count; ++l) {
@@ -259,8 +257,7 @@ __global__ void __launch_bounds__(asplit_threads<N>(), 1) adj_rows_split_kernel(
 #pragma unroll 1
     for (int y = blockIdx.x / 2; y < N; y += gridDim.x / 2) {
         const double* phi = a.phi + (size_t)y * N + r * H2;
-#pragma unroll
-        for (int m = 0; m < E; ++m) P[r * H2 + t + m * T] = phase_fixed(phi[t + m * T]);
+        phases_fixed<E>([&](int m) { return phi[t + m * T]; }, [&](int m, long long p) { P[r * H2 + t + m * T] = p; });
         line_sync<2>();
         const unsigned pp = cluster_addr(P, (unsigned)(r ^ 1)) + (unsigned)(((r ^ 1) * H2 + t) * sizeof(long long));
 #pragma unroll

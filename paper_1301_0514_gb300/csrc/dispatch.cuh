@@ -83,6 +83,30 @@ inline cudaError_t active_clusters(K kernel, int cs, int threads, size_t smem, i
     return cudaSuccess;
 }
 
+// Blocks of a kernel that are resident on the device at once, queried once per kernel and
+// device; call after set_smem.
+template <typename K>
+inline cudaError_t resident_blocks(K kernel, int threads, size_t smem, int* out) {
+    static std::mutex mu;
+    static std::map<std::pair<int, const void*>, int> seen;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const auto key = std::make_pair(dev, reinterpret_cast<const void*>(kernel));
+    std::lock_guard<std::mutex> lk(mu);
+    auto it = seen.find(key);
+    if (it != seen.end()) {
+        *out = it->second;
+        return cudaSuccess;
+    }
+    int sms = 0, per_sm = 0;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem)) != cudaSuccess) return e;
+    if (per_sm < 1) return cudaErrorInvalidConfiguration;
+    *out = seen[key] = sms * per_sm;
+    return cudaSuccess;
+}
+
 // Launch k with clusters of cs blocks along x (cs == 1: ordinary launch).
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_k(void (*k)(KArgs...), int cs, dim3 grid, dim3 block, size_t smem, cudaStream_t s,

@@ -348,9 +348,10 @@ SCINT_DEV void twiddle_powers(C w1, C w4, C (&w)[R]) {
 // SUB: the threads that share the line buffers and synchronise: the whole block (0), or
 // the SUB-thread part of the block that thread threadIdx.x belongs to, through the named
 // barrier 1 + threadIdx.x / SUB (SUB a multiple of 32 dividing the block; barrier 0 stays
-// the block's own) -- so that two independent teams can share one block.
+// the block's own; a warp of its own needs none) -- so that two independent teams can share one block.
 template <int SUB> SCINT_DEV void team_sync() {
     if constexpr (SUB == 0) __syncthreads();
+    else if constexpr (SUB == 32) __syncwarp();
     else asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)threadIdx.x / SUB), "n"(SUB) : "memory");
 }
 template <int CS, int SUB = 0> SCINT_DEV void line_sync() {
@@ -396,22 +397,14 @@ SCINT_DEV dfc ld_cluster<dfc>(unsigned addr) {
     return dfc{dfl(a, b), dfl(c, d)};
 }
 
-// PP (ping-pong, CS = 1 only): stage s writes buffer s mod 2 (buf, buf1) and stage s + 1
-// reads it, so a stage's reads and the next stage's writes touch different buffers
-// and one barrier per stage suffices (in place: two).  The last stage reads buffer
-// NSTAGE - 2; when that is buf, the next transform's first stage would overwrite it,
-// so that case keeps a barrier after the reads.
-template <typename C, int N, int DIR, int EPT, int LW, int TWM, int CS, int S, int TS = 1, bool PP = false, int SUB = 0>
+template <typename C, int N, int DIR, int EPT, int LW, int TWM, int CS, int S, int TS = 1, int SUB = 0>
 SCINT_DEV void fft_stage(C (&v)[FftPlan<N, EPT>::E], C* buf, int t, const C* __restrict__ tw,
-                         const TwiddleRegs<C, N, EPT>* tr, C* buf1 = nullptr) {
+                         const TwiddleRegs<C, N, EPT>* tr) {
     using Pl = FftPlan<N, EPT>;
     constexpr int E = Pl::E, T = Pl::T;
     constexpr int R = Pl::radix(S), P = Pl::span(S), NB = E / R;
     constexpr bool FIRST = (S == 0), LAST = (S == Pl::NSTAGE - 1);
     constexpr int HALF = N / 2;
-    static_assert(!PP || CS == 1, "ping-pong buffers are for unsplit lines");
-    C* const rbuf = PP && (S % 2 == 0) ? buf1 : buf;    // written by stage S - 1
-    C* const wbuf = PP && (S % 2 == 1) ? buf1 : buf;    // written by stage S
     C u[E];
     if constexpr (FIRST) {
         // butterfly b takes positions t + b T + r N/R = t + (b + r NB) T
@@ -424,9 +417,9 @@ SCINT_DEV void fft_stage(C (&v)[FftPlan<N, EPT>::E], C* buf, int t, const C* __r
         for (int b = 0; b < NB; ++b) {
             // N/R is a multiple of 16 here, so pad16(i + r N/R) = pad16(i) + r (N/R)(17/16).
 #pragma unroll
-            for (int r = 0; r < R; ++r) u[b * R + r] = rbuf[pad16(t + b * T) * LW + r * ((N / R) + (N / R) / 16) * LW];
+            for (int r = 0; r < R; ++r) u[b * R + r] = buf[pad16(t + b * T) * LW + r * ((N / R) + (N / R) / 16) * LW];
         }
-        if constexpr (!PP || (LAST && (Pl::NSTAGE - 2) % 2 == 0)) team_sync<SUB>();
+        team_sync<SUB>();
     } else {
         // Split line: i < N/R <= N/2, so element i + r N/R is in the upper half
         // (rank 1's buffer, local index i + (r - R/2) N/R) iff r >= R/2.
@@ -498,13 +491,13 @@ SCINT_DEV void fft_stage(C (&v)[FftPlan<N, EPT>::E], C* buf, int t, const C* __r
             if constexpr (CS == 2) j &= HALF - 1;
             // P >= 16: pad16(j + r P) = pad16(j) + r P (17/16); P == 1: j = i R and r < R <= 16
             // (j a multiple of R, so j + r stays in one group of 16); otherwise pad16 itself
-            C* dst = wbuf + pad16(j) * LW;
+            C* dst = buf + pad16(j) * LW;
 #pragma unroll
             for (int r = 0; r < R; ++r)
                 dst[(P >= 16 ? r * (P + P / 16) : (P == 1 ? r : pad16(j + r * P) - pad16(j))) * LW] = u[b * R + r];
         }
         line_sync<CS, SUB>();
-        fft_stage<C, N, DIR, EPT, LW, TWM, CS, S + 1, TS, PP, SUB>(v, buf, t, tw, tr, buf1);
+        fft_stage<C, N, DIR, EPT, LW, TWM, CS, S + 1, TS, SUB>(v, buf, t, tw, tr);
     }
 }
 
@@ -516,26 +509,13 @@ template <typename C, int N, int DIR, int EPT = 16, int LW = 1, int TWM = 0, int
 SCINT_DEV void fft_line(C (&v)[FftPlan<N, EPT>::E], C* buf, int t, const C* __restrict__ tw) {
     static_assert(TWM != 2, "register twiddles: use fft_line_tr");
     static_assert(CS == 1 || (CS == 2 && FftPlan<N, EPT>::NSTAGE > 1 && N >= 512), "split lines need N >= 512");
-    fft_stage<C, N, DIR, EPT, LW, TWM, CS, 0, TS, false, SUB>(v, buf, t, tw, nullptr);
+    fft_stage<C, N, DIR, EPT, LW, TWM, CS, 0, TS, SUB>(v, buf, t, tw, nullptr);
 }
 
 template <typename C, int N, int DIR, int EPT = 16, int LW = 1, int CS = 1, int SUB = 0>
 SCINT_DEV void fft_line_tr(C (&v)[FftPlan<N, EPT>::E], C* buf, int t, const TwiddleRegs<C, N, EPT>& tr) {
     static_assert(CS == 1 || (CS == 2 && FftPlan<N, EPT>::NSTAGE > 1 && N >= 512), "split lines need N >= 512");
-    fft_stage<C, N, DIR, EPT, LW, 2, CS, 0, 1, false, SUB>(v, buf, t, nullptr, &tr);
-}
-
-// Ping-pong forms (unsplit lines): buf1 is a second buffer laid out like buf.  Between
-// two ping-pong transforms of the same buffers no barrier is needed; any other write
-// to either buffer after one needs a __syncthreads first.
-template <typename C, int N, int DIR, int EPT = 16, int LW = 1, int TWM = 0, int SUB = 0>
-SCINT_DEV void fft_line_pp(C (&v)[FftPlan<N, EPT>::E], C* buf, C* buf1, int t, const C* __restrict__ tw) {
-    static_assert(TWM != 2, "register twiddles: use fft_line_tr_pp");
-    fft_stage<C, N, DIR, EPT, LW, TWM, 1, 0, 1, true, SUB>(v, buf, t, tw, nullptr, buf1);
-}
-template <typename C, int N, int DIR, int EPT = 16, int LW = 1, int SUB = 0>
-SCINT_DEV void fft_line_tr_pp(C (&v)[FftPlan<N, EPT>::E], C* buf, C* buf1, int t, const TwiddleRegs<C, N, EPT>& tr) {
-    fft_stage<C, N, DIR, EPT, LW, 2, 1, 0, 1, true, SUB>(v, buf, t, nullptr, &tr, buf1);
+    fft_stage<C, N, DIR, EPT, LW, 2, CS, 0, 1, SUB>(v, buf, t, nullptr, &tr);
 }
 
 // ---- lines split by one radix-2 step over a two-block cluster ------------------

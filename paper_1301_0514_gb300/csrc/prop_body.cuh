@@ -25,13 +25,10 @@ SCINT_DEV void prop_rows_body(const PropArgs& a, int bid, int tid, float2* smem3
     long long* P = reinterpret_cast<long long*>(smem32 + B * BUFL) + team * N + t;
     float2* tws = smem32 + B * BUFL + B * N;    // shared twiddle table (after P, 8 B per entry)
     const float2* twp = TWM == 1 ? tws : a.tw;
-    constexpr bool PP = ppp_row<N>();            // second line buffers after the table
-    float2* buf1 = smem32 + B * BUFL + B * N + (TWM == 1 ? Pl::TWS : 0) + team * BUFL;
     TwiddleRegs<float2, N, 16> tr;
     if constexpr (TWM == 2) tr.load(a.tw, t);
     else if constexpr (TWM == 1) fill_twiddle_table<float2, N>(tws, a.tw, tid, prow_threads<N>());
-#pragma unroll
-    for (int m = 0; m < E; ++m) P[m * T] = phase_fixed(a.phi[(size_t)y * N + t + m * T]);
+    phases_fixed<E>([&](int m) { return a.phi[(size_t)y * N + t + m * T]; }, [&](int m, long long p) { P[m * T] = p; });
     team_sync<SUB>();
 
 #pragma unroll 1
@@ -54,17 +51,13 @@ SCINT_DEV void prop_rows_body(const PropArgs& a, int bid, int tid, float2* smem3
 #pragma unroll
             for (int m = 0; m < E; ++m) v[m] = unit_phasor(P[m * T], S) * (sfy * __ldg(sf + t + m * T));
         }
-        if constexpr (PP && TWM == 2) fft_line_tr_pp<float2, N, -1, 16, 1, SUB>(v, buf, buf1, t, tr);
-        else if constexpr (PP) fft_line_pp<float2, N, -1, 16, 1, TWM, SUB>(v, buf, buf1, t, twp);
-        else if constexpr (TWM == 2) fft_line_tr<float2, N, -1, 16, 1, 1, SUB>(v, buf, t, tr);
+        if constexpr (TWM == 2) fft_line_tr<float2, N, -1, 16, 1, 1, SUB>(v, buf, t, tr);
         else fft_line<float2, N, -1, 16, 1, TWM, 1, 1, SUB>(v, buf, t, twp);
         if constexpr (!CONJ) {
             const unsigned long long hc = a.lam.h_fx[l];
 #pragma unroll
-            for (int m = 0; m < E; ++m) v[m] = cmul(v[m], transfer_phasor(hc, t + m * T, N));
-            if constexpr (PP && TWM == 2) fft_line_tr_pp<float2, N, +1, 16, 1, SUB>(v, buf, buf1, t, tr);
-            else if constexpr (PP) fft_line_pp<float2, N, +1, 16, 1, TWM, SUB>(v, buf, buf1, t, twp);
-            else if constexpr (TWM == 2) fft_line_tr<float2, N, +1, 16, 1, 1, SUB>(v, buf, t, tr);
+            for (int m = 0; m < E; ++m) v[m] = cmul(v[m], transfer_signed(hc, signed_index<N, E>(t, m)));
+            if constexpr (TWM == 2) fft_line_tr<float2, N, +1, 16, 1, 1, SUB>(v, buf, t, tr);
             else fft_line<float2, N, +1, 16, 1, TWM, 1, 1, SUB>(v, buf, t, twp);
         }
         float2* dst = a.work + (size_t)l * N * N;
@@ -80,19 +73,20 @@ SCINT_DEV void prop_rows_body(const PropArgs& a, int bid, int tid, float2* smem3
 template <int N, bool CONJ, int SUB = 0>
 SCINT_DEV void prop_cols_body(const PropArgs& a, int bid, int tid, float2* smem32) {
     using Pl = FftPlan<N, kColEPT>;
-    constexpr int TWM = pcol_twm<N>();
+    constexpr int TWM = pcol_twm<N, CONJ>();
     constexpr int T = Pl::T, E = Pl::E, W = pcol_lines<N>(), WL = pstrip<N>(), BUFL = Pl::BUF;
-    const int w = tid % W, t = tid / W;
+    // a team of T threads per column (col_teams), or W lines interleaved: element e of line w at pad16(e) * W + w
+    constexpr bool TEAMS = !CONJ && col_teams<N>();
+    constexpr int LW = TEAMS ? 1 : W, SUBC = TEAMS ? T : SUB;
+    const int w = TEAMS ? tid / T : tid % W, t = TEAMS ? tid % T : tid / W;
     const int x0 = bid * W;    // first column of the block: strip x0 / WL, offset x0 % WL
     const int x = x0 + w;
-    float2* buf = smem32 + w;     // W lines interleaved: element e of line w at pad16(e) * W + w
+    float2* buf = smem32 + (TEAMS ? w * BUFL : w);
     // passband accumulator of this thread's pixels, in registers (a shared-memory
     // copy would add a read-modify-write per wavelength to the busiest queue)
     float acc[E];
     float2* tws = smem32 + W * BUFL;   // shared twiddle table (after the line buffers)
     const float2* twp = TWM == 1 ? tws : a.tw;
-    constexpr bool PP = ppp_col<N>();   // second line buffers after the table
-    float2* buf1 = smem32 + W * BUFL + (TWM == 1 ? Pl::TWS : 0) + w;
     TwiddleRegs<float2, N, kColEPT> tr;
     if constexpr (TWM == 2) tr.load(a.tw, t);
     else if constexpr (TWM == 1) fill_twiddle_table<float2, N>(tws, a.tw, tid, pcol_threads<N>());
@@ -105,10 +99,8 @@ SCINT_DEV void prop_cols_body(const PropArgs& a, int bid, int tid, float2* smem3
         float2 v[E];
 #pragma unroll
         for (int m = 0; m < E; ++m) v[m] = __ldcg(src + (size_t)(t + m * T) * WL + w);
-        if constexpr (PP && TWM == 2) fft_line_tr_pp<float2, N, -1, kColEPT, W, SUB>(v, buf, buf1, t, tr);
-        else if constexpr (PP) fft_line_pp<float2, N, -1, kColEPT, W, TWM, SUB>(v, buf, buf1, t, twp);
-        else if constexpr (TWM == 2) fft_line_tr<float2, N, -1, kColEPT, W, 1, SUB>(v, buf, t, tr);
-        else fft_line<float2, N, -1, kColEPT, W, TWM, 1, 1, SUB>(v, buf, t, twp);
+        if constexpr (TWM == 2) fft_line_tr<float2, N, -1, kColEPT, LW, 1, SUBC>(v, buf, t, tr);
+        else fft_line<float2, N, -1, kColEPT, LW, TWM, 1, 1, SUBC>(v, buf, t, twp);
         if constexpr (CONJ) {
             // h = (Delta^2 / lambda z)^2 |FT G|^2 on the pattern grid of this wavelength (Eq. intens)
             const float nrm = a.conj.norm[l];
@@ -126,11 +118,9 @@ SCINT_DEV void prop_cols_body(const PropArgs& a, int bid, int tid, float2* smem3
         } else {
             const unsigned long long hc = a.lam.h_fx[l];
 #pragma unroll
-            for (int m = 0; m < E; ++m) v[m] = cmul(v[m], transfer_phasor(hc, t + m * T, N));
-            if constexpr (PP && TWM == 2) fft_line_tr_pp<float2, N, +1, kColEPT, W, SUB>(v, buf, buf1, t, tr);
-            else if constexpr (PP) fft_line_pp<float2, N, +1, kColEPT, W, TWM, SUB>(v, buf, buf1, t, twp);
-            else if constexpr (TWM == 2) fft_line_tr<float2, N, +1, kColEPT, W, 1, SUB>(v, buf, t, tr);
-            else fft_line<float2, N, +1, kColEPT, W, TWM, 1, 1, SUB>(v, buf, t, twp);
+            for (int m = 0; m < E; ++m) v[m] = cmul(v[m], transfer_signed(hc, signed_index<N, E>(t, m)));
+            if constexpr (TWM == 2) fft_line_tr<float2, N, +1, kColEPT, LW, 1, SUBC>(v, buf, t, tr);
+            else fft_line<float2, N, +1, kColEPT, LW, TWM, 1, 1, SUBC>(v, buf, t, twp);
         }
         // the 1/N of H_y, squared, rides on the weight (powers of two: the sums are unchanged bit for bit)
         const float wl = a.lam.weight[l] * (1.0f / ((float)N * (float)N));

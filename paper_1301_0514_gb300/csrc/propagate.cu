@@ -23,6 +23,7 @@
 #include "dispatch.cuh"
 #include "prop_body.cuh"
 #include "propagate.cuh"
+#include "stream.cuh"
 
 namespace scint {
 
@@ -72,6 +73,256 @@ prop_cols_kernel(PropArgs a) {
     prop_cols_body<N, CONJ>(a, blockIdx.x, threadIdx.x, smem32);
 }
 
+// ---- streamed passes (rows 512 to 8192, columns of the transfer function 512 to 4096) ------
+// The same arithmetic with the inputs of the next wavelength or line on their way while this one is
+// transformed: without it every warp of a block waited for its loads at the same time, at the
+// head of each wavelength.  The copies need neither registers nor load instructions (a copy by
+// cp.async had cost more than it hid, on the load/store pipe that the line exchanges keep
+// 60 % busy).  The passes are bound by issue slots (105-120 instructions per pixel and wavelength)
+// and by the load/store pipe of the exchanges; per-launch times before and after, ms:
+//                  32 wavelengths                          one wavelength
+//          rows           columns               rows             columns
+//   512    0.102 -> 0.082   0.085 -> 0.076      0.0118 -> 0.0106   0.0098 -> 0.0099
+//   1024   0.176 -> 0.152   0.160 -> 0.138      0.0171 -> 0.0147   0.0131 -> 0.0148
+//   2048   0.625 -> 0.569   0.573 -> 0.496      0.0458 -> 0.0314   0.0414 -> 0.0374
+//   4096   2.501 -> 2.352   2.562 -> 2.416      0.1657 -> 0.108    0.1637 -> 0.133
+//   8192 (8 wavelengths, rows)  3.70 -> 3.35    0.795  -> 0.525
+// The one-FFT columns keep plain loads: with half the transforms per value the copies of 16-byte
+// rows became their bound (4096^2, 8 wavelengths: 0.493 ms, streamed 0.531).
+//   Row pass: the block's phases by one bulk copy into the array that keeps their fixed-point
+//   form (converted in place, each thread its own entries), the taper of each wavelength by
+//   another; both are issued once the forward transform's barriers show that the block has read
+//   what they overwrite.
+//   Column pass: the block's columns of one wavelength as boxes of 16-byte rows, dense, into a stage
+//   of their own; a team of threads per column (col_teams), twiddles from register bases, whose
+//   products cost less than the table's loads once the columns do not share barriers (2048^2: 0.559 ms
+//   with the table).
+// With few wavelengths the blocks walk lines (walk_blocks).
+template <int N> __host__ __device__ constexpr bool row_stream() { return N >= 512 && N <= 8192; }
+template <int N> constexpr size_t prow_stream_smem() {
+    return (size_t)prow_lines<N>() * (FftPlan<N>::BUF * sizeof(float2) + N * sizeof(long long)) + N * sizeof(float) + 24;
+}
+
+template <int N, bool CONJ>
+__global__ void __launch_bounds__(prow_threads<N>(), (prow_threads<N>() <= 256 ? 2 : 1))
+prop_rows_stream_kernel(PropArgs a, int bulk) {
+    using Pl = FftPlan<N>;
+    constexpr int T = Pl::T, E = Pl::E, B = prow_lines<N>(), W = pstrip<N>(), BUFL = Pl::BUF;
+    static_assert(prow_twm<N>() == 2, "register twiddle bases");
+    extern __shared__ float2 smem32[];
+    const int team = threadIdx.x / T, t = threadIdx.x % T;
+    float2* buf = smem32 + team * BUFL;
+    long long* Pall = reinterpret_cast<long long*>(smem32 + B * BUFL);
+    long long* P = Pall + team * N + t;
+    float* sfs = reinterpret_cast<float*>(Pall + B * N);
+    unsigned long long* bar = reinterpret_cast<unsigned long long*>(sfs + N);    // phases, taper
+    unsigned* reads = reinterpret_cast<unsigned*>(bar + 2);    // rows that have read the taper
+    // below 2048 a row is a team with a barrier of its own (512^2: 3 % faster; at 2048 2 % slower)
+    constexpr int SUB = N < 2048 ? T : 0;
+    const int count = a.lam.count, tiles = N / B;
+    auto load_phi = [&](int tile) {
+        tile_expect(bar, B * N * sizeof(double));
+        bulk_load(Pall, a.phi + (size_t)tile * (B * N), B * N * sizeof(double), bar);
+    };
+    auto load_sf = [&](int l) {
+        tile_expect(bar + 1, N * sizeof(float));
+        bulk_load(sfs, a.sf + (size_t)l * N, N * sizeof(float), bar + 1);
+    };
+    if (threadIdx.x == 0) {
+        tile_init(bar);
+        tile_init(bar + 1);
+        *reads = 0u;
+        tile_init_fence();
+        if (bulk) load_phi(blockIdx.x);
+        load_sf(0);
+    }
+    TwiddleRegs<float2, N, 16> tr;
+    tr.load(a.tw, t);
+    __syncthreads();
+    unsigned phase = 0;    // bits: parity of the phases' copy, of the taper's
+    bool ok = true;
+#pragma unroll 1
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const int y = tile * B + team;
+        if (bulk) {
+            ok = ok && wait_tile(bar, phase & 1);
+            phase ^= 1;
+            phases_fixed<E>([&](int m) { return __longlong_as_double(P[m * T]); }, [&](int m, long long p) { P[m * T] = p; });
+            tile_reuse_fence();
+        } else {
+            phases_fixed<E>([&](int m) { return a.phi[(size_t)y * N + t + m * T]; }, [&](int m, long long p) { P[m * T] = p; });
+        }
+#pragma unroll 1
+        for (int l = 0; l < count; ++l) {
+            if (count > 1 || tile == (int)blockIdx.x) {
+                ok = ok && wait_tile(bar + 1, phase >> 1);
+                phase ^= 2;
+            }
+            const unsigned long long S = a.lam.scale_fx[l];
+            // 1/N of the inverse transform on the taper of the row (prop_rows_body); NaN if a copy is missing
+            const float sfy = ok ? (CONJ ? sfs[y] : sfs[y] * (1.0f / N)) : __int_as_float(0x7FFFFFFF);
+            float2 v[E];
+            if constexpr (CONJ) {
+                const unsigned long long C = a.conj.chirp_fx[l];
+                const unsigned long long cy = chirp_turns(C, y, N);
+#pragma unroll
+                for (int m = 0; m < E; ++m)
+                    v[m] = unit_phasor(P[m * T], S, cy + chirp_turns(C, t + m * T, N)) * (sfy * sfs[t + m * T]);
+            } else {
+#pragma unroll
+                for (int m = 0; m < E; ++m) v[m] = unit_phasor(P[m * T], S) * (sfy * sfs[t + m * T]);
+            }
+            fft_line_tr<float2, N, -1, 16, 1, 1, SUB>(v, buf, t, tr);
+            // the row is past its first exchange, hence done with this wavelength's taper, and with the
+            // phases at the last wavelength; the last row to get here sends for the next ones
+            if (SUB == 0 ? threadIdx.x == 0 : t == 0) {
+                __threadfence_block();
+                if (SUB == 0 || atomicAdd(reads, 1u) % B == B - 1) {
+                    const bool last = l + 1 == count, more = tile + (int)gridDim.x < tiles;
+                    if (count > 1 && (!last || more)) load_sf(last ? 0 : l + 1);
+                    if (bulk && last && more) load_phi(tile + gridDim.x);
+                }
+            }
+            if constexpr (!CONJ) {
+                const unsigned long long hc = a.lam.h_fx[l];
+#pragma unroll
+                for (int m = 0; m < E; ++m) v[m] = cmul(v[m], transfer_signed(hc, signed_index<N, E>(t, m)));
+                fft_line_tr<float2, N, +1, 16, 1, 1, SUB>(v, buf, t, tr);
+            }
+            float2* dst = a.work + (size_t)l * N * N;
+#pragma unroll
+            for (int m = 0; m < E; ++m) dst[strip_index<W>(y, t + m * T, N)] = v[m];
+        }
+    }
+    if (!ok) {    // nothing in flight may outlive the block: wait again, with the same limit
+        for (int k = 0; k < 4; ++k) wait_tile(bar + (k >> 1), k & 1);
+    }
+}
+
+// W consecutive values of a row of the map, o (+)= r; wide: o is aligned to min(4 W, 16) bytes
+template <int W>
+SCINT_DEV void store_row(float* o, float (&r)[W], int wide, int accumulate) {
+    if (accumulate) {
+#pragma unroll
+        for (int k = 0; k < W; ++k) r[k] += o[k];
+    }
+    if (!wide) {
+#pragma unroll
+        for (int k = 0; k < W; ++k) o[k] = r[k];
+    } else if constexpr (W == 2) {
+        *reinterpret_cast<float2*>(o) = make_float2(r[0], r[1]);
+    } else {
+        static_assert(W % 4 == 0, "two columns or quadruples");
+#pragma unroll
+        for (int k = 0; k < W; k += 4) *reinterpret_cast<float4*>(o + k) = make_float4(r[k], r[k + 1], r[k + 2], r[k + 3]);
+    }
+}
+
+template <int N> constexpr size_t pcol_stream_smem() {
+    return col_stage_bytes<N>() + (size_t)pcol_lines<N>() * FftPlan<N>::BUF * sizeof(float2) + 16;
+}
+
+template <int N>
+__global__ void __launch_bounds__(pcol_threads<N>(), (pcol_threads<N>() <= 256 ? 2 : 1))
+prop_cols_stream_kernel(PropArgs a, const __grid_constant__ CUtensorMap tm, int wide) {
+    using Pl = FftPlan<N, kColEPT>;
+    constexpr int T = Pl::T, E = Pl::E, W = pcol_lines<N>();
+    extern __shared__ float2 smem32[];
+    const int w = threadIdx.x / T, t = threadIdx.x % T;    // a team per column
+    float2* stage = smem32;
+    float2* bufs = stage + N * W;
+    float2* buf = bufs + w * Pl::BUF;
+    unsigned long long* bar = reinterpret_cast<unsigned long long*>(bufs + W * Pl::BUF);
+    unsigned* reads = reinterpret_cast<unsigned*>(bar + 1);    // teams that have read the stage
+    const int count = a.lam.count;
+    if (threadIdx.x == 0) {
+        tile_init(bar);
+        *reads = 0u;
+        tile_init_fence();
+        issue_columns<N>(stage, &tm, 0, blockIdx.x * W, bar);
+    }
+    TwiddleRegs<float2, N, 16> tr;
+    tr.load(a.tw, t);
+    __syncthreads();
+    unsigned parity = 0;
+    bool ok = true;
+#pragma unroll 1
+    for (int x0 = blockIdx.x * W; x0 < N; x0 += gridDim.x * W) {
+        float acc[E];
+#pragma unroll
+        for (int m = 0; m < E; ++m) acc[m] = 0.0f;
+#pragma unroll 1
+        for (int l = 0; l < count; ++l) {
+            ok = ok && wait_tile(bar, parity);
+            parity ^= 1;
+            float2 v[E];
+            const float2* col = stage + (w / kBoxCols) * N * kBoxCols + w % kBoxCols;
+#pragma unroll
+            for (int m = 0; m < E; ++m) v[m] = col[(t + m * T) * kBoxCols];
+            fft_line_tr<float2, N, -1, kColEPT, 1, 1, T>(v, buf, t, tr);
+            // the team is past its first exchange, hence done with the stage; the last team to get here
+            // sends for the next columns
+            if (t == 0) {
+                __threadfence_block();
+                if (atomicAdd(reads, 1u) % W == W - 1) {
+                    const bool last = l + 1 == count;
+                    const int nx = last ? x0 + (int)gridDim.x * W : x0;
+                    if (nx < N) issue_columns<N>(stage, &tm, last ? 0 : l + 1, nx, bar);
+                }
+            }
+            const unsigned long long hc = a.lam.h_fx[l];
+#pragma unroll
+            for (int m = 0; m < E; ++m) v[m] = cmul(v[m], transfer_signed(hc, signed_index<N, E>(t, m)));
+            fft_line_tr<float2, N, +1, kColEPT, 1, 1, T>(v, buf, t, tr);
+            // 1/N of H_y, squared, on the weight (prop_cols_body); NaN if a copy is missing
+            const float wl = ok ? a.lam.weight[l] * (1.0f / ((float)N * (float)N)) : __int_as_float(0x7FFFFFFF);
+#pragma unroll
+            for (int m = 0; m < E; ++m) acc[m] = fmaf(wl, fmaf(v[m].x, v[m].x, v[m].y * v[m].y), acc[m]);
+        }
+        // the columns side by side through the line buffers, one store of W values per row (a value of
+        // one column per thread and row had cost 0.05 ms at 4096^2: one 4-byte sector write each)
+        float* own = reinterpret_cast<float*>(buf);
+#pragma unroll
+        for (int m = 0; m < E; ++m) own[t + m * T] = acc[m];
+        __syncthreads();
+#pragma unroll 2
+        for (int y = threadIdx.x; y < N; y += pcol_threads<N>()) {
+            float r[W];
+#pragma unroll
+            for (int k = 0; k < W; ++k) r[k] = reinterpret_cast<const float*>(bufs + k * Pl::BUF)[y];
+            store_row<W>(a.intensity + (size_t)y * N + x0, r, wide, a.accumulate);
+        }
+        __syncthreads();
+    }
+    if (!ok) {
+        wait_tile(bar, 0);
+        wait_tile(bar, 1);
+    }
+}
+
+bool field_map(CUtensorMap* tm, const float2* work, int n, int count, int strip) {
+    using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                                const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+    static const Encode encode = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<Encode>(f);
+    }();
+    if (!encode || reinterpret_cast<uintptr_t>(work) % 16) return false;
+    const cuuint64_t dims[2] = {(cuuint64_t)(2 * strip), (cuuint64_t)count * (n / strip) * n};
+    const cuuint64_t strides[1] = {(cuuint64_t)strip * sizeof(float2)};
+    const cuuint32_t box[2] = {2 * kBoxCols, kBoxRows}, step[2] = {1, 1};
+    return encode(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float2*>(work), dims, strides, box, step,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // ---- lines split over a two-block cluster (N = 16384) -------------------------------
 // One radix-2 step on each side of the line transforms divides them between the two
 // blocks of a cluster (n < N/2, W = exp(-2 pi i / N)):
@@ -114,8 +365,7 @@ __global__ void __launch_bounds__(psplit_threads<N>(), 1) prop_rows_split_kernel
 #pragma unroll 1
     for (int y = blockIdx.x / 2; y < N; y += gridDim.x / 2) {
         const double* phi = a.phi + (size_t)y * N + r * H2;
-#pragma unroll
-        for (int m = 0; m < E; ++m) P[r * H2 + t + m * T] = phase_fixed(phi[t + m * T]);
+        phases_fixed<E>([&](int m) { return phi[t + m * T]; }, [&](int m, long long p) { P[r * H2 + t + m * T] = p; });
         line_sync<2>();
         const unsigned pp = cluster_addr(P, (unsigned)(r ^ 1)) + (unsigned)(((r ^ 1) * H2 + t) * sizeof(long long));
 #pragma unroll
@@ -227,8 +477,7 @@ __global__ void __launch_bounds__(psplit_threads<N>(), 1) conj_rows_split_kernel
         if (!first) cluster_wait();     // the partner has copied this block's previous phases
         first = false;
         const double* phi = a.phi + (size_t)y * N + r * H2;
-#pragma unroll
-        for (int m = 0; m < E; ++m) P[r * H2 + t + m * T] = phase_fixed(phi[t + m * T]);
+        phases_fixed<E>([&](int m) { return phi[t + m * T]; }, [&](int m, long long p) { P[r * H2 + t + m * T] = p; });
         line_sync<2>();
         const unsigned pp = cluster_addr(P, (unsigned)(r ^ 1)) + (unsigned)(((r ^ 1) * H2 + t) * sizeof(long long));
 #pragma unroll
@@ -337,9 +586,21 @@ cudaError_t launch_rows(const PropArgs& a, cudaStream_t s) {
             if (e == cudaSuccess) e = active_clusters(k, 2, psplit_threads<N>(), prow_split_smem<N>(), &nc);
             if (e != cudaSuccess) return e;
             return launch_k(k, 2, dim3(2 * std::min(nc, N)), dim3(psplit_threads<N>()), prow_split_smem<N>(), s, a);
-        } else if constexpr (prow_smem<N>() > kMaxSmem || pcol_smem<N>() > kMaxSmem) {
+        } else if constexpr (prow_smem<N>() > kMaxSmem || pcol_smem<N, true>() > kMaxSmem) {
             return cudaErrorNotSupported;
         } else {
+            if constexpr (row_stream<N>()) {
+                static_assert(prow_stream_smem<N>() <= kMaxSmem, "streamed row pass does not fit");
+                auto k = prop_rows_stream_kernel<N, CONJ>;
+                cudaError_t e = set_smem(k, prow_stream_smem<N>());
+                int blocks = 0;
+                if (e == cudaSuccess)
+                    e = walk_blocks(k, prow_threads<N>(), prow_stream_smem<N>(), N / prow_lines<N>(), a.lam.count, &blocks);
+                if (e != cudaSuccess) return e;
+                // a bulk copy starts on a 16-byte boundary: phases elsewhere are read by plain loads
+                k<<<blocks, prow_threads<N>(), prow_stream_smem<N>(), s>>>(a, reinterpret_cast<uintptr_t>(a.phi) % 16 == 0);
+                return cudaGetLastError();
+            }
             cudaError_t e = set_smem(prop_rows_kernel<N, CONJ>, prow_smem<N>());
             if (e != cudaSuccess) return e;
             prop_rows_kernel<N, CONJ><<<N / prow_lines<N>(), prow_threads<N>(), prow_smem<N>(), s>>>(a);
@@ -365,12 +626,29 @@ cudaError_t launch_cols(const PropArgs& a, cudaStream_t s) {
             if (e != cudaSuccess || !to_scratch) return e;
             transpose_add_kernel<<<dim3(N / 32, N / 32), 256, 0, s>>>(a.scratch, a.intensity, N, a.accumulate);
             return cudaGetLastError();
-        } else if constexpr (prow_smem<N>() > kMaxSmem || pcol_smem<N>() > kMaxSmem) {
+        } else if constexpr (prow_smem<N>() > kMaxSmem || pcol_smem<N, true>() > kMaxSmem) {
             return cudaErrorNotSupported;
         } else {
-            cudaError_t e = set_smem(prop_cols_kernel<N, CONJ>, pcol_smem<N>());
+            if constexpr (!CONJ && col_stream<N>()) {
+                static_assert(pcol_stream_smem<N>() <= kMaxSmem, "streamed column pass does not fit");
+                CUtensorMap tm;
+                if (field_map(&tm, a.work, N, a.lam.count, pstrip<N>())) {
+                    auto k = prop_cols_stream_kernel<N>;
+                    cudaError_t e = set_smem(k, pcol_stream_smem<N>());
+                    int blocks = 0;
+                    if (e == cudaSuccess)
+                        e = walk_blocks(k, pcol_threads<N>(), pcol_stream_smem<N>(), N / pcol_lines<N>(), a.lam.count, &blocks);
+                    if (e != cudaSuccess) return e;
+                    constexpr int align = pcol_lines<N>() == 2 ? 8 : 16;
+                    k<<<blocks, pcol_threads<N>(), pcol_stream_smem<N>(), s>>>(
+                        a, tm, reinterpret_cast<uintptr_t>(a.intensity) % align == 0);
+                    return cudaGetLastError();
+                }
+            }
+            constexpr size_t smem = pcol_smem<N, CONJ>();
+            cudaError_t e = set_smem(prop_cols_kernel<N, CONJ>, smem);
             if (e != cudaSuccess) return e;
-            prop_cols_kernel<N, CONJ><<<N / pcol_lines<N>(), pcol_threads<N>(), pcol_smem<N>(), s>>>(a);
+            prop_cols_kernel<N, CONJ><<<N / pcol_lines<N>(), pcol_threads<N>(), smem, s>>>(a);
             return cudaGetLastError();
         }
     });

@@ -18,16 +18,6 @@
 
 namespace scint {
 
-// Ping-pong FFT buffers in the propagation passes (fft.cuh: one barrier per stage
-// instead of two), off by default.  Measured on GB300 with 32 wavelengths, each pass
-// alone is faster with them (rows 1.4 % at 4096 to 10 % at 1024, columns 1-4.5 %
-// below 4096; 1.5 % slower at 4096, which would keep one buffer), but the batched
-// step on four lanes is 7.6 % slower (123.1 -> 132.5 ms): at 102 KB per row block two
-// blocks fill an SM's shared memory and the other lanes' kernels no longer share it.
-#ifndef SCINT_PROP_PINGPONG
-#define SCINT_PROP_PINGPONG 0
-#endif
-
 constexpr int kRowTw = SCINT_ROW_TWIDDLES;
 constexpr int kColTw = SCINT_COL_TWIDDLES;
 constexpr int kColEPT = 16;   // values per thread in the column passes
@@ -38,10 +28,7 @@ constexpr size_t kMaxSmem = 227 * 1024;
 // propagate.cu, adj_*_split_kernel in adjoint.cu): each block transforms one parity
 // as a whole N/2-point line.  The kernels below are the unsplit passes.
 template <int N> __host__ __device__ constexpr int pcs() { return N >= kSplitN ? 2 : 1; }
-template <int N> __host__ __device__ constexpr bool ppp_row() { return SCINT_PROP_PINGPONG; }
-template <int N> __host__ __device__ constexpr bool ppp_col() { return SCINT_PROP_PINGPONG && N < 4096; }
 template <int N> __host__ __device__ constexpr int prow_twm() { return kRowTw; }
-template <int N> __host__ __device__ constexpr int pcol_twm();   // below: depends on the shared-memory budget
 
 // rows per row-pass block, columns per column-pass block (all lines of a block
 // are transformed together); threads are per block
@@ -62,19 +49,24 @@ template <int N> __host__ __device__ constexpr int pstrip() { return pcol_lines<
 
 template <int N> constexpr size_t ptws_bytes(int twm) { return twm == 1 ? (size_t)FftPlan<N>::TWS * sizeof(float2) : 0; }
 template <int N> constexpr size_t prow_smem() {
-    return (size_t)prow_lines<N>() * ((ppp_row<N>() ? 2 : 1) * FftPlan<N>::BUF * sizeof(float2) + N * sizeof(long long)) +
+    return (size_t)prow_lines<N>() * (FftPlan<N>::BUF * sizeof(float2) + N * sizeof(long long)) +
            ptws_bytes<N>(prow_twm<N>());
 }
-// column pass: line buffers and (when it fits) the twiddle table
+// Transfer-function column blocks of these sizes give each column a team of threads with a barrier and a line buffer
+// of its own, so that one column's line exchanges run beside another's butterflies; in smaller
+// blocks (and at 8192, one column per block) the columns are interleaved across the lanes and share
+// the block's barriers.
+template <int N> __host__ __device__ constexpr bool col_teams() { return N >= 512 && N <= 4096; }
+// column pass: line buffers and, without teams, the twiddle table when it fits
 template <int N> __host__ __device__ constexpr size_t pcol_base_bytes() {
     return (size_t)pcol_lines<N>() * FftPlan<N>::BUF * sizeof(float2);
 }
-template <int N> __host__ __device__ constexpr int pcol_twm() {
-    return (kColTw == 1 && pcol_base_bytes<N>() * (ppp_col<N>() ? 2 : 1) + (size_t)FftPlan<N>::TWS * sizeof(float2) > kMaxSmem
+template <int N, bool CONJ> __host__ __device__ constexpr int pcol_twm() {
+    return !CONJ && col_teams<N>() ? 2 : (kColTw == 1 && pcol_base_bytes<N>() + (size_t)FftPlan<N>::TWS * sizeof(float2) > kMaxSmem
                 ? 2 : kColTw);
 }
-template <int N> constexpr size_t pcol_smem() {
-    return pcol_base_bytes<N>() * (ppp_col<N>() ? 2 : 1) + ptws_bytes<N>(pcol_twm<N>());
+template <int N, bool CONJ = false> constexpr size_t pcol_smem() {
+    return pcol_base_bytes<N>() + ptws_bytes<N>(pcol_twm<N, CONJ>());
 }
 
 // signed FFT frequency index of bin i
@@ -87,6 +79,29 @@ template <int WL> SCINT_DEV size_t strip_index(int y, int x, int n) {
 
 // phi (radians) -> 64-bit fixed-point turns, P = round(phi 2^32 / 2 pi)
 SCINT_DEV long long phase_fixed(double phi) { return __double2ll_rn(phi * (4294967296.0 / (2.0 * kPi))); }
+// The same for E values of a thread, P(m) = phase_fixed(phi(m)).  Below 2^21 rad the product is
+// rounded to an integer by the one FP64 addition of 1.5 2^52 it is fused with, and the integer is read
+// from the sum's bits: one instruction on the narrow FP64 pipe instead of a product and a conversion
+// (16 cycles of an SM per warp each; the row pass at one wavelength 0.142 -> 0.110 ms at 4096^2).
+// Rounded once instead of twice, the two differ next to a tie only, by 2^-32 turns.
+template <int E, typename Load, typename Store>
+SCINT_DEV void phases_fixed(Load&& load, Store&& store) {
+    double f[E];
+    unsigned top = 0;
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+        f[m] = load(m);
+        top = max(top, (unsigned)__double2hiint(f[m]) & 0x7FFFFFFFu);
+    }
+    if (top < 0x41400000u) {    // |phi| < 2^21 for every value
+        const double k = 4294967296.0 / (2.0 * kPi), magic = 0x1.8p52;
+#pragma unroll
+        for (int m = 0; m < E; ++m) store(m, __double_as_longlong(fma(f[m], k, magic)) - 0x4338000000000000ll);
+    } else {                    // large phases, infinities, NaN
+#pragma unroll
+        for (int m = 0; m < E; ++m) store(m, phase_fixed(f[m]));
+    }
+}
 
 // exp(i (phi s + add 2^-64 turns)) from P and S = round(s 2^32): the low 64
 // bits of P S are the fractional turns of phi s times 2^64 (exact reduction
@@ -105,6 +120,19 @@ SCINT_DEV float2 unit_phasor(long long P, unsigned long long S, unsigned long lo
 SCINT_DEV float2 transfer_phasor(unsigned long long C, int i, int n) {
     const long long m = sfreq(i, n);
     return unit_phasor(0, 0ull, C * (unsigned long long)(m * m));
+}
+// The same for the signed index m itself, |m| < 2^15: the upper 32 bits of C m^2 mod 2^64 are all
+// that the angle takes, so 32-bit products do (the same bits).
+SCINT_DEV float2 transfer_signed(unsigned long long C, int m) {
+    const unsigned mm = (unsigned)(m * m);
+    const unsigned hi = __umulhi((unsigned)C, mm) + (unsigned)(C >> 32) * mm;
+    float sn, cs;
+    __sincosf((float)(int)hi * (float)(2.0 * kPi * 0x1.0p-32), &sn, &cs);
+    return make_float2(cs, sn);
+}
+// signed frequency index of element t + m T of a line of N = E T values, t < T
+template <int N, int E> SCINT_DEV int signed_index(int t, int m) {
+    return t + m * (N / E) - (2 * m >= E ? N : 0);
 }
 // H_x(k)/n (the inverse transform's normalisation)
 SCINT_DEV float2 transfer_at(unsigned long long C, int i, int n) { return transfer_phasor(C, i, n) * (1.0f / n); }

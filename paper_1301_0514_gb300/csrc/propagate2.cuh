@@ -67,8 +67,7 @@ prop_rows2_kernel(PropArgs a) {
     TwiddleRegs<float2, N, EPT> tr;
     if constexpr (TWM == 2) tr.load(a.tw, t);
     else fill_twiddle_table<float2, N, EPT>(tws, a.tw, threadIdx.x, blockDim.x);
-#pragma unroll
-    for (int m = 0; m < E; ++m) P[m * T] = phase_fixed(a.phi[(size_t)y * N + t + m * T]);
+    phases_fixed<E>([&](int m) { return a.phi[(size_t)y * N + t + m * T]; }, [&](int m, long long p) { P[m * T] = p; });
     __syncthreads();
     const int nl = a.lam.count;
     cp2* const work = reinterpret_cast<cp2*>(a.work);

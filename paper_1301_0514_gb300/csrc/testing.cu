@@ -75,7 +75,7 @@ cudaError_t launch_fft_lines64(int n, int dir, double2* data, int n_lines, const
 
 __global__ void phase_fixed_kernel(const double* phi, long long* P, long long n) {
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        P[i] = phase_fixed(phi[i]);
+        phases_fixed<1>([&](int) { return phi[i]; }, [&](int, long long p) { P[i] = p; });
 }
 cudaError_t launch_phase_fixed(const double* phi, long long* P, long long n, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;

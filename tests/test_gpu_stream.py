@@ -1,0 +1,57 @@
+"""The streamed propagation passes (inputs of the next line or wavelength copied ahead): every
+number of rows per block and columns per block, few wavelengths (a block walks lines) and many
+(one line per block), and buffers off the 16-byte boundary that the copies need, which take plain
+loads and narrow stores through the same arithmetic."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+import paper_1301_0514_gb300 as S
+
+pytestmark = pytest.mark.gpu
+
+I_TOL = 2e-4      # the FP32 passes' bound against the oracle (tests/test_gpu_parity.py)
+
+
+def _off(n, dtype):
+    """An n x n tensor whose first element is one element past an aligned address."""
+    return torch.empty(n * n + 1, dtype=dtype, device="cuda")[1:].view(n, n)
+
+
+def _band(count):
+    return np.linspace(500.0, 640.0, count) if count > 1 else np.array([550.0])
+
+
+@pytest.mark.parametrize("n,count", [(512, 1), (512, 8), (1024, 1), (1024, 7), (1024, 8), (2048, 3)])
+def test_streamed_passes_match_oracle(n, count):
+    kw = dict(n=n, pixel_km=10.0, r_diff_km=60.0, lambda_nm=550.0, lambda_ref_nm=550.0, seed=20130514 + 640 + n)
+    p, po = S.params(**kw), O.ScreenParams(**kw)
+    phi = O.make_screen(po)
+    want = O.sum_passband(phi, po, _band(count))
+    got = S.sum_passband(p, torch.from_numpy(phi).cuda(), _band(count)).cpu().numpy()
+    assert np.abs(got - want).max() <= I_TOL
+
+
+@pytest.mark.parametrize("n", [512, 1024, 2048, 4096, 8192])
+@pytest.mark.parametrize("count", [1, 2, 9])
+def test_streamed_passes_off_alignment(n, count):
+    """The same bits from buffers off the 16-byte boundary, and the wavelengths one at a time (each
+    pixel's sum then rounds once more per wavelength)."""
+    if n == 8192 and count > 2:
+        pytest.skip("the same code as at 4096 with one row per block")
+    p = S.params(n=n, pixel_km=10.0, r_diff_km=60.0, lambda_nm=550.0, seed=5)
+    phi = S.make_screen(p)
+    lam = _band(count)
+    want = S.sum_passband(p, phi, lam)
+    phi2, out2 = _off(n, torch.float64), _off(n, torch.float32)
+    assert phi2.data_ptr() % 16 and out2.data_ptr() % 8
+    phi2.copy_(phi)
+    S.sum_passband(p, phi2, lam, out=out2)
+    assert torch.equal(out2, want)
+    out2.fill_(0.0)
+    for l in lam:
+        S.sum_passband(p, phi2, [l], [1.0 / count], out=out2, accumulate=True)
+    assert (out2 - want).abs().max().item() <= count * 2.0 ** -23 * want.max().item()
+    pc = S.params(n=n, pixel_km=100.0 * (512.0 / n) ** 0.5, r_diff_km=600.0, lambda_nm=550.0, seed=5)
+    assert torch.equal(S.sum_passband_conjugate(pc, phi2, lam, out=out2), S.sum_passband_conjugate(pc, phi, lam))
