@@ -52,6 +52,22 @@ __host__ __device__ constexpr double cos16(int j) {
     }
 }
 
+// cos(2 pi j / 32); sin(2 pi j / 32) = cos(2 pi (j - 8) / 32)
+__host__ __device__ constexpr double cos32(int j) {
+    j = ((j % 32) + 32) % 32;
+    if (j % 2 == 0) return cos16(j / 2);
+    switch (j) {
+        case 1: case 31: return 0.98078528040323044913;
+        case 3: case 29: return 0.83146961230254523708;
+        case 5: case 27: return 0.55557023301960222474;
+        case 7: case 25: return 0.19509032201612826785;
+        case 9: case 23: return -0.19509032201612826785;
+        case 11: case 21: return -0.55557023301960222474;
+        case 13: case 19: return -0.83146961230254523708;
+        default: return -0.98078528040323044913;
+    }
+}
+
 // a * exp(DIR * 2 pi i J16 / 16), J16 a compile-time multiple of 1/16 turn
 template <int J16, int DIR, typename C>
 SCINT_DEV C rot16(C a) {
@@ -516,6 +532,51 @@ template <typename C, int N, int DIR, int EPT = 16, int LW = 1, int CS = 1, int 
 SCINT_DEV void fft_line_tr(C (&v)[FftPlan<N, EPT>::E], C* buf, int t, const TwiddleRegs<C, N, EPT>& tr) {
     static_assert(CS == 1 || (CS == 2 && FftPlan<N, EPT>::NSTAGE > 1 && N >= 512), "split lines need N >= 512");
     fft_stage<C, N, DIR, EPT, LW, 2, CS, 0, 1, SUB>(v, buf, t, nullptr, &tr);
+}
+
+// ---- long FP32 lines: two half lines in one team -----------------------------------
+// An N-point line (N = 8192) as one radix-2 step in registers and two N/2-point lines one after
+// the other through one N/2-point buffer: thread t of T = N/32 holds the values at t + m T (a[m])
+// and at N/2 + t + m T (b[m]), m < 16.  Against sixteen values per thread and stages
+// 16 16 16 2: two exchanges per transform instead of three, half the buffer, and a team of half
+// the threads, so that two lines share an SM and one's exchanges run beside the other's butterflies.
+//   forward (decimation in frequency): a, b -> X at the frequencies 2k (a[m]) and 2k + 1 (b[m]), k = t + m T
+//   inverse (decimation in time):      the reverse, unnormalised
+template <int N> struct LongPlan {
+    using Half = FftPlan<N / 2>;
+    static constexpr int T = Half::T, H = Half::E, BUF = Half::BUF;
+    static_assert(H == 16, "sixteen values of each half per thread");
+};
+// W_N^(t + m T) = W_N^t W_32^m from the thread's W_N^t
+template <int M> SCINT_DEV float2 long_twiddle(float2 w0) {
+    if constexpr (M == 0) return w0;
+    else return cmul(w0, make_float2((float)cos32(M), (float)-cos32(M - 8)));
+}
+template <int N, int M = 0>
+SCINT_DEV void long_split(float2* a, float2* b, float2 w0) {
+    if constexpr (M < LongPlan<N>::H) {
+        const float2 d = a[M] - b[M];
+        a[M] = a[M] + b[M];
+        b[M] = cmul(d, long_twiddle<M>(w0));
+        long_split<N, M + 1>(a, b, w0);
+    }
+}
+template <int N, int M = 0>
+SCINT_DEV void long_join(float2* a, float2* b, float2 w0) {
+    if constexpr (M < LongPlan<N>::H) {
+        const float2 y = cfma(b[M], conjc(long_twiddle<M>(w0)), a[M]);    // A + conj(W) B, then A - conj(W) B = 2 A - that
+        b[M] = twice_minus(a[M], y);
+        a[M] = y;
+        long_join<N, M + 1>(a, b, w0);
+    }
+}
+template <int N, int DIR, int SUB = 0>
+SCINT_DEV void fft_long(float2 (&a)[16], float2 (&b)[16], float2* buf, int t, const TwiddleRegs<float2, N / 2, 16>& tr,
+                        float2 w0) {
+    if constexpr (DIR < 0) long_split<N>(a, b, w0);
+    fft_line_tr<float2, N / 2, DIR, 16, 1, 1, SUB>(a, buf, t, tr);
+    fft_line_tr<float2, N / 2, DIR, 16, 1, 1, SUB>(b, buf, t, tr);
+    if constexpr (DIR > 0) long_join<N>(a, b, w0);
 }
 
 // ---- lines split by one radix-2 step over a two-block cluster ------------------

@@ -98,7 +98,7 @@ prop_cols_kernel(PropArgs a) {
 //   products cost less than the table's loads once the columns do not share barriers (2048^2: 0.559 ms
 //   with the table).
 // With few wavelengths the blocks walk lines (walk_blocks).
-template <int N> __host__ __device__ constexpr bool row_stream() { return N >= 512 && N <= 8192; }
+template <int N> __host__ __device__ constexpr bool row_stream() { return N >= 512 && N <= 4096; }
 template <int N> constexpr size_t prow_stream_smem() {
     return (size_t)prow_lines<N>() * (FftPlan<N>::BUF * sizeof(float2) + N * sizeof(long long)) + N * sizeof(float) + 24;
 }
@@ -189,9 +189,10 @@ prop_rows_stream_kernel(PropArgs a, int bulk) {
                 for (int m = 0; m < E; ++m) v[m] = cmul(v[m], transfer_signed(hc, signed_index<N, E>(t, m)));
                 fft_line_tr<float2, N, +1, 16, 1, 1, SUB>(v, buf, t, tr);
             }
-            float2* dst = a.work + (size_t)l * N * N;
+            static_assert(T % W == 0, "whole strips between a thread's values");
+            float2* dst = a.work + (size_t)l * N * N + strip_index<W>(y, t, N);
 #pragma unroll
-            for (int m = 0; m < E; ++m) dst[strip_index<W>(y, t + m * T, N)] = v[m];
+            for (int m = 0; m < E; ++m) dst[(size_t)(m * T) * N] = v[m];
         }
     }
     if (!ok) {    // nothing in flight may outlive the block: wait again, with the same limit
@@ -298,6 +299,171 @@ prop_cols_stream_kernel(PropArgs a, const __grid_constant__ CUtensorMap tm, int 
         wait_tile(bar, 0);
         wait_tile(bar, 1);
     }
+}
+
+// ---- lines of 8192 points: two half lines per team (fft_long) ----------------------------
+// Row pass: 256 threads per row, two rows per SM; the phases by bulk copy as above, the taper
+// from its table (no room beside two rows' phases).
+// Column pass: 256 threads and one column per block, two blocks per SM, so that one column's
+// loads run behind the other's transforms; the passband sums in shared memory (the values take
+// the registers).  Clusters of four blocks share a strip and put their four columns' sums
+// side by side through distributed shared memory: one 16-byte store per row and cluster instead
+// of a 4-byte one per row and column.
+template <int N> __host__ __device__ constexpr bool long_lines() { return N == 8192; }
+template <int N> constexpr size_t prow_long_smem() { return (size_t)LongPlan<N>::BUF * sizeof(float2) + N * sizeof(long long) + 16; }
+
+template <int N, bool CONJ>
+__global__ void __launch_bounds__(LongPlan<N>::T, 2) prop_rows_long_kernel(PropArgs a, int bulk) {
+    using Pl = LongPlan<N>;
+    constexpr int T = Pl::T, H = Pl::H, W = pstrip<N>();
+    extern __shared__ float2 smem32[];
+    const int t = threadIdx.x;
+    float2* buf = smem32;
+    long long* Pall = reinterpret_cast<long long*>(smem32 + Pl::BUF);
+    long long* P = Pall + t;
+    unsigned long long* bar = reinterpret_cast<unsigned long long*>(Pall + N);
+    auto load_phi = [&](int y) {
+        tile_expect(bar, N * sizeof(double));
+        bulk_load(Pall, a.phi + (size_t)y * N, N * sizeof(double), bar);
+    };
+    if (t == 0) {
+        tile_init(bar);
+        tile_init_fence();
+        if (bulk) load_phi(blockIdx.x);
+    }
+    TwiddleRegs<float2, N / 2, 16> tr;
+    tr.load(a.tw, t, 2);
+    const float2 w0 = __ldg(a.tw + t);
+    __syncthreads();
+    unsigned parity = 0;
+    bool ok = true;
+#pragma unroll 1
+    for (int y = blockIdx.x; y < N; y += gridDim.x) {
+        if (bulk) {
+            ok = ok && wait_tile(bar, parity);
+            parity ^= 1;
+            phases_fixed<2 * H>([&](int m) { return __longlong_as_double(P[m * T]); }, [&](int m, long long p) { P[m * T] = p; });
+            tile_reuse_fence();
+        } else {
+            phases_fixed<2 * H>([&](int m) { return a.phi[(size_t)y * N + t + m * T]; }, [&](int m, long long p) { P[m * T] = p; });
+        }
+#pragma unroll 1
+        for (int l = 0; l < a.lam.count; ++l) {
+            const unsigned long long S = a.lam.scale_fx[l];
+            const float* sf = a.sf + (size_t)l * N;
+            // 1/N of the inverse transform on the taper of the row; NaN if a copy is missing
+            const float sfy = ok ? (CONJ ? sf[y] : sf[y] * (1.0f / N)) : __int_as_float(0x7FFFFFFF);
+            float2 va[H], vb[H];
+            if constexpr (CONJ) {
+                const unsigned long long C = a.conj.chirp_fx[l];
+                const unsigned long long cy = chirp_turns(C, y, N);
+#pragma unroll
+                for (int m = 0; m < H; ++m) {
+                    const int x = t + m * T, z = x + N / 2;
+                    va[m] = unit_phasor(P[m * T], S, cy + chirp_turns(C, x, N)) * (sfy * __ldg(sf + x));
+                    vb[m] = unit_phasor(P[m * T + N / 2], S, cy + chirp_turns(C, z, N)) * (sfy * __ldg(sf + z));
+                }
+            } else {
+#pragma unroll
+                for (int m = 0; m < H; ++m) {
+                    const int x = t + m * T, z = x + N / 2;
+                    va[m] = unit_phasor(P[m * T], S) * (sfy * __ldg(sf + x));
+                    vb[m] = unit_phasor(P[m * T + N / 2], S) * (sfy * __ldg(sf + z));
+                }
+            }
+            fft_long<N, -1>(va, vb, buf, t, tr, w0);
+            // every thread is past an exchange, hence done with the phases at the last wavelength
+            if (bulk && t == 0 && l + 1 == a.lam.count && y + (int)gridDim.x < N) load_phi(y + gridDim.x);
+            float2* dst = a.work + (size_t)l * N * N + strip_index<W>(y, CONJ ? 2 * t : t, N);
+            if constexpr (CONJ) {
+                // the frequencies 2k and 2k + 1 are neighbours in the strip
+#pragma unroll
+                for (int m = 0; m < H; ++m)
+                    *reinterpret_cast<float4*>(dst + (size_t)(2 * m * T) * N) =
+                        make_float4(va[m].x, va[m].y, vb[m].x, vb[m].y);
+            } else {
+                const unsigned long long hc = a.lam.h_fx[l];
+#pragma unroll
+                for (int m = 0; m < H; ++m) {
+                    const int f = 2 * signed_index<N / 2, H>(t, m);
+                    va[m] = cmul(va[m], transfer_signed(hc, f));
+                    vb[m] = cmul(vb[m], transfer_signed(hc, f + 1));
+                }
+                fft_long<N, +1>(va, vb, buf, t, tr, w0);
+#pragma unroll
+                for (int m = 0; m < H; ++m) {
+                    dst[(size_t)(m * T) * N] = va[m];
+                    dst[(size_t)(m * T + N / 2) * N] = vb[m];
+                }
+            }
+        }
+    }
+    if (!ok) {
+        wait_tile(bar, 0);
+        wait_tile(bar, 1);
+    }
+}
+
+constexpr int kLongCluster = 4;
+template <int N> constexpr size_t pcol_long_smem() { return (size_t)LongPlan<N>::BUF * sizeof(float2) + N * sizeof(float); }
+
+template <int N>
+__global__ void __launch_bounds__(LongPlan<N>::T, 2) prop_cols_long_kernel(PropArgs a, int wide) {
+    using Pl = LongPlan<N>;
+    constexpr int T = Pl::T, H = Pl::H, WL = pstrip<N>(), C = kLongCluster;
+    static_assert(WL == C, "a cluster per strip");
+    extern __shared__ float2 smem32[];
+    auto cl = cooperative_groups::this_cluster();
+    const int t = threadIdx.x, r = (int)cl.block_rank();
+    float2* buf = smem32;
+    float* acc = reinterpret_cast<float*>(smem32 + Pl::BUF);    // own entries until the end
+    TwiddleRegs<float2, N / 2, 16> tr;
+    tr.load(a.tw, t, 2);
+    const float2 w0 = __ldg(a.tw + t);
+    const int x0 = (int)blockIdx.x / C * C;
+    const float2* col = a.work + (size_t)x0 * N + r;
+#pragma unroll 1
+    for (int l = 0; l < a.lam.count; ++l) {
+        const float2* src = col + (size_t)l * N * N;
+        float2 va[H], vb[H];
+#pragma unroll
+        for (int m = 0; m < H; ++m) {
+            va[m] = __ldcg(src + (size_t)(t + m * T) * WL);
+            vb[m] = __ldcg(src + (size_t)(t + m * T + N / 2) * WL);
+        }
+        fft_long<N, -1>(va, vb, buf, t, tr, w0);
+        const unsigned long long hc = a.lam.h_fx[l];
+#pragma unroll
+        for (int m = 0; m < H; ++m) {
+            const int f = 2 * signed_index<N / 2, H>(t, m);
+            va[m] = cmul(va[m], transfer_signed(hc, f));
+            vb[m] = cmul(vb[m], transfer_signed(hc, f + 1));
+        }
+        fft_long<N, +1>(va, vb, buf, t, tr, w0);
+        // 1/N of H_y, squared, on the weight (prop_cols_body)
+        const float wl = a.lam.weight[l] * (1.0f / ((float)N * (float)N));
+#pragma unroll
+        for (int m = 0; m < H; ++m) {
+            float* p = acc + t + m * T;
+            float* q = p + N / 2;
+            const float pa = l ? *p : 0.0f, qa = l ? *q : 0.0f;
+            *p = fmaf(wl, fmaf(va[m].x, va[m].x, va[m].y * va[m].y), pa);
+            *q = fmaf(wl, fmaf(vb[m].x, vb[m].x, vb[m].y * vb[m].y), qa);
+        }
+    }
+    cl.sync();
+    // rank r stores its quarter of the rows, the cluster's four columns side by side
+    const float* part[C];
+#pragma unroll
+    for (int k = 0; k < C; ++k) part[k] = cl.map_shared_rank(acc, k);
+#pragma unroll 4
+    for (int y = r * (N / C) + t; y < (r + 1) * (N / C); y += T) {
+        float s[C];
+#pragma unroll
+        for (int k = 0; k < C; ++k) s[k] = part[k][y];
+        store_row<C>(a.intensity + (size_t)y * N + x0, s, wide, a.accumulate);
+    }
+    cl.sync();    // no block leaves before its sums are read
 }
 
 bool field_map(CUtensorMap* tm, const float2* work, int n, int count, int strip) {
@@ -589,6 +755,16 @@ cudaError_t launch_rows(const PropArgs& a, cudaStream_t s) {
         } else if constexpr (prow_smem<N>() > kMaxSmem || pcol_smem<N, true>() > kMaxSmem) {
             return cudaErrorNotSupported;
         } else {
+            if constexpr (long_lines<N>()) {
+                static_assert(2 * (prow_long_smem<N>() + 1024) <= 228 * 1024, "two rows per SM");
+                auto k = prop_rows_long_kernel<N, CONJ>;
+                cudaError_t e = set_smem(k, prow_long_smem<N>());
+                int blocks = 0;
+                if (e == cudaSuccess) e = walk_blocks(k, LongPlan<N>::T, prow_long_smem<N>(), N, a.lam.count, &blocks);
+                if (e != cudaSuccess) return e;
+                k<<<blocks, LongPlan<N>::T, prow_long_smem<N>(), s>>>(a, reinterpret_cast<uintptr_t>(a.phi) % 16 == 0);
+                return cudaGetLastError();
+            }
             if constexpr (row_stream<N>()) {
                 static_assert(prow_stream_smem<N>() <= kMaxSmem, "streamed row pass does not fit");
                 auto k = prop_rows_stream_kernel<N, CONJ>;
@@ -629,6 +805,14 @@ cudaError_t launch_cols(const PropArgs& a, cudaStream_t s) {
         } else if constexpr (prow_smem<N>() > kMaxSmem || pcol_smem<N, true>() > kMaxSmem) {
             return cudaErrorNotSupported;
         } else {
+            if constexpr (!CONJ && long_lines<N>()) {
+                static_assert(2 * (pcol_long_smem<N>() + 1024) <= 228 * 1024, "two columns per SM");
+                auto k = prop_cols_long_kernel<N>;
+                const cudaError_t e = set_smem(k, pcol_long_smem<N>());
+                if (e != cudaSuccess) return e;
+                return launch_k(k, kLongCluster, dim3(N), dim3(LongPlan<N>::T), pcol_long_smem<N>(), s, a,
+                                (int)(reinterpret_cast<uintptr_t>(a.intensity) % 16 == 0));
+            }
             if constexpr (!CONJ && col_stream<N>()) {
                 static_assert(pcol_stream_smem<N>() <= kMaxSmem, "streamed column pass does not fit");
                 CUtensorMap tm;

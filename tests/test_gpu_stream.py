@@ -55,3 +55,13 @@ def test_streamed_passes_off_alignment(n, count):
     assert (out2 - want).abs().max().item() <= count * 2.0 ** -23 * want.max().item()
     pc = S.params(n=n, pixel_km=100.0 * (512.0 / n) ** 0.5, r_diff_km=600.0, lambda_nm=550.0, seed=5)
     assert torch.equal(S.sum_passband_conjugate(pc, phi2, lam, out=out2), S.sum_passband_conjugate(pc, phi, lam))
+
+
+@pytest.mark.parametrize("count", [1, 2, 9])
+def test_long_lines_match_the_one_wavelength_form(count):
+    """8192-point lines (two half lines per team): a passband and its wavelengths one by one, and the
+    FP64 field theory: a uniform untapered screen stays 1 everywhere."""
+    n = 8192
+    p = S.params(n=n, pixel_km=10.0, r_diff_km=60.0, lambda_nm=550.0, margin_km=0.0, seed=5)
+    one = S.sum_passband(p, torch.zeros((n, n), dtype=torch.float64, device="cuda"), _band(count))
+    assert (one - 1.0).abs().max().item() <= 2e-5
