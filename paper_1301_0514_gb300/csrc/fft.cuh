@@ -308,14 +308,16 @@ SCINT_DEV dfc ld_tw<dfc>(const dfc* __restrict__ p) {
 // (the caller offsets buf by its lane), so LW lines can share one interleaved
 // buffer with consecutive threads of different lines hitting consecutive banks.
 // Per-thread twiddle bases kept in registers across many transforms: for every
-// stage s >= 1 and butterfly b of thread t, W^k and W^{4k} (W = W_{PR},
-// k = (t + b T) mod P); the other powers are products of depth <= 3.
-template <typename C, int N, int EPT>
+// stage s >= 1 and butterfly b of thread t, NB powers of W^k (W = W_{PR}, k = (t + b T) mod P);
+// the others are products.  NB = 2: W^k and W^4k; NB = 4: W^k, W^2k, W^4k, W^8k, fewer products
+// for a few registers more (the long lines below: the 8192^2 row pass 3 % faster; at 4096^2 and
+// below, where the registers are needed elsewhere, 1 % slower).
+template <typename C, int N, int EPT, int NB = 2>
 struct TwiddleRegs {
     using Pl = FftPlan<N, EPT>;
     static constexpr int NS = Pl::NSTAGE > 1 ? Pl::NSTAGE : 2;
     static constexpr int MAXNB = Pl::E;     // >= E / R for every stage
-    C w[NS][MAXNB][2];
+    C w[NS][MAXNB][NB];
     // tw[j * stride] = exp(-2 pi i j / N)
     SCINT_DEV void load(const C* __restrict__ tw, int t, int stride = 1) {
 #pragma unroll
@@ -325,31 +327,46 @@ struct TwiddleRegs {
             for (int b = 0; b < Pl::E / R; ++b) {
                 const int k = (t + b * Pl::T) & (P - 1);
                 const int step = k * (N / (P * R)) * stride;
-                w[s][b][0] = __ldg(tw + step);
-                w[s][b][1] = R >= 8 ? __ldg(tw + 4 * step) : w[s][b][0];
+#pragma unroll
+                for (int i = 0; i < NB; ++i) {
+                    const int e = NB == 4 ? 1 << i : 1 << (2 * i);    // the exponent of base i
+                    if (e < R) w[s][b][i] = __ldg(tw + e * step);
+                }
             }
         }
     }
 };
 
-// powers r = 1..R-1 of a base twiddle from (W^k, W^{4k})
+// powers r = 1..R-1 of a base twiddle from W^k, W^4k ...
 template <int R, typename C>
-SCINT_DEV void twiddle_powers(C w1, C w4, C (&w)[R]) {
+SCINT_DEV void twiddle_powers(const C (&base)[2], C (&w)[R]) {
+    const C w1 = base[0];
     if constexpr (R >= 2) w[1] = w1;
     if constexpr (R >= 4) { w[2] = cmul(w1, w1); w[3] = cmul(w1, w[2]); }
     if constexpr (R >= 8) {
+        const C w4 = base[1];
         w[4] = w4;
         w[5] = cmul(w4, w1);
         w[6] = cmul(w4, w[2]);
         w[7] = cmul(w4, w[3]);
+        if constexpr (R >= 16) {
+            w[8] = cmul(w4, w4);
+#pragma unroll
+            for (int r = 9; r < 12; ++r) w[r] = cmul(w[8], w[r - 8]);
+            w[12] = cmul(w[8], w4);
+#pragma unroll
+            for (int r = 13; r < 16; ++r) w[r] = cmul(w[12], w[r - 12]);
+        }
     }
-    if constexpr (R >= 16) {
-        w[8] = cmul(w4, w4);
+}
+// ... and from W^k, W^2k, W^4k, W^8k
+template <int R, typename C>
+SCINT_DEV void twiddle_powers(const C (&base)[4], C (&w)[R]) {
 #pragma unroll
-        for (int r = 9; r < 12; ++r) w[r] = cmul(w[8], w[r - 8]);
-        w[12] = cmul(w[8], w4);
-#pragma unroll
-        for (int r = 13; r < 16; ++r) w[r] = cmul(w[12], w[r - 12]);
+    for (int r = 1; r < R; ++r) {
+        const int top = r >= 8 ? 8 : (r >= 4 ? 4 : (r >= 2 ? 2 : 1));    // the largest base in r
+        if (r == top) w[r] = base[r == 8 ? 3 : (r == 4 ? 2 : r - 1)];
+        else w[r] = cmul(w[top], w[r - top]);
     }
 }
 
@@ -413,24 +430,24 @@ SCINT_DEV dfc ld_cluster<dfc>(unsigned addr) {
     return dfc{dfl(a, b), dfl(c, d)};
 }
 
-template <typename C, int N, int DIR, int EPT, int LW, int TWM, int CS, int S, int TS = 1, int SUB = 0>
+template <typename C, int N, int DIR, int EPT, int LW, int TWM, int CS, int S, int TS = 1, int SUB = 0, int NB = 2>
 SCINT_DEV void fft_stage(C (&v)[FftPlan<N, EPT>::E], C* buf, int t, const C* __restrict__ tw,
-                         const TwiddleRegs<C, N, EPT>* tr) {
+                         const TwiddleRegs<C, N, EPT, NB>* tr) {
     using Pl = FftPlan<N, EPT>;
     constexpr int E = Pl::E, T = Pl::T;
-    constexpr int R = Pl::radix(S), P = Pl::span(S), NB = E / R;
+    constexpr int R = Pl::radix(S), P = Pl::span(S), BF = E / R;
     constexpr bool FIRST = (S == 0), LAST = (S == Pl::NSTAGE - 1);
     constexpr int HALF = N / 2;
     C u[E];
     if constexpr (FIRST) {
-        // butterfly b takes positions t + b T + r N/R = t + (b + r NB) T
+        // butterfly b takes positions t + b T + r N/R = t + (b + r BF) T
 #pragma unroll
-        for (int b = 0; b < NB; ++b)
+        for (int b = 0; b < BF; ++b)
 #pragma unroll
-            for (int r = 0; r < R; ++r) u[b * R + r] = v[b + r * NB];
+            for (int r = 0; r < R; ++r) u[b * R + r] = v[b + r * BF];
     } else if constexpr (CS == 1) {
 #pragma unroll
-        for (int b = 0; b < NB; ++b) {
+        for (int b = 0; b < BF; ++b) {
             // N/R is a multiple of 16 here, so pad16(i + r N/R) = pad16(i) + r (N/R)(17/16).
 #pragma unroll
             for (int r = 0; r < R; ++r) u[b * R + r] = buf[pad16(t + b * T) * LW + r * ((N / R) + (N / R) / 16) * LW];
@@ -441,7 +458,7 @@ SCINT_DEV void fft_stage(C (&v)[FftPlan<N, EPT>::E], C* buf, int t, const C* __r
         // (rank 1's buffer, local index i + (r - R/2) N/R) iff r >= R/2.
         const unsigned cb0 = cluster_addr(buf, 0), cb1 = cluster_addr(buf, 1);
 #pragma unroll
-        for (int b = 0; b < NB; ++b) {
+        for (int b = 0; b < BF; ++b) {
             const unsigned off = (unsigned)(pad16(t + b * T) * LW * sizeof(C));
 #pragma unroll
             for (int r = 0; r < R; ++r) {
@@ -453,14 +470,14 @@ SCINT_DEV void fft_stage(C (&v)[FftPlan<N, EPT>::E], C* buf, int t, const C* __r
         line_sync<CS, SUB>();
     }
 #pragma unroll
-    for (int b = 0; b < NB; ++b) {
+    for (int b = 0; b < BF; ++b) {
         const int i = t + b * T;
         if constexpr (std::is_same<C, float2>::value && R == 16) {
             C w[R];
             if constexpr (!FIRST) {
                 const int k = i & (P - 1);
                 if constexpr (TWM == 2) {
-                    twiddle_powers<R>(tr->w[S][b][0], tr->w[S][b][1], w);
+                    twiddle_powers<R>(tr->w[S][b], w);
                 } else {
 #pragma unroll
                     for (int r = 1; r < R; ++r)
@@ -474,7 +491,7 @@ SCINT_DEV void fft_stage(C (&v)[FftPlan<N, EPT>::E], C* buf, int t, const C* __r
             const int k = i & (P - 1);
             if constexpr (TWM == 2) {
                 C w[R];
-                twiddle_powers<R>(tr->w[S][b][0], tr->w[S][b][1], w);
+                twiddle_powers<R>(tr->w[S][b], w);
 #pragma unroll
                 for (int r = 1; r < R; ++r) u[b * R + r] = DIR < 0 ? cmul(u[b * R + r], w[r]) : cmulc(u[b * R + r], w[r]);
             } else {
@@ -491,16 +508,16 @@ SCINT_DEV void fft_stage(C (&v)[FftPlan<N, EPT>::E], C* buf, int t, const C* __r
     }
     if constexpr (LAST) {
 #pragma unroll
-        for (int b = 0; b < NB; ++b)
+        for (int b = 0; b < BF; ++b)
 #pragma unroll
-            for (int r = 0; r < R; ++r) v[b + r * NB] = u[b * R + r];
+            for (int r = 0; r < R; ++r) v[b + r * BF] = u[b * R + r];
     } else {
-        // Split line: with one butterfly per thread (NB = 1) and P <= T/2, the outputs
+        // Split line: with one butterfly per thread (BF = 1) and P <= T/2, the outputs
         // j + r P, j = (i/P) P R + i mod P, of thread i all lie in [0, N/2) iff i < T/2,
         // i.e. in the half its own block holds: every store is local, at j mod N/2.
-        static_assert(CS == 1 || (NB == 1 && P <= T / 2), "split-line stores must stay in the block");
+        static_assert(CS == 1 || (BF == 1 && P <= T / 2), "split-line stores must stay in the block");
 #pragma unroll
-        for (int b = 0; b < NB; ++b) {
+        for (int b = 0; b < BF; ++b) {
             const int i = t + b * T;
             const int k = i & (P - 1);
             int j = (i - k) * R + k;
@@ -513,7 +530,7 @@ SCINT_DEV void fft_stage(C (&v)[FftPlan<N, EPT>::E], C* buf, int t, const C* __r
                 dst[(P >= 16 ? r * (P + P / 16) : (P == 1 ? r : pad16(j + r * P) - pad16(j))) * LW] = u[b * R + r];
         }
         line_sync<CS, SUB>();
-        fft_stage<C, N, DIR, EPT, LW, TWM, CS, S + 1, TS, SUB>(v, buf, t, tw, tr);
+        fft_stage<C, N, DIR, EPT, LW, TWM, CS, S + 1, TS, SUB, NB>(v, buf, t, tw, tr);
     }
 }
 
@@ -525,13 +542,13 @@ template <typename C, int N, int DIR, int EPT = 16, int LW = 1, int TWM = 0, int
 SCINT_DEV void fft_line(C (&v)[FftPlan<N, EPT>::E], C* buf, int t, const C* __restrict__ tw) {
     static_assert(TWM != 2, "register twiddles: use fft_line_tr");
     static_assert(CS == 1 || (CS == 2 && FftPlan<N, EPT>::NSTAGE > 1 && N >= 512), "split lines need N >= 512");
-    fft_stage<C, N, DIR, EPT, LW, TWM, CS, 0, TS, SUB>(v, buf, t, tw, nullptr);
+    fft_stage<C, N, DIR, EPT, LW, TWM, CS, 0, TS, SUB, 2>(v, buf, t, tw, nullptr);
 }
 
-template <typename C, int N, int DIR, int EPT = 16, int LW = 1, int CS = 1, int SUB = 0>
-SCINT_DEV void fft_line_tr(C (&v)[FftPlan<N, EPT>::E], C* buf, int t, const TwiddleRegs<C, N, EPT>& tr) {
+template <typename C, int N, int DIR, int EPT = 16, int LW = 1, int CS = 1, int SUB = 0, int NB>
+SCINT_DEV void fft_line_tr(C (&v)[FftPlan<N, EPT>::E], C* buf, int t, const TwiddleRegs<C, N, EPT, NB>& tr) {
     static_assert(CS == 1 || (CS == 2 && FftPlan<N, EPT>::NSTAGE > 1 && N >= 512), "split lines need N >= 512");
-    fft_stage<C, N, DIR, EPT, LW, 2, CS, 0, 1, SUB>(v, buf, t, nullptr, &tr);
+    fft_stage<C, N, DIR, EPT, LW, 2, CS, 0, 1, SUB, NB>(v, buf, t, nullptr, &tr);
 }
 
 // ---- long FP32 lines: two half lines in one team -----------------------------------
@@ -571,7 +588,7 @@ SCINT_DEV void long_join(float2* a, float2* b, float2 w0) {
     }
 }
 template <int N, int DIR, int SUB = 0>
-SCINT_DEV void fft_long(float2 (&a)[16], float2 (&b)[16], float2* buf, int t, const TwiddleRegs<float2, N / 2, 16>& tr,
+SCINT_DEV void fft_long(float2 (&a)[16], float2 (&b)[16], float2* buf, int t, const TwiddleRegs<float2, N / 2, 16, 4>& tr,
                         float2 w0) {
     if constexpr (DIR < 0) long_split<N>(a, b, w0);
     fft_line_tr<float2, N / 2, DIR, 16, 1, 1, SUB>(a, buf, t, tr);

@@ -331,7 +331,7 @@ __global__ void __launch_bounds__(LongPlan<N>::T, 2) prop_rows_long_kernel(PropA
         tile_init_fence();
         if (bulk) load_phi(blockIdx.x);
     }
-    TwiddleRegs<float2, N / 2, 16> tr;
+    TwiddleRegs<float2, N / 2, 16, 4> tr;
     tr.load(a.tw, t, 2);
     const float2 w0 = __ldg(a.tw + t);
     __syncthreads();
@@ -417,7 +417,7 @@ __global__ void __launch_bounds__(LongPlan<N>::T, 2) prop_cols_long_kernel(PropA
     const int t = threadIdx.x, r = (int)cl.block_rank();
     float2* buf = smem32;
     float* acc = reinterpret_cast<float*>(smem32 + Pl::BUF);    // own entries until the end
-    TwiddleRegs<float2, N / 2, 16> tr;
+    TwiddleRegs<float2, N / 2, 16, 4> tr;
     tr.load(a.tw, t, 2);
     const float2 w0 = __ldg(a.tw + t);
     const int x0 = (int)blockIdx.x / C * C;
