@@ -198,7 +198,7 @@ def sampling_ratio(p: "ScintParams", lambdas_nm=None) -> float:
         r = lib().scint_sampling_ratio(ctypes.byref(p), None, 0)
     else:
         lam = np.ascontiguousarray(lambdas_nm, dtype=np.float64)
-        r = lib().scint_sampling_ratio(ctypes.byref(p), lam.ctypes.data_as(ctypes.c_void_p), len(lam))
+        r = lib().scint_sampling_ratio(ctypes.byref(p), _host(lam), len(lam))
     if r < 0:
         raise ScintError(1, lib().scint_last_error().decode())   # SCINT_EINVAL
     return r
@@ -206,15 +206,23 @@ def sampling_ratio(p: "ScintParams", lambdas_nm=None) -> float:
 
 def _stream(stream) -> int:
     if stream is None:
-        stream = torch.cuda.current_stream()
+        if not torch.cuda.is_initialized():
+            torch.cuda.init()
+        # the handle of the current device's current stream, without building a Stream object around it
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
-def _dev(t: torch.Tensor, dtype, numel: int, name: str):
+def _dev(t: torch.Tensor, dtype, numel: int, name: str) -> int:
     if not (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype == dtype and t.is_contiguous()
             and t.numel() == numel):
         raise ValueError(f"{name} must be a contiguous CUDA {dtype} tensor with {numel} elements")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
+
+
+def _host(a: Optional[np.ndarray]) -> Optional[int]:
+    """Address of a contiguous host array (data_as would build a typed pointer and cast it)."""
+    return None if a is None else a.__array_interface__["data"][0]
 
 
 def workspace_bytes(p: ScintParams, n_lambda: int = 1) -> int:
@@ -224,7 +232,7 @@ def workspace_bytes(p: ScintParams, n_lambda: int = 1) -> int:
 def _workspace(p: ScintParams, n_lambda: int, workspace, device):
     if workspace is None:
         workspace = torch.empty(workspace_bytes(p, n_lambda), dtype=torch.uint8, device=device)
-    return workspace, ctypes.c_void_p(workspace.data_ptr()), workspace.numel()
+    return workspace, workspace.data_ptr(), workspace.numel()
 
 
 def make_screen(p: ScintParams, out: Optional[torch.Tensor] = None, workspace=None, stream=None,
@@ -270,7 +278,7 @@ def sum_passband(p: ScintParams, phi: torch.Tensor, lambdas_nm: Sequence[float],
     ws, wp, wb = _workspace(p, len(lam), workspace, phi.device)
     _check_warn(lib().scint_sum_passband(
         ctypes.byref(p), _dev(phi, torch.float64, p.n * p.n, "phi"),
-        lam.ctypes.data_as(ctypes.c_void_p), None if w is None else w.ctypes.data_as(ctypes.c_void_p),
+        _host(lam), _host(w),
         len(lam), _dev(out, torch.float32, p.n * p.n, "intensity"), int(bool(accumulate)), wp, wb,
         _stream(stream)))
     return out
@@ -355,7 +363,7 @@ def sum_passband_conjugate(p: ScintParams, phi: torch.Tensor, lambdas_nm: Sequen
         wp, wb = ctypes.c_void_p(workspace.data_ptr()), workspace.numel() * workspace.element_size()
     _check_warn(lib().scint_sum_passband_conjugate(
         ctypes.byref(p), _dev(phi, torch.float64, p.n * p.n, "phi"),
-        lam.ctypes.data_as(ctypes.c_void_p), None if w is None else w.ctypes.data_as(ctypes.c_void_p),
+        _host(lam), _host(w),
         len(lam), _dev(out, torch.float32, p.n * p.n, "intensity"), int(bool(accumulate)), wp, wb,
         _stream(stream)))
     return out
@@ -374,7 +382,7 @@ def lightcurve(p: ScintParams, intensity: torch.Tensor, tracks, n_samples: int,
     if out is None:
         out = torch.empty((tr.shape[0], n_samples), dtype=torch.float32, device=intensity.device)
     _check(lib().scint_lightcurve(ctypes.byref(p), _dev(intensity, torch.float32, p.n * p.n, "intensity"),
-                                  tr.ctypes.data_as(ctypes.c_void_p), tr.shape[0], n_samples,
+                                  _host(tr), tr.shape[0], n_samples,
                                   _dev(out, torch.float32, tr.shape[0] * n_samples, "curves"),
                                   _stream(stream)))
     return out
@@ -411,9 +419,9 @@ def lightcurve_adjoint(p: ScintParams, phi: torch.Tensor, lambdas_nm, tracks, n_
         out = torch.empty((p.n, p.n), dtype=torch.float64, device=phi.device)
     ws, wp, wb = _workspace(p, len(lam), workspace, phi.device)
     _check_warn(lib().scint_lightcurve_adjoint(
-        ctypes.byref(p), _dev(phi, torch.float64, p.n * p.n, "phi"), lam.ctypes.data_as(ctypes.c_void_p),
-        None if w is None else w.ctypes.data_as(ctypes.c_void_p), len(lam),
-        tr.ctypes.data_as(ctypes.c_void_p), tr.shape[0], n_samples,
+        ctypes.byref(p), _dev(phi, torch.float64, p.n * p.n, "phi"), _host(lam),
+        _host(w), len(lam),
+        _host(tr), tr.shape[0], n_samples,
         _dev(grad_curves, torch.float32, tr.shape[0] * n_samples, "grad_curves"),
         _dev(out, torch.float64, p.n * p.n, "grad_phi"), int(bool(accumulate)), wp, wb, _stream(stream)))
     return out
@@ -450,7 +458,7 @@ def batch_items(entries) -> "ctypes.Array":
         arr[i].params = p
         arr[i].phi = _opt_dev(e.get("phi"), torch.float64, nn, "phi")
         arr[i].intensity = _opt_dev(e.get("intensity"), torch.float32, nn, "intensity")
-        arr[i].tracks = tr.ctypes.data if tr.shape[0] else None
+        arr[i].tracks = _host(tr) if tr.shape[0] else None
         arr[i].n_tracks = tr.shape[0]
         arr[i].n_samples = ns
         arr[i].curves = _opt_dev(e.get("curves"), torch.float32, tr.shape[0] * ns, "curves")
@@ -478,8 +486,8 @@ def run_batch(items, lambdas_nm, weights=None, n_lanes: int = 0, workspace: Opti
         if not (workspace.is_cuda and workspace.is_contiguous()):
             raise ValueError("workspace must be a contiguous CUDA tensor")
         wp, wb = ctypes.c_void_p(workspace.data_ptr()), workspace.numel() * workspace.element_size()
-    _check_warn(lib().scint_run_batch(arr, len(arr), lam.ctypes.data_as(ctypes.c_void_p),
-                                 None if w is None else w.ctypes.data_as(ctypes.c_void_p), len(lam),
+    _check_warn(lib().scint_run_batch(arr, len(arr), _host(lam),
+                                 _host(w), len(lam),
                                  int(n_lanes), wp, wb, _stream(stream)))
     return arr
 
@@ -600,8 +608,8 @@ def tune_batch(items, lambdas_nm, weights=None, workspace: Optional[torch.Tensor
     wp, wb = (None, 0) if workspace is None else (ctypes.c_void_p(workspace.data_ptr()),
                                                   workspace.numel() * workspace.element_size())
     lanes, ms, mode = _i(0), ctypes.c_double(0.0), _i(0)
-    _check(lib().scint_tune_batch(arr, len(arr), lam.ctypes.data_as(ctypes.c_void_p),
-                                  None if w is None else w.ctypes.data_as(ctypes.c_void_p), len(lam), wp, wb,
+    _check(lib().scint_tune_batch(arr, len(arr), _host(lam),
+                                  _host(w), len(lam), wp, wb,
                                   ctypes.byref(lanes), ctypes.byref(ms), ctypes.byref(mode), _stream(stream)))
     return lanes.value, ms.value, mode.value
 

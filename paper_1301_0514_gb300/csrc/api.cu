@@ -594,15 +594,18 @@ int fiducial_zone(const scint_params* p, int* i0, int* i1) {
     if (p->margin_km == 0.0) return 1;
     const double L = screen_len(p);
     const double m = taper_margin(p, p->lambda_nm) + 0.5 * refraction_radius(p, p->lambda_nm) + p->source_radius_km;
-    int a = -1, b = -1;
-    for (int i = 0; i < n; ++i) {
+    // first and last pixel whose centre x(i) = (i + 1/2) pixel has m <= x(i) <= L - m: the estimate from
+    // the division is off by one at most, the comparisons below settle it
+    auto inside = [&](int i) {
         const double x = (i + 0.5) * p->pixel_km;
-        if (x >= m && x <= L - m) {
-            if (a < 0) a = i;
-            b = i;
-        }
-    }
-    if (a < 0) return 0;
+        return x >= m && x <= L - m;
+    };
+    const double g = std::fmin(m / p->pixel_km, (double)n);
+    int a = std::max(0, (int)std::floor(g - 0.5) - 1);
+    while (a < n && (a + 0.5) * p->pixel_km < m) ++a;
+    if (a >= n || !inside(a)) return 0;
+    int b = std::min(n - 1, std::max(a, (int)std::ceil(n - g) + 1));
+    while (!inside(b)) --b;
     *i0 = a;
     *i1 = b + 1;
     return 1;

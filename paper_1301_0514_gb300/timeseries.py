@@ -33,7 +33,12 @@ def decorrelation(p: _lib.ScintParams, intensity: torch.Tensor, tracks, separati
     each separation: a (n_tracks, n_separations) float64 device tensor."""
     base = np.asarray(tracks, dtype=np.float64).reshape(-1, 4)
     sep = np.asarray(separations_px, dtype=np.float64)
-    all_tracks = np.concatenate([parallel_tracks(tr, sep) for tr in base], axis=0)
+    # parallel_tracks of every base track at once
+    sin, cos = (np.array([f(th) for th in base[:, 2]])[:, None] for f in (math.sin, math.cos))
+    all_tracks = np.empty((len(base), len(sep), 4))
+    all_tracks[:, :, 0] = base[:, 0:1] - sep * sin
+    all_tracks[:, :, 1] = base[:, 1:2] + sep * cos
+    all_tracks[:, :, 2:] = base[:, None, 2:]
     curves = _lib.lightcurve(p, intensity, all_tracks, n_samples, stream=stream)
     # one launch: every curve against the first curve of its group (separation 0 first)
     r = _lib.curve_correlation(curves, curves, a_rows=len(base), a_stride=len(sep) * n_samples, stream=stream)

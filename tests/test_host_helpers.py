@@ -70,3 +70,18 @@ def test_parallel_tracks_are_parallel_and_offset_perpendicularly(theta):
         assert abs(off @ d) < 1e-12                              # perpendicular to the motion
         assert np.linalg.norm(off) == pytest.approx(abs(s), abs=1e-12)
     np.testing.assert_allclose(tr, O.parallel_tracks(base, seps), rtol=0, atol=1e-12)
+
+
+def test_fiducial_zone_bounds_match_the_oracle_pixel_by_pixel():
+    """The zone's first and last pixel (found from a division and settled by comparisons) against the
+    oracle's mask over every pixel: margins on pixel centres, empty zones, no margin, odd pixel sizes."""
+    rng = np.random.default_rng(20130514)
+    for i in range(400):
+        n = int(2 ** rng.integers(4, 14))
+        pix = float(rng.choice([10.0, 0.1, 7.3, rng.uniform(0.5, 60.0)]))
+        margin = float(rng.choice([-1.0, 0.0, pix * rng.integers(0, n // 2), pix * (rng.integers(0, n // 4) + 0.5)]))
+        kw = dict(n=n, pixel_km=pix, r_diff_km=float(rng.uniform(30.0, 3e6)), lambda_nm=550.0, lambda_ref_nm=550.0,
+                  source_radius_km=float(rng.choice([0.0, rng.uniform(0.0, 0.3) * n * pix])), margin_km=margin)
+        i0, i1, _, exists = S.fiducial_zone(S.params(**kw))
+        o0, o1, whole = O.fiducial_slice(O.ScreenParams(**kw))
+        assert (i0, i1) == (o0, o1) and exists == (not whole), kw
