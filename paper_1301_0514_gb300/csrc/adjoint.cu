@@ -19,28 +19,23 @@
 
 #include "dispatch.cuh"
 #include "propagate.cuh"
+#include "track.cuh"
 
 namespace scint {
 
 // ---- bilinear scatter (transpose of lightcurve_kernel) ---------------------------
-__global__ void lightcurve_adjoint_kernel(CurveAdjArgs a) {
+__global__ void lightcurve_adjoint_kernel(const __grid_constant__ CurveAdjArgs a) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     const int c = blockIdx.y;
     if (s >= a.n_samples || c >= a.n_tracks) return;
-    const Track tr = a.tr[c];
-    const double d = (double)s * tr.ds;
-    const double x = fma(d, tr.c, tr.x0);
-    const double y = fma(d, tr.s, tr.y0);
-    const double fx = floor(x), fy = floor(y);
-    const float tx = (float)(x - fx), ty = (float)(y - fy);
     const int n = a.n;
-    long long ix = (long long)fx % n, iy = (long long)fy % n;
-    if (ix < 0) ix += n;
-    if (iy < 0) iy += n;
-    const int ix1 = (int)(ix + 1 == n ? 0 : ix + 1), iy1 = (int)(iy + 1 == n ? 0 : iy + 1);
+    int ix, iy;
+    float tx, ty;
+    track_sample(a.tr[c], s, n, ix, iy, tx, ty);
+    const int ix1 = (ix + 1) & (n - 1), iy1 = (iy + 1) & (n - 1);
     const float g = a.grad_curves[(size_t)c * a.n_samples + s];
-    atomicAdd(a.grad_map + iy * n + ix, g * (1.0f - tx) * (1.0f - ty));
-    atomicAdd(a.grad_map + iy * n + ix1, g * tx * (1.0f - ty));
+    atomicAdd(a.grad_map + (size_t)iy * n + ix, g * (1.0f - tx) * (1.0f - ty));
+    atomicAdd(a.grad_map + (size_t)iy * n + ix1, g * tx * (1.0f - ty));
     atomicAdd(a.grad_map + (size_t)iy1 * n + ix, g * (1.0f - tx) * ty);
     atomicAdd(a.grad_map + (size_t)iy1 * n + ix1, g * tx * ty);
 }

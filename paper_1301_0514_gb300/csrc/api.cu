@@ -1178,18 +1178,28 @@ int scint_lightcurve(const scint_params* p, const float* intensity, const double
     for (int i = 0; i < 4 * n_tracks; ++i)
         if (!std::isfinite(tracks[i])) return fail(SCINT_EINVAL, "track parameters must be finite");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    for (int t0 = 0; t0 < n_tracks; t0 += kTracksPerLaunch) {
-        CurveArgs a{};
+    // one launch for up to 64 tracks, or up to 512 with the larger argument
+    auto launch = [&](auto& a, int t0, int count) -> int {
         a.n = p->n;
-        a.n_tracks = std::min(kTracksPerLaunch, n_tracks - t0);
+        a.n_tracks = count;
         a.n_samples = n_samples;
         a.intensity = intensity;
         a.curves = curves + (size_t)t0 * n_samples;
-        for (int i = 0; i < a.n_tracks; ++i) {
-            const double* tr = tracks + 4 * (t0 + i);
-            a.tr[i] = Track{tr[0], tr[1], std::cos(tr[2]), std::sin(tr[2]), tr[3]};
+        for (int i = 0; i < count; ++i) a.tr[i] = make_track(p->n, tracks + 4 * (t0 + i));
+        SCINT_LAUNCH(K_LIGHTCURVE, 20.0 * count * (double)n_samples, 0.0, s, launch_lightcurve(a, s));
+        return SCINT_OK;
+    };
+    for (int t0 = 0; t0 < n_tracks;) {
+        const int left = n_tracks - t0, count = std::min(left, left > kTracksPerLaunch ? kManyTracks : kTracksPerLaunch);
+        if (count <= kTracksPerLaunch) {
+            CurveArgs<kTracksPerLaunch> a;
+            rc = launch(a, t0, count);
+        } else {
+            CurveArgs<kManyTracks> a;
+            rc = launch(a, t0, count);
         }
-        SCINT_LAUNCH(K_LIGHTCURVE, 20.0 * a.n_tracks * (double)n_samples, 0.0, s, launch_lightcurve(a, s));
+        if (rc) return rc;
+        t0 += count;
     }
     return ok();
 }
@@ -1320,10 +1330,7 @@ int scint_lightcurve_adjoint(const scint_params* p, const double* phi, const dou
         a.n_samples = n_samples;
         a.grad_curves = grad_curves + (size_t)t0 * n_samples;
         a.grad_map = gmap;
-        for (int i = 0; i < a.n_tracks; ++i) {
-            const double* tr = tracks + 4 * (t0 + i);
-            a.tr[i] = Track{tr[0], tr[1], std::cos(tr[2]), std::sin(tr[2]), tr[3]};
-        }
+        for (int i = 0; i < a.n_tracks; ++i) a.tr[i] = make_track(n, tracks + 4 * (t0 + i));
         SCINT_LAUNCH(K_LC_ADJ, 20.0 * a.n_tracks * (double)n_samples, 0.0, s, launch_lightcurve_adjoint(a, s));
     }
     // the disk filter is real and even, hence self-adjoint

@@ -117,6 +117,11 @@ SCINT_DEV double f2d_bits(float f) {
                                  ((unsigned long long)(b & 0x7FFFFFu) << 29);
     return __longlong_as_double(e ? (long long)d : 0ll);
 }
+// a value f2d_bits does not widen exactly: subnormal, infinite or NaN
+SCINT_DEV bool f2d_unusual(float f) {
+    const unsigned m = __float_as_uint(f) & 0x7FFFFFFFu;
+    return m - 1u < 0x7FFFFFu || m >= 0x7F800000u;
+}
 // s * a as a double: the product in double-float, then one FP64 addition (the FP64 pipe of
 // GB300 is narrow; the conversions of to_double and an FP64 multiply would cost three more)
 SCINT_DEV double scaled_to_double(dfl a, dfl s) {

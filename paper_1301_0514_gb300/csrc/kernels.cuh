@@ -150,15 +150,21 @@ __host__ __device__ constexpr size_t smooth_pairs_floats(int n) { return n >= kS
 cudaError_t launch_smooth_pass(const SmoothArgs& a, int which, cudaStream_t s);
 
 // -------- observables --------------------------------------------------------
-struct Track { double x0, y0, c, s, ds; };
-constexpr int kTracksPerLaunch = 64;
+// A track's start and step as fractions of the periodic grid, 0.64 fixed point (x / n mod 1): sample s
+// sits at x0 + s dx mod 2^64, whose upper bits are the pixel and the next 32 its fraction (resolution
+// n 2^-64 pixels, the wrap is the overflow), so that the kernels need no FP64 operation.
+struct Track { uint64_t x0, y0, dx, dy; };
+Track make_track(int n, const double* t);    // t = (x0, y0, theta, ds) in pixels
+constexpr int kTracksPerLaunch = 64, kManyTracks = 512;
+// K: the tracks an argument holds (kTracksPerLaunch, or kManyTracks for more: 20 KB of arguments)
+template <int K>
 struct CurveArgs {
     int n, n_tracks, n_samples;
     const float* intensity;
     float* curves;           // n_tracks * n_samples (this launch's slice)
-    Track tr[kTracksPerLaunch];
+    Track tr[K];
 };
-cudaError_t launch_lightcurve(const CurveArgs& a, cudaStream_t s);
+template <int K> cudaError_t launch_lightcurve(const CurveArgs<K>& a, cudaStream_t s);
 
 // -------- adjoint -------------------------------------------------------------
 struct CurveAdjArgs {

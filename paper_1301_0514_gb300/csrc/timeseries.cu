@@ -96,24 +96,65 @@ __device__ double block_sum_all(double v) {
     return t;
 }
 
+// U samples of a thread (0 past the end) as doubles, through their bits unless one of them is unusual:
+// on GB300's narrow FP64 pipe a conversion costs as much as two additions.
+template <int U>
+SCINT_DEV void load_widened(const float* x, int s, int step, int n, double (&d)[U]) {
+    float v[U];
+    bool odd = false;
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+        v[k] = s + k * step < n ? x[s + k * step] : 0.0f;
+        odd |= f2d_unusual(v[k]);
+    }
+    if (!odd) {
+#pragma unroll
+        for (int k = 0; k < U; ++k) d[k] = f2d_bits(v[k]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < U; ++k) d[k] = (double)v[k];
+    }
+}
+
+// The FP64 pipe bounds it (384 pairs of 4096 samples: 61 -> 54 us, 85 % busy before): four samples of a thread at a
+// time, each with sums of its own, so that the additions do not wait for one another.
 __global__ void __launch_bounds__(256) correlation_kernel(const float* a, int group, long long a_stride,
                                                           const float* b, int n, double* r) {
     const int i = blockIdx.x;
     const float* x = a + (size_t)(i / group) * a_stride;
     const float* y = b + (size_t)i * n;
-    double sx = 0.0, sy = 0.0;
-    for (int s = threadIdx.x; s < n; s += blockDim.x) {
-        sx += x[s];
-        sy += y[s];
+    constexpr int U = 4;
+    const int step = blockDim.x;
+    double ax[U] = {}, ay[U] = {};
+    for (int s = threadIdx.x; s < n; s += U * step) {
+        double xv[U], yv[U];
+        load_widened(x, s, step, n, xv);
+        load_widened(y, s, step, n, yv);
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+            ax[k] += xv[k];
+            ay[k] += yv[k];
+        }
     }
-    const double mx = block_sum_all(sx) / n, my = block_sum_all(sy) / n;
-    double sxy = 0.0, sxx = 0.0, syy = 0.0;
-    for (int s = threadIdx.x; s < n; s += blockDim.x) {
-        const double dx = x[s] - mx, dy = y[s] - my;
-        sxy = fma(dx, dy, sxy);
-        sxx = fma(dx, dx, sxx);
-        syy = fma(dy, dy, syy);
+    const double mx = block_sum_all((ax[0] + ax[1]) + (ax[2] + ax[3])) / n;
+    const double my = block_sum_all((ay[0] + ay[1]) + (ay[2] + ay[3])) / n;
+    double axy[U] = {}, axx[U] = {}, ayy[U] = {};
+    for (int s = threadIdx.x; s < n; s += U * step) {
+        double xv[U], yv[U];
+        load_widened(x, s, step, n, xv);
+        load_widened(y, s, step, n, yv);
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+            if (s + k * step < n) {
+                const double dx = xv[k] - mx, dy = yv[k] - my;
+                axy[k] = fma(dx, dy, axy[k]);
+                axx[k] = fma(dx, dx, axx[k]);
+                ayy[k] = fma(dy, dy, ayy[k]);
+            }
+        }
     }
+    double sxy = (axy[0] + axy[1]) + (axy[2] + axy[3]), sxx = (axx[0] + axx[1]) + (axx[2] + axx[3]),
+           syy = (ayy[0] + ayy[1]) + (ayy[2] + ayy[3]);
     sxy = block_sum_all(sxy);
     sxx = block_sum_all(sxx);
     syy = block_sum_all(syy);
