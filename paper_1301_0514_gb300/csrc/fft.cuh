@@ -68,6 +68,21 @@ __host__ __device__ constexpr double cos32(int j) {
     }
 }
 
+// cos(2 pi j / 64), j = 0..16 (the first quadrant); sin(2 pi j / 64) = cos(2 pi (16 - j) / 64)
+__host__ __device__ constexpr double cos64q(int j) {
+    switch (j) {
+        case 1: return 0.99518472667219688624;
+        case 3: return 0.95694033573220886494;
+        case 5: return 0.88192126434835502971;
+        case 7: return 0.77301045336273696081;
+        case 9: return 0.63439328416364549822;
+        case 11: return 0.47139673682599764856;
+        case 13: return 0.29028467725446236764;
+        case 15: return 0.09801714032956060199;
+        default: return cos32(j / 2);
+    }
+}
+
 // a * exp(DIR * 2 pi i J16 / 16), J16 a compile-time multiple of 1/16 turn
 template <int J16, int DIR, typename C>
 SCINT_DEV C rot16(C a) {

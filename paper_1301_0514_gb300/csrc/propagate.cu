@@ -496,127 +496,225 @@ bool field_map(CUtensorMap* tm, const float2* work, int n, int count, int strip)
 //     X_{2k} = FFT_{N/2}(a)_k, X_{2k+1} = FFT_{N/2}(b)_k;
 //   inverse, decimation in time: A' = IFFT_{N/2}(Y_{2k}), B' = IFFT_{N/2}(Y_{2k+1}),
 //     y_n = A'_n + W^{-n} B'_n, y_{n+N/2} = A'_n - W^{-n} B'_n.
-// Block r takes the parity-r half-problem, a whole N/2-point line in its own shared
-// memory with block barriers only, and H at the frequencies 2k + r.  Each block forms
-// its a or b from both halves of the input (row pass: the whole line's phases sit in
-// both blocks; column pass: both blocks read the whole column, the second read from
-// L2).  The halves meet once per wavelength: each block publishes its A' or B' and
-// fetches the half of the other one that its outputs need (block 0 makes y_n and
-// y_{n+N/2} for n < N/4, block 1 for N/4 <= n < N/2).  The fetch is followed by a
-// split arrive/wait, so the next wavelength's input is formed while the partner
-// finishes reading.
+// Block r takes the parity-r half-problem, an 8192-point line of two half lines (fft_long: 256
+// threads, two blocks per SM), and H at the frequencies 2k + r.  It reads and writes the
+// line at its quarters n in [r N/4, (r + 1) N/4) and n + N/2 only: each input is read, and each
+// phasor formed, by one block, which keeps its parity's a_n or b_n and hands the other to its
+// partner through shared memory; the same exchange before the last step brings what the block's
+// outputs need.  Per wavelength the halves meet twice, each time a full cluster barrier after the
+// values are published and a split one after they are read.
+// Block 1's quarter is the upper half of its half-problem, so it runs fft_long with the halves
+// swapped: W_{N/2}^n changes sign, and array a is always the part the block keeps.
+// Measured per 16384^2 pass at one wavelength, against 512 threads with sixteen values each, one
+// block per SM, whole lines read by both blocks: rows 3.97 -> 3.13 ms, columns 3.10 -> 2.63 ms (with the transpose).
 template <int N> __host__ __device__ constexpr int psplit_threads() { return FftPlan<N / 2>::T; }
-template <int N> constexpr size_t prow_split_smem() {
+template <int N> constexpr size_t conj_row_split_smem() {
     return (size_t)FftPlan<N / 2>::BUF * sizeof(float2) + (size_t)N * sizeof(long long);
 }
-template <int N> constexpr size_t pcol_split_smem() {
+template <int N> constexpr size_t conj_col_split_smem() {
     return (size_t)(FftPlan<N / 2>::BUF + FftPlan<N / 2>::TWS) * sizeof(float2);
 }
+template <int N> __host__ __device__ constexpr int lsplit_threads() { return LongPlan<N / 2>::T; }
+template <int N> constexpr size_t prow_split_smem() {
+    return (size_t)LongPlan<N / 2>::BUF * sizeof(float2) + (size_t)(N / 2) * sizeof(long long) + 16;
+}
+template <int N> constexpr size_t pcol_split_smem() {
+    return (size_t)LongPlan<N / 2>::BUF * sizeof(float2) + (size_t)(N / 2) * sizeof(float);
+}
+
+// W_N^(n0 + m N/64) from W_N^n0, m < 16
+template <int M> SCINT_DEV float2 quarter_twiddle(float2 w0) {
+    if constexpr (M == 0) return w0;
+    else return cmul(w0, make_float2((float)cos64q(M), (float)-cos64q(16 - M)));
+}
+// The forward exchange: (x0, x1) = x at n = r N/4 + t + m T and n + N/2 (m < 16) become this block's
+// parity: a the part at its own quarter, b the partner's.  Begins by waiting for the partner's last
+// read of buf, ends with a split arrive: wait before buf is written again.
+template <int N, int M = 0>
+SCINT_DEV void quarter_split(float2* x0, float2* x1, float2* out, int r, float2 wq) {
+    if constexpr (M < 16) {
+        const float2 sum = x0[M] + x1[M], dif = cmul(x0[M] - x1[M], quarter_twiddle<M>(wq));
+        x0[M] = r == 0 ? sum : dif;
+        out[pad16(M * LongPlan<N / 2>::T)] = r == 0 ? dif : sum;    // T is a multiple of 16
+        quarter_split<N, M + 1>(x0, x1, out, r, wq);
+    }
+}
+template <int N>
+SCINT_DEV void exchange_forward(float2 (&a)[16], float2 (&b)[16], float2* buf, int t, int r, float2 wq) {
+    constexpr int T = LongPlan<N / 2>::T;
+    cluster_wait();
+    quarter_split<N>(a, b, buf + pad16(t), r, wq);
+    line_sync<2>();
+    const unsigned pb = cluster_addr(buf, (unsigned)(r ^ 1)) + (unsigned)(pad16(t) * sizeof(float2));
+#pragma unroll
+    for (int m = 0; m < 16; ++m) b[m] = ld_cluster<float2>(pb + (unsigned)(m * (T + T / 16) * sizeof(float2)));
+    cluster_arrive();
+}
+// The inverse exchange: a = this block's parity at its own quarter, b at the partner's; on exit
+// a = y_n and b = y_{n+N/2} at its own quarter.  Same barriers.
+template <int N, int M = 0>
+SCINT_DEV void quarter_join(float2* a, float2* q, int r, float2 wq) {
+    if constexpr (M < 16) {
+        const float2 A = r == 0 ? a[M] : q[M], B = r == 0 ? q[M] : a[M];
+        const float2 y = cfma(B, conjc(quarter_twiddle<M>(wq)), A);
+        q[M] = twice_minus(A, y);
+        a[M] = y;
+        quarter_join<N, M + 1>(a, q, r, wq);
+    }
+}
+template <int N>
+SCINT_DEV void exchange_inverse(float2 (&a)[16], float2 (&b)[16], float2* buf, int t, int r, float2 wq) {
+    constexpr int T = LongPlan<N / 2>::T;
+    float2* out = buf + pad16(t);
+#pragma unroll
+    for (int m = 0; m < 16; ++m) out[m * (T + T / 16)] = b[m];
+    line_sync<2>();
+    const unsigned pb = cluster_addr(buf, (unsigned)(r ^ 1)) + (unsigned)(pad16(t) * sizeof(float2));
+#pragma unroll
+    for (int m = 0; m < 16; ++m) b[m] = ld_cluster<float2>(pb + (unsigned)(m * (T + T / 16) * sizeof(float2)));
+    cluster_arrive();
+    quarter_join<N>(a, b, r, wq);
+}
+// signed frequency of fft_long's a[m] (b[m]: + 2) in block r
+template <int N> SCINT_DEV int split_index(int t, int m, int r) { return 4 * signed_index<N / 4, 16>(t, m) + r; }
 
 template <int N>
-__global__ void __launch_bounds__(psplit_threads<N>(), 1) prop_rows_split_kernel(PropArgs a) {
-    constexpr int H2 = N / 2;
-    using Pl = FftPlan<H2>;
-    constexpr int T = Pl::T, E = Pl::E, W = pstrip<N>();
+__global__ void __launch_bounds__(lsplit_threads<N>(), 2) prop_rows_split_kernel(PropArgs a, int bulk) {
+    constexpr int H2 = N / 2, M = N / 4;
+    using Pl = LongPlan<H2>;
+    constexpr int T = Pl::T, W = pstrip<N>();
     extern __shared__ float2 smem32[];
     const int r = (int)cooperative_groups::this_cluster().block_rank();
-    const int t = threadIdx.x;
+    const int t = threadIdx.x, n0 = r * M + t;
     float2* buf = smem32;
-    // the whole line's fixed-point phases: this block converts its half (FP64) and copies
-    // the partner's; each thread reads back only the entries it wrote
-    long long* P = reinterpret_cast<long long*>(smem32 + Pl::BUF);
-    TwiddleRegs<float2, H2, 16> tr;
-    tr.load(a.tw, t, 2);    // the N-point table at even indices
+    long long* Pall = reinterpret_cast<long long*>(smem32 + Pl::BUF);    // this block's quarters
+    long long* P = Pall + t;
+    unsigned long long* bar = reinterpret_cast<unsigned long long*>(Pall + H2);
+    auto load_phi = [&](int y) {
+        const double* phi = a.phi + (size_t)y * N + r * M;
+        tile_expect(bar, H2 * sizeof(double));
+        bulk_load(Pall, phi, M * sizeof(double), bar);
+        bulk_load(Pall + M, phi + H2, M * sizeof(double), bar);
+    };
+    if (t == 0) {
+        tile_init(bar);
+        tile_init_fence();
+        if (bulk) load_phi(blockIdx.x / 2);
+    }
+    TwiddleRegs<float2, M, 16, 4> tr;
+    tr.load(a.tw, t, 4);    // the N-point table at every fourth index
+    const float2 wq = __ldg(a.tw + n0), w1 = __ldg(a.tw + 2 * t), w0 = r ? make_float2(-w1.x, -w1.y) : w1;
+    __syncthreads();
+    cluster_arrive();
+    unsigned parity = 0;
+    bool ok = true;
     // persistent: the cluster takes rows y, y + clusters, ...
 #pragma unroll 1
     for (int y = blockIdx.x / 2; y < N; y += gridDim.x / 2) {
-        const double* phi = a.phi + (size_t)y * N + r * H2;
-        phases_fixed<E>([&](int m) { return phi[t + m * T]; }, [&](int m, long long p) { P[r * H2 + t + m * T] = p; });
-        line_sync<2>();
-        const unsigned pp = cluster_addr(P, (unsigned)(r ^ 1)) + (unsigned)(((r ^ 1) * H2 + t) * sizeof(long long));
-#pragma unroll
-        for (int m = 0; m < E; ++m)
-            P[(r ^ 1) * H2 + t + m * T] = ld_cluster<long long>(pp + (unsigned)(m * T * sizeof(long long)));
-        cluster_arrive();
+        if (bulk) {
+            ok = ok && wait_tile(bar, parity);
+            parity ^= 1;
+            phases_fixed<32>([&](int m) { return __longlong_as_double(P[m * T]); }, [&](int m, long long p) { P[m * T] = p; });
+            tile_reuse_fence();
+        } else {
+            const double* phi = a.phi + (size_t)y * N + n0;
+            phases_fixed<32>([&](int m) { return phi[m * T + (m < 16 ? 0 : H2 - M)]; },
+                             [&](int m, long long p) { P[m * T] = p; });
+        }
 #pragma unroll 1
         for (int l = 0; l < a.lam.count; ++l) {
             const unsigned long long S = a.lam.scale_fx[l];
             const float* sf = a.sf + (size_t)l * N;
-            const float sfy = sf[y];
-            float2 v[E];
+            // 1/N of the inverse transform on the taper of the row; NaN if a copy is missing
+            const float sfy = ok ? sf[y] * (1.0f / N) : __int_as_float(0x7FFFFFFF);
+            float2 va[16], vb[16];
 #pragma unroll
-            for (int m = 0; m < E; ++m) {
-                const int e = t + m * T;
-                const float2 x0 = unit_phasor(P[e], S) * (sfy * __ldg(sf + e));
-                const float2 x1 = unit_phasor(P[e + H2], S) * (sfy * __ldg(sf + e + H2));
-                v[m] = r == 0 ? x0 + x1 : cmul(x0 - x1, __ldg(a.tw + e));
+            for (int m = 0; m < 16; ++m) {
+                va[m] = unit_phasor(P[m * T], S) * (sfy * __ldg(sf + n0 + m * T));
+                vb[m] = unit_phasor(P[m * T + M], S) * (sfy * __ldg(sf + n0 + m * T + H2));
             }
-            cluster_wait();      // the partner has read this block's buffer
-            fft_line_tr<float2, H2, -1, 16, 1>(v, buf, t, tr);
+            exchange_forward<N>(va, vb, buf, t, r, wq);
+            // every thread is past a barrier, hence done with the phases at the last wavelength
+            if (bulk && t == 0 && l + 1 == a.lam.count && y + (int)gridDim.x / 2 < N) load_phi(y + gridDim.x / 2);
+            cluster_wait();
+            fft_long<H2, -1>(va, vb, buf, t, tr, w0);
             const unsigned long long hc = a.lam.h_fx[l];
 #pragma unroll
-            for (int m = 0; m < E; ++m) v[m] = cmul(v[m], transfer_at(hc, 2 * (t + m * T) + r, N));
-            fft_line_tr<float2, H2, +1, 16, 1>(v, buf, t, tr);
-            float2* dst = a.work + (size_t)l * N * N;
-            split_combine<float2, H2>(v, buf, t, r, a.tw, [&](int, int n, float2 y0, float2 y1) {
-                dst[strip_index<W>(y, n, N)] = y0;
-                dst[strip_index<W>(y, n + H2, N)] = y1;
-            });
+            for (int m = 0; m < 16; ++m) {
+                const int f = split_index<N>(t, m, r);
+                va[m] = cmul(va[m], transfer_signed(hc, f));
+                vb[m] = cmul(vb[m], transfer_signed(hc, f + 2));
+            }
+            fft_long<H2, +1>(va, vb, buf, t, tr, w0);
+            exchange_inverse<N>(va, vb, buf, t, r, wq);
+            float2* dst = a.work + (size_t)l * N * N + strip_index<W>(y, n0, N);
+#pragma unroll
+            for (int m = 0; m < 16; ++m) {
+                dst[(size_t)(m * T) * N] = va[m];
+                dst[(size_t)(m * T + H2) * N] = vb[m];
+            }
         }
-        cluster_wait();    // the partner is done with this block's buffers (no block leaves before)
+    }
+    cluster_wait();    // no block leaves before its buffer is read
+    if (!ok) {
+        wait_tile(bar, 0);
+        wait_tile(bar, 1);
     }
 }
 
 template <int N>
-__global__ void __launch_bounds__(psplit_threads<N>(), 1) prop_cols_split_kernel(PropArgs a) {
-    constexpr int H2 = N / 2;
-    using Pl = FftPlan<H2>;
-    constexpr int T = Pl::T, E = Pl::E, WL = pstrip<N>();
+__global__ void __launch_bounds__(lsplit_threads<N>(), 2) prop_cols_split_kernel(PropArgs a) {
+    constexpr int H2 = N / 2, M = N / 4;
+    using Pl = LongPlan<H2>;
+    constexpr int T = Pl::T, WL = pstrip<N>();
     extern __shared__ float2 smem32[];
     const int r = (int)cooperative_groups::this_cluster().block_rank();
-    const int t = threadIdx.x;
+    const int t = threadIdx.x, n0 = r * M + t;
     float2* buf = smem32;
-    float2* tws = smem32 + Pl::BUF;
-    fill_twiddle_table<float2, H2>(tws, a.tw, t, T, 2);
+    float* acc = reinterpret_cast<float*>(smem32 + Pl::BUF) + t;    // own entries
+    TwiddleRegs<float2, M, 16, 4> tr;
+    tr.load(a.tw, t, 4);
+    const float2 wq = __ldg(a.tw + n0), w1 = __ldg(a.tw + 2 * t), w0 = r ? make_float2(-w1.x, -w1.y) : w1;
+    cluster_arrive();
     // persistent: the cluster takes columns x, x + clusters, ...
 #pragma unroll 1
     for (int x = blockIdx.x / 2; x < N; x += gridDim.x / 2) {
-        float acc[E];
-#pragma unroll
-        for (int m = 0; m < E; ++m) acc[m] = 0.0f;
-        cluster_arrive();    // the first wait below also publishes the twiddle table to the block
 #pragma unroll 1
         for (int l = 0; l < a.lam.count; ++l) {
-            const float2* src = a.work + (size_t)l * N * N + (size_t)(x / WL) * N * WL + (x % WL);
-            float2 v[E];
+            const float2* src = a.work + (size_t)l * N * N + (size_t)(x / WL) * N * WL + (x % WL) + (size_t)n0 * WL;
+            float2 va[16], vb[16];
 #pragma unroll
-            for (int m = 0; m < E; ++m) {
-                const int e = t + m * T;
-                const float2 x0 = src[(size_t)e * WL], x1 = src[(size_t)(e + H2) * WL];
-                v[m] = r == 0 ? x0 + x1 : cmul(x0 - x1, __ldg(a.tw + e));
+            for (int m = 0; m < 16; ++m) {
+                va[m] = __ldcg(src + (size_t)(m * T) * WL);
+                vb[m] = __ldcg(src + (size_t)(m * T + H2) * WL);
             }
+            exchange_forward<N>(va, vb, buf, t, r, wq);
             cluster_wait();
-            fft_line<float2, H2, -1, 16, 1, 1, 1>(v, buf, t, tws);
+            fft_long<H2, -1>(va, vb, buf, t, tr, w0);
             const unsigned long long hc = a.lam.h_fx[l];
 #pragma unroll
-            for (int m = 0; m < E; ++m) v[m] = cmul(v[m], transfer_at(hc, 2 * (t + m * T) + r, N));
-            fft_line<float2, H2, +1, 16, 1, 1, 1>(v, buf, t, tws);
-            const float wl = a.lam.weight[l];
-            split_combine<float2, H2>(v, buf, t, r, a.tw, [&](int j, int, float2 y0, float2 y1) {
-                acc[2 * j] = fmaf(wl, fmaf(y0.x, y0.x, y0.y * y0.y), acc[2 * j]);
-                acc[2 * j + 1] = fmaf(wl, fmaf(y1.x, y1.x, y1.y * y1.y), acc[2 * j + 1]);
-            });
-        }
-        cluster_wait();
-        // column-major, so that the stores coalesce; transpose_add_kernel puts it in place
-        float* col = a.scratch + (size_t)x * N;
+            for (int m = 0; m < 16; ++m) {
+                const int f = split_index<N>(t, m, r);
+                va[m] = cmul(va[m], transfer_signed(hc, f));
+                vb[m] = cmul(vb[m], transfer_signed(hc, f + 2));
+            }
+            fft_long<H2, +1>(va, vb, buf, t, tr, w0);
+            exchange_inverse<N>(va, vb, buf, t, r, wq);
+            // 1/N of H_y, squared, on the weight (prop_cols_body); the last sum goes out column-major, so that
+            // the stores coalesce (transpose_add_kernel puts it in place)
+            const float wl = a.lam.weight[l] * (1.0f / ((float)N * (float)N));
+            const bool last = l + 1 == a.lam.count;
+            float* col = last ? a.scratch + (size_t)x * N + n0 : acc;
+            const int half = last ? H2 : M;
 #pragma unroll
-        for (int j = 0; j < E / 2; ++j) {
-            const int n = t + (j + r * (E / 2)) * T;
-            col[n] = acc[2 * j];
-            col[n + H2] = acc[2 * j + 1];
+            for (int m = 0; m < 16; ++m) {
+                const float p = l ? acc[m * T] : 0.0f, q = l ? acc[m * T + M] : 0.0f;
+                col[m * T] = fmaf(wl, fmaf(va[m].x, va[m].x, va[m].y * va[m].y), p);
+                col[m * T + half] = fmaf(wl, fmaf(vb[m].x, vb[m].x, vb[m].y * vb[m].y), q);
+            }
         }
     }
+    cluster_wait();
 }
 
 // One-FFT mode (Eq. intens, Eq. Gxy) at N = 16384: forward transforms only, so the
@@ -744,14 +842,23 @@ template <bool CONJ>
 cudaError_t launch_rows(const PropArgs& a, cudaStream_t s) {
     return dispatch_n(a.n, [&](auto nc) -> cudaError_t {
         constexpr int N = decltype(nc)::value;
-        if constexpr (pcs<N>() == 2) {
-            static_assert(prow_split_smem<N>() <= kMaxSmem, "split row pass does not fit");
-            auto k = CONJ ? conj_rows_split_kernel<N> : prop_rows_split_kernel<N>;
+        if constexpr (pcs<N>() == 2 && CONJ) {
+            static_assert(conj_row_split_smem<N>() <= kMaxSmem, "split row pass does not fit");
+            auto k = conj_rows_split_kernel<N>;
+            cudaError_t e = set_smem(k, conj_row_split_smem<N>());
+            int nc = 0;
+            if (e == cudaSuccess) e = active_clusters(k, 2, psplit_threads<N>(), conj_row_split_smem<N>(), &nc);
+            if (e != cudaSuccess) return e;
+            return launch_k(k, 2, dim3(2 * std::min(nc, N)), dim3(psplit_threads<N>()), conj_row_split_smem<N>(), s, a);
+        } else if constexpr (pcs<N>() == 2) {
+            static_assert(2 * (prow_split_smem<N>() + 1024) <= 228 * 1024, "two blocks per SM");
+            auto k = prop_rows_split_kernel<N>;
             cudaError_t e = set_smem(k, prow_split_smem<N>());
             int nc = 0;
-            if (e == cudaSuccess) e = active_clusters(k, 2, psplit_threads<N>(), prow_split_smem<N>(), &nc);
+            if (e == cudaSuccess) e = active_clusters(k, 2, lsplit_threads<N>(), prow_split_smem<N>(), &nc);
             if (e != cudaSuccess) return e;
-            return launch_k(k, 2, dim3(2 * std::min(nc, N)), dim3(psplit_threads<N>()), prow_split_smem<N>(), s, a);
+            return launch_k(k, 2, dim3(2 * std::min(nc, N)), dim3(lsplit_threads<N>()), prow_split_smem<N>(), s, a,
+                            (int)(reinterpret_cast<uintptr_t>(a.phi) % 16 == 0));
         } else if constexpr (prow_smem<N>() > kMaxSmem || pcol_smem<N, true>() > kMaxSmem) {
             return cudaErrorNotSupported;
         } else {
@@ -790,15 +897,17 @@ cudaError_t launch_cols(const PropArgs& a, cudaStream_t s) {
     return dispatch_n(a.n, [&](auto nc) -> cudaError_t {
         constexpr int N = decltype(nc)::value;
         if constexpr (pcs<N>() == 2) {
-            static_assert(pcol_split_smem<N>() <= kMaxSmem, "split column pass does not fit");
             const bool to_scratch = !CONJ || a.conj.direct;    // intensity through the transpose
             if (to_scratch && !a.scratch) return cudaErrorInvalidValue;
+            constexpr size_t smem = CONJ ? conj_col_split_smem<N>() : pcol_split_smem<N>();
+            constexpr int threads = CONJ ? psplit_threads<N>() : lsplit_threads<N>();
+            static_assert(smem <= kMaxSmem, "split column pass does not fit");
             auto k = CONJ ? conj_cols_split_kernel<N> : prop_cols_split_kernel<N>;
-            cudaError_t e = set_smem(k, pcol_split_smem<N>());
+            cudaError_t e = set_smem(k, smem);
             int nc = 0;
-            if (e == cudaSuccess) e = active_clusters(k, 2, psplit_threads<N>(), pcol_split_smem<N>(), &nc);
+            if (e == cudaSuccess) e = active_clusters(k, 2, threads, smem, &nc);
             if (e != cudaSuccess) return e;
-            e = launch_k(k, 2, dim3(2 * std::min(nc, N)), dim3(psplit_threads<N>()), pcol_split_smem<N>(), s, a);
+            e = launch_k(k, 2, dim3(2 * std::min(nc, N)), dim3(threads), smem, s, a);
             if (e != cudaSuccess || !to_scratch) return e;
             transpose_add_kernel<<<dim3(N / 32, N / 32), 256, 0, s>>>(a.scratch, a.intensity, N, a.accumulate);
             return cudaGetLastError();
