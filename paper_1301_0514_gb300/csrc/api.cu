@@ -136,6 +136,15 @@ size_t ws_prop(int n, int g) {
     return up((size_t)n * 8) + up((size_t)g * n * 4) + up((size_t)field_slots(g) * n * n * 8) +
            (n >= kSplitN ? up((size_t)n * n * 4) : 0);
 }
+// the transfer function's tables of a group: part of every workspace size given out, taken where
+// there is room (group_tables), so that a workspace of ws_prop alone still does
+size_t ws_transfer(int n, int g) { return up((size_t)g * transfer_entries(n) * 8); }
+// the largest group of up to g wavelengths that a workspace of `bytes` holds besides `rest`; one smaller,
+// rather than without its tables
+int group_size(int n, int g, size_t bytes, size_t rest) {
+    while (g > 1 && rest + ws_prop(n, g) + ws_transfer(n, g) > bytes) --g;
+    return g;
+}
 size_t ws_prop64(int n) { return n <= kMax64N ? up((size_t)n * 16) + up((size_t)n * n * 16) : 0; }
 size_t ws_smooth(int n) {
     return up((size_t)n * 8) + up((size_t)(n / 2 + 1) * n * 8) + up(smooth_pairs_floats(n) * 4);
@@ -432,9 +441,20 @@ void fill_lambda(LambdaSet& ls, int i, const scint_params* p, double lam, double
     ls.h_fx[i] = 0ull - ((uint64_t)std::llround(std::ldexp(c - std::floor(c), 52)) << 12);
 }
 
+// A place for the group's transfer-function tables: after its buffers (cg), or for one wavelength in
+// the twiddle slot when the twiddles are kept elsewhere (transfer_entries(n) <= n); else the passes
+// evaluate it (a workspace of the least size under a capture that has no kept twiddles).
+void group_tables(TableArgs& ta, PropArgs& pa, const Carver& cg, float2* slot, const float2* tw) {
+    const size_t bytes = ws_transfer(ta.n, ta.count);
+    if (cg.used + bytes <= cg.size) ta.h = reinterpret_cast<float2*>(cg.base + cg.used);
+    else if (ta.count == 1 && tw != slot) ta.h = slot;
+    for (int i = 0; i < ta.count; ++i) ta.h_fx[i] = pa.lam.h_fx[i];
+    pa.h = ta.h;
+}
+
 // Propagate one wavelength group [l0, l0 + g) into the intensity map.
 int run_group(const scint_params* p, const double* phi, const double* lam, const double* wts,
-              int l0, int g, float* intensity, int accumulate, Carver& c, const float2* tw,
+              int l0, int g, float* intensity, int accumulate, Carver& c, float2* slot, const float2* tw,
               cudaStream_t s) {
     const int n = p->n;
     static_assert(kMaxLambda >= SCINT_MAX_LAMBDA, "lambda table size");
@@ -456,6 +476,7 @@ int run_group(const scint_params* p, const double* phi, const double* lam, const
     pa.sf = ta.sf;
     pa.work = cg.take<float2>((size_t)field_slots(g) * n * n * 8);
     pa.scratch = n >= kSplitN ? cg.take<float>((size_t)n * n * 4) : nullptr;
+    group_tables(ta, pa, cg, slot, tw);
     pa.intensity = intensity;
     pa.accumulate = accumulate;
     pa.one = 1.0f;
@@ -486,19 +507,17 @@ int passband_impl(const scint_params* p, const double* phi, const double* lambda
     if (weights) w.assign(weights, weights + n_lambda);
     const int n = p->n;
     // group size: all wavelengths if the workspace allows, else the largest that fits
-    int g = n_lambda;
-    if (ws) {
-        while (g > 1 && ws_prop(n, g) > ws_bytes) --g;
-    }
+    const int g = ws ? group_size(n, n_lambda, ws_bytes, 0) : n_lambda;
     Carver c{};
-    rc = resolve_ws(ws, ws_bytes, ws_prop(n, g), s, &c);
+    rc = resolve_ws(ws, ws_bytes, ws_prop(n, g) + (ws ? 0 : ws_transfer(n, g)), s, &c);
     if (rc) return rc;
+    float2* slot = c.take<float2>((size_t)n * 8);
     const float2* tw = nullptr;
-    rc = twiddles32(n, keep_tables, s, c.take<float2>((size_t)n * 8), &tw);
+    rc = twiddles32(n, keep_tables, s, slot, &tw);
     if (rc) return rc;
     for (int l0 = 0; l0 < n_lambda; l0 += g) {
         const int gg = std::min(g, n_lambda - l0);
-        rc = run_group(p, phi, lambdas, w.data(), l0, gg, intensity, accumulate || l0 > 0, c, tw, s);
+        rc = run_group(p, phi, lambdas, w.data(), l0, gg, intensity, accumulate || l0 > 0, c, slot, tw, s);
         if (rc) return rc;
     }
     return ok();
@@ -673,8 +692,12 @@ int validate_passband(const scint_params* p, const double* lambdas, const double
 }
 size_t aligned_bytes(size_t b) { return up(b); }
 size_t forward_workspace_bytes(int n, int g) {
-    return std::max(std::max(ws_synth(n), ws_prop(n, g)), std::max(ws_smooth(n), ws_moments()));
+    return std::max(std::max(ws_synth(n), ws_prop(n, g) + ws_transfer(n, g)), std::max(ws_smooth(n), ws_moments()));
 }
+size_t least_workspace_bytes(int n) {
+    return std::max(std::max(ws_synth(n), ws_prop(n, 1)), std::max(ws_smooth(n), ws_moments()));
+}
+size_t transfer_table_bytes(int n, int n_lambda) { return ws_transfer(n, n_lambda); }
 int pool_workspace(size_t bytes, cudaStream_t s, void** out) { return pool_get(bytes, s, out); }
 bool autotune_on() { return g_autotune.load() != 0; }
 bool has_plan(int n) { return plan_known(n); }
@@ -717,7 +740,7 @@ PersistLayout persist_layout(const int* sizes, int n, int n_lambda, int n_slots)
     L.sf = off;
     for (int i = 0; i < n; ++i) off += up((size_t)n_lambda * sizes[i] * 4);
     L.slots = off;
-    L.slot_bytes = std::max(up((size_t)field_slots(n_lambda) * nmax * nmax * 8), forward_workspace_bytes(nmax, 1));
+    L.slot_bytes = std::max(up((size_t)field_slots(n_lambda) * nmax * nmax * 8), least_workspace_bytes(nmax));
     off += (size_t)n_slots * L.slot_bytes;
     L.total = off;
     return L;
@@ -732,7 +755,7 @@ void persist_testing(int withhold, int wait_limit) {
 
 int persist_propagate(const scint_params* const* params, const double* const* phis, float* const* intensities,
                       int n, const double* lambdas, const double* weights, int n_lambda, char* ws, int n_slots,
-                      int** status_out, cudaStream_t s) {
+                      char* tables, int** status_out, cudaStream_t s) {
     std::vector<int> sizes(n);
     for (int i = 0; i < n; ++i) sizes[i] = params[i]->n;
     const PersistLayout L = persist_layout(sizes.data(), n, n_lambda, n_slots);
@@ -784,6 +807,12 @@ int persist_propagate(const scint_params* const* params, const double* const* ph
         }
         ta.sf = reinterpret_cast<float*>(sf_of[i]);
         pa.sf = ta.sf;
+        if (tables) {
+            ta.h = reinterpret_cast<float2*>(tables);
+            tables += ws_transfer(nn, n_lambda);
+            for (int l = 0; l < n_lambda; ++l) ta.h_fx[l] = pa.lam.h_fx[l];
+            pa.h = ta.h;
+        }
         pa.work = reinterpret_cast<float2*>(ws + L.slots + (size_t)(k % n_slots) * L.slot_bytes);
         pa.scratch = nullptr;
         pa.intensity = intensities[i];
@@ -879,10 +908,10 @@ size_t scint_workspace_bytes(const scint_params* p, int n_lambda) {
     if (check_params(p) || n_lambda < 1) return 0;
     const int n = p->n;
     size_t b = ws_synth(n);
-    b = std::max(b, ws_prop(n, std::min(n_lambda, SCINT_MAX_LAMBDA)));
+    const int g = std::min(n_lambda, SCINT_MAX_LAMBDA);
     b = std::max(b, ws_smooth(n));
     b = std::max(b, ws_moments());
-    b = std::max(b, ws_adjoint(n, std::min(n_lambda, SCINT_MAX_LAMBDA)));
+    b = std::max(b, ws_adjoint(n, g) + ws_transfer(n, g));    // the propagation's part included
     b = std::max(b, ws_prop64(n));
     return b;
 }
@@ -1045,7 +1074,7 @@ int scint_tune(int n, int n_lambda, scint_plan* out, void* stream) {
     scint_plan prev{};
     if (had) plan_for(n, &prev);
     if (cand.size() > 1) {
-        const size_t wsb = ws_prop(n, g);
+        const size_t wsb = ws_prop(n, g) + ws_transfer(n, g);
         void *phi = nullptr, *inten = nullptr, *ws = nullptr;
         cudaEvent_t e0 = nullptr, e1 = nullptr;
         auto cleanup = [&] {
@@ -1305,20 +1334,18 @@ int scint_lightcurve_adjoint(const scint_params* p, const double* phi, const dou
     g_warning.clear();
     note_sampling(p, lambdas_nm, n_lambda);
     const int n = p->n;
-    int g = n_lambda;
-    if (workspace) {
-        while (g > 1 && ws_adjoint(n, g) > workspace_bytes) --g;
-    }
+    const int g = workspace ? group_size(n, n_lambda, workspace_bytes, ws_adjoint(n, 1) - ws_prop(n, 1)) : n_lambda;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     Carver c{};
-    rc = resolve_ws(workspace, workspace_bytes, ws_adjoint(n, g), s, &c);
+    rc = resolve_ws(workspace, workspace_bytes, ws_adjoint(n, g) + (workspace ? 0 : ws_transfer(n, g)), s, &c);
     if (rc) return rc;
     float* gmap = c.take<float>((size_t)n * n * 4);
     float2* spec = c.take<float2>((size_t)(n / 2 + 1) * n * 8);
     float2* spairs = smooth_pairs_floats(n) ? c.take<float2>(smooth_pairs_floats(n) * 4) : nullptr;
     Carver cp = c;                       // propagation buffers: twiddles, then group tables and fields
     const float2* tw = nullptr;
-    rc = twiddles32(n, true, s, cp.take<float2>((size_t)n * 8), &tw);
+    float2* slot = cp.take<float2>((size_t)n * 8);
+    rc = twiddles32(n, true, s, slot, &tw);
     if (rc) return rc;
     const double nn = (double)n * n;
     // g_I = B^T g_c
@@ -1365,7 +1392,9 @@ int scint_lightcurve_adjoint(const scint_params* p, const double* phi, const dou
         Carver cg = cp;
         ta.sf = cg.take<float>((size_t)gg * n * 4);
         pa.sf = ta.sf;
-        pa.work = cg.take<float2>((size_t)gg * n * n * 8);
+        pa.work = cg.take<float2>((size_t)field_slots(gg) * n * n * 8);
+        if (n >= kSplitN) cg.take<float>((size_t)n * n * 4);    // the forward columns' scratch: not used here
+        group_tables(ta, pa, cg, slot, tw);
         AdjArgs aa{};
         aa.n = n;
         aa.phi = phi;

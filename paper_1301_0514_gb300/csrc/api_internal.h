@@ -30,6 +30,10 @@ size_t aligned_bytes(size_t b);
 // Workspace of the forward path of one N x N screen (synthesis, a passband
 // group of g wavelengths, smoothing, moments): the maximum over its calls.
 size_t forward_workspace_bytes(int n, int g);
+// The least that the same calls accept (one wavelength, no room for the transfer function's tables),
+// and those tables' bytes.
+size_t least_workspace_bytes(int n);
+size_t transfer_table_bytes(int n, int n_lambda);
 // The per-device pool: at least `bytes`, grown outside stream capture only.
 int pool_workspace(size_t bytes, cudaStream_t s, void** out);
 // Destroy the batch executor's streams and events (csrc/batch.cu).
@@ -55,11 +59,12 @@ bool persist_batch_supported(const int* sizes, int n);
 constexpr int kPersistMaxScreensHost = 256;   // screens one persistent launch takes (kPersistMaxScreens)
 // Run the propagation of every screen (phi in, intensity out; passband lambdas/weights)
 // in one persistent launch on stream s; ws must hold persist_layout(...).total bytes.
+// tables: room for transfer_table_bytes of every screen, one after the other, or NULL.
 // withhold / wait_limit: see scint_testing_persist.  The status word (0 or
 // SCINT_ETIMEOUT once the launch has run) is at *status_out.
 int persist_propagate(const scint_params* const* params, const double* const* phis, float* const* intensities,
                       int n, const double* lambdas, const double* weights, int n_lambda, char* ws, int n_slots,
-                      int** status_out, cudaStream_t s);
+                      char* tables, int** status_out, cudaStream_t s);
 void persist_testing(int withhold, int wait_limit);
 
 }  // namespace scint

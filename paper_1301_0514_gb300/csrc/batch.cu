@@ -91,6 +91,13 @@ size_t lane_bytes(const Sizes& z, int g) {
            scint::forward_workspace_bytes(z.n_max, g);
 }
 
+// The least that a lane takes: one wavelength at a time, without the transfer function's tables.
+size_t least_lane_bytes(const Sizes& z) {
+    const size_t nn = (size_t)z.n_max * z.n_max;
+    return (z.scratch_phi ? scint::aligned_bytes(nn * 8) : 0) + (z.scratch_i ? scint::aligned_bytes(nn * 4) : 0) +
+           scint::least_workspace_bytes(z.n_max);
+}
+
 // Host checks of the whole batch, before anything is launched.
 int check_batch(const scint_batch_item* items, int n_items, const double* lambdas, const double* weights,
                 int n_lambda, int n_lanes) {
@@ -186,6 +193,14 @@ size_t persistent_bytes(const scint_batch_item* items, int n_items, int n_lambda
     return b;
 }
 
+// bytes of the transfer function's tables of every screen: part of the size given out, used where
+// the workspace has room for them
+size_t persistent_table_bytes(const scint_batch_item* items, int n_items, int n_lambda) {
+    size_t b = 0;
+    for (int i = 0; i < n_items; ++i) b += scint::transfer_table_bytes(items[i].params.n, n_lambda);
+    return b;
+}
+
 // smoothing, light curves and m of one item (the tail of run_item)
 int finish_item(const scint_batch_item& it, float* inten, void* ws, size_t wsb, cudaStream_t s) {
     const scint_params* p = &it.params;
@@ -213,6 +228,7 @@ int run_persistent(const scint_batch_item* items, int n_items, const double* lam
     for (int i = 0; i < n_items; ++i) sizes[i] = items[i].params.n;
     const scint::PersistLayout PL = scint::persist_layout(sizes.data(), n_items, n_lambda, n_slots);
     const size_t need = persistent_bytes(items, n_items, n_lambda, n_slots);
+    const size_t tables = persistent_table_bytes(items, n_items, n_lambda);
     int rc;
     if (workspace) {
         if (reinterpret_cast<uintptr_t>(workspace) % 256)
@@ -223,8 +239,9 @@ int run_persistent(const scint_batch_item* items, int n_items, const double* lam
                      workspace_bytes, need);
             return set_error(SCINT_ENOMEM, msg);
         }
-    } else if ((rc = scint::pool_workspace(need, caller, &workspace))) {
-        return rc;
+    } else {
+        workspace_bytes = need + tables;
+        if ((rc = scint::pool_workspace(workspace_bytes, caller, &workspace))) return rc;
     }
     char* ws = static_cast<char*>(workspace);
     char* cur = ws + PL.total;
@@ -293,7 +310,7 @@ int run_persistent(const scint_batch_item* items, int n_items, const double* lam
     if (rc) return rc;
     int* status = nullptr;
     if ((rc = scint::persist_propagate(prm.data(), phc.data(), in.data(), n_items, lambdas, weights, n_lambda, ws,
-                                       n_slots, &status, caller)))
+                                       n_slots, workspace_bytes >= need + tables ? ws + need : nullptr, &status, caller)))
         return rc;
     {
         std::lock_guard<std::mutex> sl(g_status_mu);
@@ -348,7 +365,8 @@ size_t scint_batch_workspace_bytes(const scint_batch_item* items, int n_items, i
     size_t b = (size_t)std::min(n_lanes, n_items) * lane_bytes(z, std::min(n_lambda, SCINT_MAX_LAMBDA));
     if (persistent_ok(items, n_items))
         b = std::max(b, persistent_bytes(items, n_items, std::min(n_lambda, SCINT_MAX_LAMBDA),
-                                         persist_slots(n_lanes, n_items)));
+                                         persist_slots(n_lanes, n_items)) +
+                            persistent_table_bytes(items, n_items, std::min(n_lambda, SCINT_MAX_LAMBDA)));
     return b;
 }
 
@@ -384,10 +402,10 @@ int scint_run_batch(const scint_batch_item* items, int n_items, const double* la
         if (reinterpret_cast<uintptr_t>(workspace) % 256)
             return set_error(SCINT_EINVAL, "workspace must be 256-byte aligned");
         slice = workspace_bytes / n_lanes / 256 * 256;
-        if (slice < lane_bytes(z, 1)) {
+        if (slice < least_lane_bytes(z)) {
             char msg[160];
             snprintf(msg, sizeof msg, "workspace of %zu bytes is smaller than the %zu bytes needed by %d lanes",
-                     workspace_bytes, (size_t)n_lanes * lane_bytes(z, 1), n_lanes);
+                     workspace_bytes, (size_t)n_lanes * least_lane_bytes(z), n_lanes);
             return set_error(SCINT_ENOMEM, msg);
         }
     } else {
@@ -515,7 +533,7 @@ int scint_tune_batch(const scint_batch_item* items, int n_items, const double* l
             if (rc) break;
             if (workspace) {
                 const size_t need = mode == 1 ? persistent_bytes(items, n_items, n_lambda, persist_slots(lanes, n_items))
-                                              : (size_t)lanes * lane_bytes(z, 1);
+                                              : (size_t)lanes * least_lane_bytes(z);
                 if (workspace_bytes < need) continue;
             }
             double t = 1e300;

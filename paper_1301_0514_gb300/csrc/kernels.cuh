@@ -79,6 +79,7 @@ struct PropArgs {
     const double* phi;       // n*n radians at lambda_ref
     const float2* tw;        // FP32 twiddles
     const float* sf;         // per lambda: n taper values
+    const float2* h;         // per lambda: transfer_entries(n) values of H_x, or NULL (each pass evaluates its own)
     float2* work;            // per lambda: n*n complex64, strip layout
     float* intensity;        // n*n
     int accumulate;          // add to intensity instead of overwriting
@@ -87,11 +88,17 @@ struct PropArgs {
     ConjSet conj;            // used by the one-FFT mode only
     float one;               // 1.0f: the multiplier of the packed passes' additions (fft2.cuh)
 };
-// The taper table of a wavelength group (SF at the pixel centres, per wavelength).
+// The tables of a wavelength group, per wavelength: the taper SF at the pixel centres and, if h is
+// set, the transfer function H_x.  H_x is even: up to n = 4096 entry i is H_x(i), i = 0..n/2 (and one of
+// padding, for 16-byte rows); at 8192 entry i is frequency i in FFT order; at kSplitN the even
+// frequencies in order, then the odd ones.
+__host__ __device__ constexpr int transfer_entries(int n) { return n <= 4096 ? n / 2 + 2 : n; }
 struct TableArgs {
     int n, count;
     double margin_px[kMaxLambda];     // taper margin in pixels (0 = no taper)
+    uint64_t h_fx[kMaxLambda];        // LambdaSet::h_fx
     float* sf;
+    float2* h;
 };
 cudaError_t launch_prop_tables(const TableArgs& a, cudaStream_t s);
 // conj = false: transfer function (FFT, H, IFFT per axis); true: one-FFT method.

@@ -6,6 +6,18 @@
 
 namespace scint {
 
+// v times H_x, from a half table h or evaluated here
+template <int N, int E>
+SCINT_DEV void apply_transfer(float2 (&v)[E], const float2* h, unsigned long long hc, int t) {
+    if (h) {
+#pragma unroll
+        for (int m = 0; m < E; ++m) v[m] = cmul(v[m], __ldg(h + half_index<N, E>(t, m)));
+    } else {
+#pragma unroll
+        for (int m = 0; m < E; ++m) v[m] = cmul(v[m], transfer_signed(hc, signed_index<N, E>(t, m)));
+    }
+}
+
 // ---- row pass ------------------------------------------------------------------
 // The pass bodies take the block index, the thread index and the block's shared memory
 // as arguments, so that the persistent batch kernel (persist.cu) runs the same code as
@@ -56,7 +68,7 @@ SCINT_DEV void prop_rows_body(const PropArgs& a, int bid, int tid, float2* smem3
         if constexpr (!CONJ) {
             const unsigned long long hc = a.lam.h_fx[l];
 #pragma unroll
-            for (int m = 0; m < E; ++m) v[m] = cmul(v[m], transfer_signed(hc, signed_index<N, E>(t, m)));
+            for (int m = 0; m < E; ++m) v[m] = cmul(v[m], transfer_fast(hc, signed_index<N, E>(t, m)));
             if constexpr (TWM == 2) fft_line_tr<float2, N, +1, 16, 1, 1, SUB>(v, buf, t, tr);
             else fft_line<float2, N, +1, 16, 1, TWM, 1, 1, SUB>(v, buf, t, twp);
         }
@@ -117,8 +129,7 @@ SCINT_DEV void prop_cols_body(const PropArgs& a, int bid, int tid, float2* smem3
             continue;
         } else {
             const unsigned long long hc = a.lam.h_fx[l];
-#pragma unroll
-            for (int m = 0; m < E; ++m) v[m] = cmul(v[m], transfer_signed(hc, signed_index<N, E>(t, m)));
+            apply_transfer<N, E>(v, N <= 4096 && a.h ? a.h + (size_t)l * transfer_entries(N) : nullptr, hc, t);
             if constexpr (TWM == 2) fft_line_tr<float2, N, +1, kColEPT, LW, 1, SUBC>(v, buf, t, tr);
             else fft_line<float2, N, +1, kColEPT, LW, TWM, 1, 1, SUBC>(v, buf, t, twp);
         }

@@ -27,15 +27,21 @@
 
 namespace scint {
 
-// ---- taper table --------------------------------------------------------------
+// ---- tables ---------------------------------------------------------------------
 // raised-sine taper SF at the pixel centre (i + 1/2), symmetric about the centre
-// (Sect. 3.2.1); H is not tabulated: the passes compute it from one fixed-point
-// constant per wavelength (transfer_at)
-__global__ void prop_tables_kernel(TableArgs a) {
+// (Sect. 3.2.1), and the transfer function
+__global__ void prop_tables_kernel(const __grid_constant__ TableArgs a) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int l = blockIdx.y;
-    if (i >= a.n) return;
-    const int n = a.n;
+    const int l = blockIdx.y, n = a.n, entries = transfer_entries(n);
+    if (a.h && i < entries) {
+        int m = i;    // the entry's frequency
+        if (n > 4096) {
+            if (n >= kSplitN) m = i < n / 2 ? 2 * i : 2 * (i - n / 2) + 1;
+            if (m >= n / 2) m -= n;
+        }
+        a.h[(size_t)l * entries + i] = transfer_signed(a.h_fx[l], m);
+    }
+    if (i >= n) return;
     const double lm = a.margin_px[l];
     double sf = 1.0;
     if (lm > 0.0) {
@@ -49,7 +55,7 @@ __global__ void prop_tables_kernel(TableArgs a) {
 }
 
 cudaError_t launch_prop_tables(const TableArgs& a, cudaStream_t s) {
-    dim3 grid((a.n + 255) / 256, a.count);
+    dim3 grid((std::max(a.n, a.h ? transfer_entries(a.n) : 0) + 255) / 256, a.count);
     prop_tables_kernel<<<grid, 256, 0, s>>>(a);
     return cudaGetLastError();
 }
@@ -82,11 +88,10 @@ prop_cols_kernel(PropArgs a) {
 // and by the load/store pipe of the exchanges; per-launch times before and after, ms:
 //                  32 wavelengths                          one wavelength
 //          rows           columns               rows             columns
-//   512    0.102 -> 0.082   0.085 -> 0.076      0.0118 -> 0.0106   0.0098 -> 0.0099
-//   1024   0.176 -> 0.152   0.160 -> 0.138      0.0171 -> 0.0147   0.0131 -> 0.0148
-//   2048   0.625 -> 0.569   0.573 -> 0.496      0.0458 -> 0.0314   0.0414 -> 0.0374
-//   4096   2.501 -> 2.352   2.562 -> 2.416      0.1657 -> 0.108    0.1637 -> 0.133
-//   8192 (8 wavelengths, rows)  3.70 -> 3.35    0.795  -> 0.525
+//   512    0.102 -> 0.079   0.085 -> 0.078      0.0118 -> 0.0106   0.0098 -> 0.0100
+//   1024   0.176 -> 0.152   0.160 -> 0.140      0.0171 -> 0.0145   0.0131 -> 0.0140
+//   2048   0.625 -> 0.571   0.573 -> 0.490      0.0458 -> 0.0307   0.0414 -> 0.0350
+//   4096   2.501 -> 2.371   2.562 -> 2.463      0.1657 -> 0.1075   0.1637 -> 0.1312
 // The one-FFT columns keep plain loads: with half the transforms per value the copies of 16-byte
 // rows became their bound (4096^2, 8 wavelengths: 0.493 ms, streamed 0.531).
 //   Row pass: the block's phases by one bulk copy into the array that keeps their fixed-point
@@ -186,7 +191,7 @@ prop_rows_stream_kernel(PropArgs a, int bulk) {
             if constexpr (!CONJ) {
                 const unsigned long long hc = a.lam.h_fx[l];
 #pragma unroll
-                for (int m = 0; m < E; ++m) v[m] = cmul(v[m], transfer_signed(hc, signed_index<N, E>(t, m)));
+                for (int m = 0; m < E; ++m) v[m] = cmul(v[m], transfer_fast(hc, signed_index<N, E>(t, m)));
                 fft_line_tr<float2, N, +1, 16, 1, 1, SUB>(v, buf, t, tr);
             }
             static_assert(T % W == 0, "whole strips between a thread's values");
@@ -220,7 +225,7 @@ SCINT_DEV void store_row(float* o, float (&r)[W], int wide, int accumulate) {
 }
 
 template <int N> constexpr size_t pcol_stream_smem() {
-    return col_stage_bytes<N>() + (size_t)pcol_lines<N>() * FftPlan<N>::BUF * sizeof(float2) + 16;
+    return col_stage_bytes<N>() + (size_t)(pcol_lines<N>() * FftPlan<N>::BUF + transfer_entries(N)) * sizeof(float2) + 24;
 }
 
 template <int N>
@@ -233,19 +238,27 @@ prop_cols_stream_kernel(PropArgs a, const __grid_constant__ CUtensorMap tm, int 
     float2* stage = smem32;
     float2* bufs = stage + N * W;
     float2* buf = bufs + w * Pl::BUF;
-    unsigned long long* bar = reinterpret_cast<unsigned long long*>(bufs + W * Pl::BUF);
-    unsigned* reads = reinterpret_cast<unsigned*>(bar + 1);    // teams that have read the stage
+    constexpr int HT = transfer_entries(N);
+    float2* hs = bufs + W * Pl::BUF;
+    unsigned long long* bar = reinterpret_cast<unsigned long long*>(hs + HT);    // stage, H
+    unsigned* reads = reinterpret_cast<unsigned*>(bar + 2);    // teams that have read the stage, H
     const int count = a.lam.count;
+    auto load_h = [&](int l) {
+        tile_expect(bar + 1, HT * sizeof(float2));
+        bulk_load(hs, a.h + (size_t)l * HT, HT * sizeof(float2), bar + 1);
+    };
     if (threadIdx.x == 0) {
         tile_init(bar);
-        *reads = 0u;
+        tile_init(bar + 1);
+        reads[0] = reads[1] = 0u;
         tile_init_fence();
         issue_columns<N>(stage, &tm, 0, blockIdx.x * W, bar);
+        load_h(0);
     }
     TwiddleRegs<float2, N, 16> tr;
     tr.load(a.tw, t);
     __syncthreads();
-    unsigned parity = 0;
+    unsigned parity = 0;    // bits: the stage's, H's
     bool ok = true;
 #pragma unroll 1
     for (int x0 = blockIdx.x * W; x0 < N; x0 += gridDim.x * W) {
@@ -254,7 +267,7 @@ prop_cols_stream_kernel(PropArgs a, const __grid_constant__ CUtensorMap tm, int 
         for (int m = 0; m < E; ++m) acc[m] = 0.0f;
 #pragma unroll 1
         for (int l = 0; l < count; ++l) {
-            ok = ok && wait_tile(bar, parity);
+            ok = ok && wait_tile(bar, parity & 1);
             parity ^= 1;
             float2 v[E];
             const float2* col = stage + (w / kBoxCols) * N * kBoxCols + w % kBoxCols;
@@ -271,10 +284,18 @@ prop_cols_stream_kernel(PropArgs a, const __grid_constant__ CUtensorMap tm, int 
                     if (nx < N) issue_columns<N>(stage, &tm, last ? 0 : l + 1, nx, bar);
                 }
             }
-            const unsigned long long hc = a.lam.h_fx[l];
+            const bool more = x0 + (int)gridDim.x * W < N;
+            if (count > 1 || x0 == (int)blockIdx.x * W) {
+                ok = ok && wait_tile(bar + 1, parity >> 1);
+                parity ^= 2;
+            }
 #pragma unroll
-            for (int m = 0; m < E; ++m) v[m] = cmul(v[m], transfer_signed(hc, signed_index<N, E>(t, m)));
+            for (int m = 0; m < E; ++m) v[m] = cmul(v[m], hs[half_index<N, E>(t, m)]);
             fft_line_tr<float2, N, +1, kColEPT, 1, 1, T>(v, buf, t, tr);
+            if (count > 1 && t == 0) {    // the same for H
+                __threadfence_block();
+                if (atomicAdd(reads + 1, 1u) % W == W - 1 && (l + 1 < count || more)) load_h(l + 1 < count ? l + 1 : 0);
+            }
             // 1/N of H_y, squared, on the weight (prop_cols_body); NaN if a copy is missing
             const float wl = ok ? a.lam.weight[l] * (1.0f / ((float)N * (float)N)) : __int_as_float(0x7FFFFFFF);
 #pragma unroll
@@ -296,12 +317,13 @@ prop_cols_stream_kernel(PropArgs a, const __grid_constant__ CUtensorMap tm, int 
         __syncthreads();
     }
     if (!ok) {
-        wait_tile(bar, 0);
-        wait_tile(bar, 1);
+        for (int k = 0; k < 4; ++k) wait_tile(bar + (k >> 1), k & 1);
     }
 }
 
 // ---- lines of 8192 points: two half lines per team (fft_long) ----------------------------
+// Per launch against 512 threads with sixteen values each: rows 3.70 -> 3.0 ms (8 wavelengths), 0.795 ->
+// 0.495 (one); columns 3.95 -> 2.9 and 1.09 -> 0.56.
 // Row pass: 256 threads per row, two rows per SM; the phases by bulk copy as above, the taper
 // from its table (no room beside two rows' phases).
 // Column pass: 256 threads and one column per block, two blocks per SM, so that one column's
@@ -311,6 +333,29 @@ prop_cols_stream_kernel(PropArgs a, const __grid_constant__ CUtensorMap tm, int 
 // of a 4-byte one per row and column.
 template <int N> __host__ __device__ constexpr bool long_lines() { return N == 8192; }
 template <int N> constexpr size_t prow_long_smem() { return (size_t)LongPlan<N>::BUF * sizeof(float2) + N * sizeof(long long) + 16; }
+
+// a and b times H at the frequencies 2k and 2k + 1, k = t + m T (TAB: from the table)
+template <int N, bool TAB>
+SCINT_DEV void long_transfer(float2 (&a)[16], float2 (&b)[16], const PropArgs& p, int l, int t) {
+    constexpr int T = LongPlan<N>::T;
+    if constexpr (TAB) {
+        const float4* h = reinterpret_cast<const float4*>(p.h + (size_t)l * N) + t;
+#pragma unroll
+        for (int m = 0; m < 16; ++m) {
+            const float4 q = __ldg(h + m * T);
+            a[m] = cmul(a[m], make_float2(q.x, q.y));
+            b[m] = cmul(b[m], make_float2(q.z, q.w));
+        }
+    } else {
+        const unsigned long long hc = p.lam.h_fx[l];
+#pragma unroll
+        for (int m = 0; m < 16; ++m) {
+            const int f = 2 * signed_index<N / 2, 16>(t, m);
+            a[m] = cmul(a[m], transfer_signed(hc, f));
+            b[m] = cmul(b[m], transfer_signed(hc, f + 1));
+        }
+    }
+}
 
 template <int N, bool CONJ>
 __global__ void __launch_bounds__(LongPlan<N>::T, 2) prop_rows_long_kernel(PropArgs a, int bulk) {
@@ -386,8 +431,8 @@ __global__ void __launch_bounds__(LongPlan<N>::T, 2) prop_rows_long_kernel(PropA
 #pragma unroll
                 for (int m = 0; m < H; ++m) {
                     const int f = 2 * signed_index<N / 2, H>(t, m);
-                    va[m] = cmul(va[m], transfer_signed(hc, f));
-                    vb[m] = cmul(vb[m], transfer_signed(hc, f + 1));
+                    va[m] = cmul(va[m], transfer_fast(hc, f));
+                    vb[m] = cmul(vb[m], transfer_fast(hc, f + 1));
                 }
                 fft_long<N, +1>(va, vb, buf, t, tr, w0);
 #pragma unroll
@@ -407,7 +452,7 @@ __global__ void __launch_bounds__(LongPlan<N>::T, 2) prop_rows_long_kernel(PropA
 constexpr int kLongCluster = 4;
 template <int N> constexpr size_t pcol_long_smem() { return (size_t)LongPlan<N>::BUF * sizeof(float2) + N * sizeof(float); }
 
-template <int N>
+template <int N, bool TAB>
 __global__ void __launch_bounds__(LongPlan<N>::T, 2) prop_cols_long_kernel(PropArgs a, int wide) {
     using Pl = LongPlan<N>;
     constexpr int T = Pl::T, H = Pl::H, WL = pstrip<N>(), C = kLongCluster;
@@ -432,13 +477,7 @@ __global__ void __launch_bounds__(LongPlan<N>::T, 2) prop_cols_long_kernel(PropA
             vb[m] = __ldcg(src + (size_t)(t + m * T + N / 2) * WL);
         }
         fft_long<N, -1>(va, vb, buf, t, tr, w0);
-        const unsigned long long hc = a.lam.h_fx[l];
-#pragma unroll
-        for (int m = 0; m < H; ++m) {
-            const int f = 2 * signed_index<N / 2, H>(t, m);
-            va[m] = cmul(va[m], transfer_signed(hc, f));
-            vb[m] = cmul(vb[m], transfer_signed(hc, f + 1));
-        }
+        long_transfer<N, TAB>(va, vb, a, l, t);
         fft_long<N, +1>(va, vb, buf, t, tr, w0);
         // 1/N of H_y, squared, on the weight (prop_cols_body)
         const float wl = a.lam.weight[l] * (1.0f / ((float)N * (float)N));
@@ -506,7 +545,7 @@ bool field_map(CUtensorMap* tm, const float2* work, int n, int count, int strip)
 // Block 1's quarter is the upper half of its half-problem, so it runs fft_long with the halves
 // swapped: W_{N/2}^n changes sign, and array a is always the part the block keeps.
 // Measured per 16384^2 pass at one wavelength, against 512 threads with sixteen values each, one
-// block per SM, whole lines read by both blocks: rows 3.97 -> 3.13 ms, columns 3.10 -> 2.63 ms (with the transpose).
+// block per SM, whole lines read by both blocks: rows 4.2 -> 3.1 ms, columns 3.1 -> 2.7 ms (with the transpose).
 template <int N> __host__ __device__ constexpr int psplit_threads() { return FftPlan<N / 2>::T; }
 template <int N> constexpr size_t conj_row_split_smem() {
     return (size_t)FftPlan<N / 2>::BUF * sizeof(float2) + (size_t)N * sizeof(long long);
@@ -575,10 +614,31 @@ SCINT_DEV void exchange_inverse(float2 (&a)[16], float2 (&b)[16], float2* buf, i
     cluster_arrive();
     quarter_join<N>(a, b, r, wq);
 }
-// signed frequency of fft_long's a[m] (b[m]: + 2) in block r
-template <int N> SCINT_DEV int split_index(int t, int m, int r) { return 4 * signed_index<N / 4, 16>(t, m) + r; }
+// a and b times H at the frequencies 2k + r of fft_long's k (a: k = 2 (t + m T), b: the next)
+// (TAB: from the table)
+template <int N, bool TAB>
+SCINT_DEV void split_transfer(float2 (&a)[16], float2 (&b)[16], const PropArgs& p, int l, int t, int r) {
+    constexpr int T = LongPlan<N / 2>::T;
+    if constexpr (TAB) {
+        const float4* h = reinterpret_cast<const float4*>(p.h + (size_t)l * N + r * (N / 2)) + t;
+#pragma unroll
+        for (int m = 0; m < 16; ++m) {
+            const float4 q = __ldg(h + m * T);
+            a[m] = cmul(a[m], make_float2(q.x, q.y));
+            b[m] = cmul(b[m], make_float2(q.z, q.w));
+        }
+    } else {
+        const unsigned long long hc = p.lam.h_fx[l];
+#pragma unroll
+        for (int m = 0; m < 16; ++m) {
+            const int f = 4 * signed_index<N / 4, 16>(t, m) + r;
+            a[m] = cmul(a[m], transfer_signed(hc, f));
+            b[m] = cmul(b[m], transfer_signed(hc, f + 2));
+        }
+    }
+}
 
-template <int N>
+template <int N, bool TAB>
 __global__ void __launch_bounds__(lsplit_threads<N>(), 2) prop_rows_split_kernel(PropArgs a, int bulk) {
     constexpr int H2 = N / 2, M = N / 4;
     using Pl = LongPlan<H2>;
@@ -638,13 +698,7 @@ __global__ void __launch_bounds__(lsplit_threads<N>(), 2) prop_rows_split_kernel
             if (bulk && t == 0 && l + 1 == a.lam.count && y + (int)gridDim.x / 2 < N) load_phi(y + gridDim.x / 2);
             cluster_wait();
             fft_long<H2, -1>(va, vb, buf, t, tr, w0);
-            const unsigned long long hc = a.lam.h_fx[l];
-#pragma unroll
-            for (int m = 0; m < 16; ++m) {
-                const int f = split_index<N>(t, m, r);
-                va[m] = cmul(va[m], transfer_signed(hc, f));
-                vb[m] = cmul(vb[m], transfer_signed(hc, f + 2));
-            }
+            split_transfer<N, TAB>(va, vb, a, l, t, r);
             fft_long<H2, +1>(va, vb, buf, t, tr, w0);
             exchange_inverse<N>(va, vb, buf, t, r, wq);
             float2* dst = a.work + (size_t)l * N * N + strip_index<W>(y, n0, N);
@@ -662,7 +716,7 @@ __global__ void __launch_bounds__(lsplit_threads<N>(), 2) prop_rows_split_kernel
     }
 }
 
-template <int N>
+template <int N, bool TAB>
 __global__ void __launch_bounds__(lsplit_threads<N>(), 2) prop_cols_split_kernel(PropArgs a) {
     constexpr int H2 = N / 2, M = N / 4;
     using Pl = LongPlan<H2>;
@@ -691,13 +745,7 @@ __global__ void __launch_bounds__(lsplit_threads<N>(), 2) prop_cols_split_kernel
             exchange_forward<N>(va, vb, buf, t, r, wq);
             cluster_wait();
             fft_long<H2, -1>(va, vb, buf, t, tr, w0);
-            const unsigned long long hc = a.lam.h_fx[l];
-#pragma unroll
-            for (int m = 0; m < 16; ++m) {
-                const int f = split_index<N>(t, m, r);
-                va[m] = cmul(va[m], transfer_signed(hc, f));
-                vb[m] = cmul(vb[m], transfer_signed(hc, f + 2));
-            }
+            split_transfer<N, TAB>(va, vb, a, l, t, r);
             fft_long<H2, +1>(va, vb, buf, t, tr, w0);
             exchange_inverse<N>(va, vb, buf, t, r, wq);
             // 1/N of H_y, squared, on the weight (prop_cols_body); the last sum goes out column-major, so that
@@ -852,7 +900,7 @@ cudaError_t launch_rows(const PropArgs& a, cudaStream_t s) {
             return launch_k(k, 2, dim3(2 * std::min(nc, N)), dim3(psplit_threads<N>()), conj_row_split_smem<N>(), s, a);
         } else if constexpr (pcs<N>() == 2) {
             static_assert(2 * (prow_split_smem<N>() + 1024) <= 228 * 1024, "two blocks per SM");
-            auto k = prop_rows_split_kernel<N>;
+            auto k = a.h ? prop_rows_split_kernel<N, true> : prop_rows_split_kernel<N, false>;
             cudaError_t e = set_smem(k, prow_split_smem<N>());
             int nc = 0;
             if (e == cudaSuccess) e = active_clusters(k, 2, lsplit_threads<N>(), prow_split_smem<N>(), &nc);
@@ -902,7 +950,7 @@ cudaError_t launch_cols(const PropArgs& a, cudaStream_t s) {
             constexpr size_t smem = CONJ ? conj_col_split_smem<N>() : pcol_split_smem<N>();
             constexpr int threads = CONJ ? psplit_threads<N>() : lsplit_threads<N>();
             static_assert(smem <= kMaxSmem, "split column pass does not fit");
-            auto k = CONJ ? conj_cols_split_kernel<N> : prop_cols_split_kernel<N>;
+            auto k = CONJ ? conj_cols_split_kernel<N> : (a.h ? prop_cols_split_kernel<N, true> : prop_cols_split_kernel<N, false>);
             cudaError_t e = set_smem(k, smem);
             int nc = 0;
             if (e == cudaSuccess) e = active_clusters(k, 2, threads, smem, &nc);
@@ -916,7 +964,7 @@ cudaError_t launch_cols(const PropArgs& a, cudaStream_t s) {
         } else {
             if constexpr (!CONJ && long_lines<N>()) {
                 static_assert(2 * (pcol_long_smem<N>() + 1024) <= 228 * 1024, "two columns per SM");
-                auto k = prop_cols_long_kernel<N>;
+                auto k = a.h ? prop_cols_long_kernel<N, true> : prop_cols_long_kernel<N, false>;
                 const cudaError_t e = set_smem(k, pcol_long_smem<N>());
                 if (e != cudaSuccess) return e;
                 return launch_k(k, kLongCluster, dim3(N), dim3(LongPlan<N>::T), pcol_long_smem<N>(), s, a,
@@ -925,7 +973,7 @@ cudaError_t launch_cols(const PropArgs& a, cudaStream_t s) {
             if constexpr (!CONJ && col_stream<N>()) {
                 static_assert(pcol_stream_smem<N>() <= kMaxSmem, "streamed column pass does not fit");
                 CUtensorMap tm;
-                if (field_map(&tm, a.work, N, a.lam.count, pstrip<N>())) {
+                if (a.h && field_map(&tm, a.work, N, a.lam.count, pstrip<N>())) {
                     auto k = prop_cols_stream_kernel<N>;
                     cudaError_t e = set_smem(k, pcol_stream_smem<N>());
                     int blocks = 0;

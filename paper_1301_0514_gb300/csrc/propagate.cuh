@@ -121,18 +121,39 @@ SCINT_DEV float2 transfer_phasor(unsigned long long C, int i, int n) {
     const long long m = sfreq(i, n);
     return unit_phasor(0, 0ull, C * (unsigned long long)(m * m));
 }
-// The same for the signed index m itself, |m| < 2^15: the upper 32 bits of C m^2 mod 2^64 are all
-// that the angle takes, so 32-bit products do (the same bits).
-SCINT_DEV float2 transfer_signed(unsigned long long C, int m) {
+// The same for the signed index m, |m| < 2^15: the upper 32 bits of C m^2 mod 2^64 are all that the
+// angle takes, so 32-bit products do (the same bits).  The row passes up to 8192 evaluate H_x so: their
+// load/store pipe is the busier one, and a table in shared memory had cost 2-4 % of them with 32
+// wavelengths (8192, from global memory: 12 %).
+SCINT_DEV float2 transfer_fast(unsigned long long C, int m) {
     const unsigned mm = (unsigned)(m * m);
     const unsigned hi = __umulhi((unsigned)C, mm) + (unsigned)(C >> 32) * mm;
     float sn, cs;
     __sincosf((float)(int)hi * (float)(2.0 * kPi * 0x1.0p-32), &sn, &cs);
     return make_float2(cs, sn);
 }
+// The same to FP32 accuracy, for the column passes' tables and the 16384-point lines (TableArgs; ~25
+// instructions where there is no table): the turns are reduced to an eighth of a turn around a quarter turn
+// before the sine and cosine.  The hardware sine's absolute error of 4e-7, once for the screen
+// and once for each axis, is the larger part of the passes' error; without it on one axis the
+// intensities' error against 64 bits is below what it was with twiddles from the exact table in the
+// columns and one factorisation less in the long lines (one wavelength at 4096^2: 8.9e-7 -> 8.2e-7, 48 screens 8.0e-7 -> 7.1e-7).
+SCINT_DEV float2 transfer_signed(unsigned long long C, int m) {
+    const unsigned mm = (unsigned)(m * m);
+    const int turns = (int)(__umulhi((unsigned)C, mm) + (unsigned)(C >> 32) * mm);
+    const unsigned q = ((unsigned)turns + 0x20000000u) >> 30;
+    float sn, cs;
+    sincospif((float)(int)((unsigned)turns - (q << 30)) * 0x1.0p-31f, &sn, &cs);
+    const float re = q & 1u ? sn : cs, im = q & 1u ? cs : sn;    // times i^q
+    return make_float2(q == 1u || q == 2u ? -re : re, q >= 2u ? -im : im);
+}
 // signed frequency index of element t + m T of a line of N = E T values, t < T
 template <int N, int E> SCINT_DEV int signed_index(int t, int m) {
     return t + m * (N / E) - (2 * m >= E ? N : 0);
+}
+// its entry in a half table, |signed_index|
+template <int N, int E> SCINT_DEV int half_index(int t, int m) {
+    return 2 * m >= E ? N - (t + m * (N / E)) : t + m * (N / E);
 }
 // H_x(k)/n (the inverse transform's normalisation)
 SCINT_DEV float2 transfer_at(unsigned long long C, int i, int n) { return transfer_phasor(C, i, n) * (1.0f / n); }

@@ -65,3 +65,45 @@ def test_long_lines_match_the_one_wavelength_form(count):
     p = S.params(n=n, pixel_km=10.0, r_diff_km=60.0, lambda_nm=550.0, margin_km=0.0, seed=5)
     one = S.sum_passband(p, torch.zeros((n, n), dtype=torch.float64, device="cuda"), _band(count))
     assert (one - 1.0).abs().max().item() <= 2e-5
+
+
+def _least_bytes(n, g=1):
+    """The twiddles, the tapers and the fields of a group (and the column-major sums at 16384): what a
+    propagation accepts without its transfer-function tables."""
+    up = lambda b: (b + 255) // 256 * 256  # noqa: E731
+    slots = g if g == 1 else (g + 1) // 2 * 2
+    return up(n * 8) + up(g * n * 4) + up(slots * n * n * 8) + (up(n * n * 4) if n >= 16384 else 0)
+
+
+@pytest.mark.parametrize("n", [64, 512, 1024, 4096, 8192, 16384])
+def test_least_workspace_and_capture_without_tables(n):
+    """The same bits when the transfer function's tables have room in the workspace, only in the
+    twiddles' slot (one wavelength, twiddles kept), or nowhere (a capture before any call): one
+    expression gives the values in all three."""
+    p = S.params(n=n, pixel_km=10.0, r_diff_km=60.0, lambda_nm=550.0, seed=5)
+    phi = S.make_screen(p)
+    want = S.propagate(p, phi)
+    small = torch.empty(_least_bytes(n), dtype=torch.uint8, device="cuda")
+    assert torch.equal(S.propagate(p, phi, workspace=small), want)
+    with pytest.raises(S.ScintError):
+        S.propagate(p, phi, workspace=small[:-256])
+    torch.cuda.synchronize()
+    S.release()
+    out = torch.zeros((n, n), dtype=torch.float32, device="cuda")
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        S.propagate(p, phi, out=out, workspace=small)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, want)
+
+
+@pytest.mark.parametrize("n", [256, 2048])
+def test_least_group_workspace(n):
+    """A group's least workspace still runs the passband (in smaller groups)."""
+    p = S.params(n=n, pixel_km=10.0, r_diff_km=60.0, lambda_nm=550.0, seed=5)
+    phi, lam = S.make_screen(p), _band(5)
+    ws = torch.empty(_least_bytes(n, 4), dtype=torch.uint8, device="cuda")
+    want = S.sum_passband(p, phi, lam)
+    got = S.sum_passband(p, phi, lam, workspace=ws)
+    assert (got - want).abs().max().item() <= 5 * 2.0 ** -23 * want.max().item()
