@@ -1019,28 +1019,58 @@ SCINT_DEV Sample sample_at(int X, int n, long long r_fx) {
 // all wavelengths.  Lanes take consecutive output rows of one column, so the
 // four bilinear taps of a warp read consecutive elements of two pattern columns
 // (patterns are column-major); the tile goes out through shared memory as rows.
-constexpr int kResTile = 32;
-__global__ void __launch_bounds__(256) resample_tiled_kernel(ResampleArgs a) {
+// The taps' places of the tile's 32 columns and 32 rows are worked out once per kResLambda wavelengths,
+// by one thread each, and read from shared memory (in place, per pixel and wavelength, their
+// 64-bit products were half of the 49 instructions: 4096^2, 8 wavelengths 0.292 -> 0.193 ms).
+constexpr int kResTile = 32, kResLambda = 16;
+struct Tap {
+    int i0;      // wrapped
+    float f;
+};
+SCINT_DEV Tap tap_at(int X, int n, long long r_fx) {
+    const Sample s = sample_at(X, n, r_fx);
+    return Tap{s.i0 & (n - 1), s.f};
+}
+__global__ void __launch_bounds__(256) resample_tiled_kernel(const __grid_constant__ ResampleArgs a) {
     __shared__ float tile[kResTile][kResTile + 1];   // [x][y]
+    __shared__ Tap tx[kResLambda][kResTile], ty[kResLambda][kResTile];
     const int n = a.n;
     const int X0 = blockIdx.x * kResTile, Y0 = blockIdx.y * kResTile;
     const int ly = threadIdx.x % kResTile, lx = threadIdx.x / kResTile;   // lx in [0, 8)
     float acc[kResTile / 8] = {};
-    for (int l = 0; l < a.count; ++l) {
-        const long long r = a.r_fx[l];
-        const float* h = a.pattern + (size_t)l * n * n;
-        const Sample sy = sample_at(Y0 + ly, n, r);
-        const int y0 = sy.i0 & (n - 1), y1 = (y0 + 1) & (n - 1);
-        const float wl = a.weight[l];
+    for (int l0 = 0; l0 < a.count; l0 += kResLambda) {
+        const int g = min(kResLambda, a.count - l0);
+        __syncthreads();
+        for (int i = threadIdx.x; i < 2 * kResTile * g; i += 256) {
+            const int l = i / (2 * kResTile), k = i % kResTile;
+            const long long r = a.r_fx[l0 + l];
+            if (i % (2 * kResTile) < kResTile) tx[l][k] = tap_at(X0 + k, n, r);
+            else ty[l][k] = tap_at(Y0 + k, n, r);
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int l = 0; l < g; ++l) {
+            const float* h = a.pattern + (size_t)(l0 + l) * n * n;
+            const Tap sy = ty[l][ly];
+            const int y0 = sy.i0, y1 = (y0 + 1) & (n - 1);
+            const float wl = a.weight[l0 + l];
+            float h00[kResTile / 8], h01[kResTile / 8], h10[kResTile / 8], h11[kResTile / 8], fx[kResTile / 8];
 #pragma unroll
-        for (int q = 0; q < kResTile / 8; ++q) {
-            const Sample sx = sample_at(X0 + lx + 8 * q, n, r);
-            const int x0 = sx.i0 & (n - 1), x1 = (x0 + 1) & (n - 1);
-            const float* c0 = h + (size_t)x0 * n;
-            const float* c1 = h + (size_t)x1 * n;
-            const float h00 = __ldg(c0 + y0), h01 = __ldg(c0 + y1), h10 = __ldg(c1 + y0), h11 = __ldg(c1 + y1);
-            const float left = fmaf(sy.f, h01 - h00, h00), right = fmaf(sy.f, h11 - h10, h10);
-            acc[q] = fmaf(wl, fmaf(sx.f, right - left, left), acc[q]);
+            for (int q = 0; q < kResTile / 8; ++q) {
+                const Tap sx = tx[l][lx + 8 * q];
+                const float* c0 = h + (size_t)sx.i0 * n;
+                const float* c1 = h + (size_t)((sx.i0 + 1) & (n - 1)) * n;
+                fx[q] = sx.f;
+                h00[q] = __ldg(c0 + y0);
+                h01[q] = __ldg(c0 + y1);
+                h10[q] = __ldg(c1 + y0);
+                h11[q] = __ldg(c1 + y1);
+            }
+#pragma unroll
+            for (int q = 0; q < kResTile / 8; ++q) {
+                const float left = fmaf(sy.f, h01[q] - h00[q], h00[q]), right = fmaf(sy.f, h11[q] - h10[q], h10[q]);
+                acc[q] = fmaf(wl, fmaf(fx[q], right - left, left), acc[q]);
+            }
         }
     }
 #pragma unroll
