@@ -1,6 +1,7 @@
 // Light curves (Sect. 3.3) and the modulation index m = sigma_I / mean(I) (Sect. 4).
 #include <cmath>
 
+#include "dispatch.cuh"
 #include "kernels.cuh"
 #include "track.cuh"
 
@@ -22,6 +23,7 @@ Track make_track(int n, const double* t) {
 // operations per sample and 64 tracks per launch, 30 us in 2 now).
 template <int K>
 __global__ void __launch_bounds__(256) lightcurve_kernel(const __grid_constant__ CurveArgs<K> a) {
+    begin_after_previous();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     const int c = blockIdx.y;
     if (s >= a.n_samples || c >= a.n_tracks) return;
@@ -42,8 +44,7 @@ template <int K>
 cudaError_t launch_lightcurve(const CurveArgs<K>& a, cudaStream_t s) {
     if (a.n_tracks <= 0 || a.n_samples <= 0) return cudaSuccess;
     dim3 grid((a.n_samples + 255) / 256, a.n_tracks);
-    lightcurve_kernel<K><<<grid, 256, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_next(lightcurve_kernel<K>, grid, dim3(256), 0, s, a);
 }
 template cudaError_t launch_lightcurve<kTracksPerLaunch>(const CurveArgs<kTracksPerLaunch>&, cudaStream_t);
 template cudaError_t launch_lightcurve<kManyTracks>(const CurveArgs<kManyTracks>&, cudaStream_t);

@@ -31,6 +31,7 @@ namespace scint {
 // raised-sine taper SF at the pixel centre (i + 1/2), symmetric about the centre
 // (Sect. 3.2.1), and the transfer function
 __global__ void prop_tables_kernel(const __grid_constant__ TableArgs a) {
+    begin_after_previous();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int l = blockIdx.y, n = a.n, entries = transfer_entries(n);
     if (a.h && i < entries) {
@@ -56,8 +57,7 @@ __global__ void prop_tables_kernel(const __grid_constant__ TableArgs a) {
 
 cudaError_t launch_prop_tables(const TableArgs& a, cudaStream_t s) {
     dim3 grid((std::max(a.n, a.h ? transfer_entries(a.n) : 0) + 255) / 256, a.count);
-    prop_tables_kernel<<<grid, 256, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_next(prop_tables_kernel, grid, dim3(256), 0, s, a);
 }
 
 // Resident row blocks per SM the register budget is set for (build-time choice, 2 by default;
@@ -69,6 +69,7 @@ template <int N, bool CONJ>
 __global__ void __launch_bounds__(prow_threads<N>(), (prow_threads<N>() <= 256 ? SCINT_ROW_MIN_BLOCKS : 1))
 prop_rows_kernel(PropArgs a) {
     extern __shared__ float2 smem32[];
+    begin_pass<N>();
     prop_rows_body<N, CONJ>(a, blockIdx.x, threadIdx.x, smem32);
 }
 
@@ -76,6 +77,7 @@ template <int N, bool CONJ>
 __global__ void __launch_bounds__(pcol_threads<N>(), (pcol_threads<N>() <= 256 ? 2 : 1))
 prop_cols_kernel(PropArgs a) {
     extern __shared__ float2 smem32[];
+    begin_pass<N>();
     prop_cols_body<N, CONJ>(a, blockIdx.x, threadIdx.x, smem32);
 }
 
@@ -115,6 +117,7 @@ prop_rows_stream_kernel(PropArgs a, int bulk) {
     constexpr int T = Pl::T, E = Pl::E, B = prow_lines<N>(), W = pstrip<N>(), BUFL = Pl::BUF;
     static_assert(prow_twm<N>() == 2, "register twiddle bases");
     extern __shared__ float2 smem32[];
+    begin_pass<N>();
     const int team = threadIdx.x / T, t = threadIdx.x % T;
     float2* buf = smem32 + team * BUFL;
     long long* Pall = reinterpret_cast<long long*>(smem32 + B * BUFL);
@@ -234,6 +237,7 @@ prop_cols_stream_kernel(PropArgs a, const __grid_constant__ CUtensorMap tm, int 
     using Pl = FftPlan<N, kColEPT>;
     constexpr int T = Pl::T, E = Pl::E, W = pcol_lines<N>();
     extern __shared__ float2 smem32[];
+    begin_pass<N>();
     const int w = threadIdx.x / T, t = threadIdx.x % T;    // a team per column
     float2* stage = smem32;
     float2* bufs = stage + N * W;
@@ -929,13 +933,13 @@ cudaError_t launch_rows(const PropArgs& a, cudaStream_t s) {
                     e = walk_blocks(k, prow_threads<N>(), prow_stream_smem<N>(), N / prow_lines<N>(), a.lam.count, &blocks);
                 if (e != cudaSuccess) return e;
                 // a bulk copy starts on a 16-byte boundary: phases elsewhere are read by plain loads
-                k<<<blocks, prow_threads<N>(), prow_stream_smem<N>(), s>>>(a, reinterpret_cast<uintptr_t>(a.phi) % 16 == 0);
-                return cudaGetLastError();
+                return launch_pass<N>(a.lam.count, k, dim3(blocks), dim3(prow_threads<N>()), prow_stream_smem<N>(), s, a,
+                                      (int)(reinterpret_cast<uintptr_t>(a.phi) % 16 == 0));
             }
             cudaError_t e = set_smem(prop_rows_kernel<N, CONJ>, prow_smem<N>());
             if (e != cudaSuccess) return e;
-            prop_rows_kernel<N, CONJ><<<N / prow_lines<N>(), prow_threads<N>(), prow_smem<N>(), s>>>(a);
-            return cudaGetLastError();
+            return launch_pass<N>(a.lam.count, prop_rows_kernel<N, CONJ>, dim3(N / prow_lines<N>()), dim3(prow_threads<N>()),
+                                  prow_smem<N>(), s, a);
         }
     });
 }
@@ -981,16 +985,15 @@ cudaError_t launch_cols(const PropArgs& a, cudaStream_t s) {
                         e = walk_blocks(k, pcol_threads<N>(), pcol_stream_smem<N>(), N / pcol_lines<N>(), a.lam.count, &blocks);
                     if (e != cudaSuccess) return e;
                     constexpr int align = pcol_lines<N>() == 2 ? 8 : 16;
-                    k<<<blocks, pcol_threads<N>(), pcol_stream_smem<N>(), s>>>(
-                        a, tm, reinterpret_cast<uintptr_t>(a.intensity) % align == 0);
-                    return cudaGetLastError();
+                    return launch_pass<N>(a.lam.count, k, dim3(blocks), dim3(pcol_threads<N>()), pcol_stream_smem<N>(), s, a, tm,
+                                          (int)(reinterpret_cast<uintptr_t>(a.intensity) % align == 0));
                 }
             }
             constexpr size_t smem = pcol_smem<N, CONJ>();
             cudaError_t e = set_smem(prop_cols_kernel<N, CONJ>, smem);
             if (e != cudaSuccess) return e;
-            prop_cols_kernel<N, CONJ><<<N / pcol_lines<N>(), pcol_threads<N>(), smem, s>>>(a);
-            return cudaGetLastError();
+            return launch_pass<N>(a.lam.count, prop_cols_kernel<N, CONJ>, dim3(N / pcol_lines<N>()), dim3(pcol_threads<N>()), smem,
+                                  s, a);
         }
     });
 }

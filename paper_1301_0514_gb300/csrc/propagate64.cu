@@ -44,6 +44,7 @@ SCINT_DEV double2 transfer64(const Prop64Args& a, int i) {
 // sinpi too.  With the tables, twiddles kept between calls and four values per thread at 256^2 both
 // passes took 83 -> 37 us there (FP64 pipe 33 -> 63 % busy), 168 -> 101 us at 512^2, 587 -> 346 us at 1024^2.
 __global__ void prop64_tables_kernel(Prop64Args a, double2* h, double* sf) {
+    begin_after_previous();
     const int i = blockIdx.x * blockDim.x + threadIdx.x, half = a.n / 2;
     if (i <= half) h[i] = transfer64(a, i);
     if (i < half) sf[i] = taper64(i, a.n, a.margin_px);
@@ -69,6 +70,7 @@ template <int N> __host__ __device__ constexpr int p64_ept() {
 
 template <int N, bool TAB>
 __global__ void __launch_bounds__(FftPlan<N, p64_ept<N>()>::T) prop64_rows_kernel(Prop64Args a) {
+    begin_pass<N>();
     constexpr int EPT = p64_ept<N>();
     using Pl = FftPlan<N, EPT>;
     constexpr int T = Pl::T, E = Pl::E;
@@ -94,6 +96,7 @@ __global__ void __launch_bounds__(FftPlan<N, p64_ept<N>()>::T) prop64_rows_kerne
 
 template <int N, bool TAB>
 __global__ void __launch_bounds__(FftPlan<N, p64_ept<N>()>::T) prop64_cols_kernel(Prop64Args a) {
+    begin_pass<N>();
     constexpr int EPT = p64_ept<N>();
     using Pl = FftPlan<N, EPT>;
     constexpr int T = Pl::T, E = Pl::E;
@@ -116,10 +119,8 @@ cudaError_t launch_passes64(const Prop64Args& a, cudaStream_t s) {
     if (e == cudaSuccess) e = set_smem(prop64_cols_kernel<N, TAB>, p64_smem<N>());
     if (e != cudaSuccess) return e;
     constexpr int T = FftPlan<N, p64_ept<N>()>::T;
-    prop64_rows_kernel<N, TAB><<<N, T, p64_smem<N>(), s>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    prop64_cols_kernel<N, TAB><<<N, T, p64_smem<N>(), s>>>(a);
-    return cudaGetLastError();
+    if ((e = launch_pass<N>(1, prop64_rows_kernel<N, TAB>, dim3(N), dim3(T), p64_smem<N>(), s, a)) != cudaSuccess) return e;
+    return launch_pass<N>(1, prop64_cols_kernel<N, TAB>, dim3(N), dim3(T), p64_smem<N>(), s, a);
 }
 
 cudaError_t launch_prop64(const Prop64Args& args, void* tables, cudaStream_t s) {
@@ -133,8 +134,7 @@ cudaError_t launch_prop64(const Prop64Args& args, void* tables, cudaStream_t s) 
             double2* h = static_cast<double2*>(tables);
             double* sf = reinterpret_cast<double*>(h + N / 2 + 1);
             static_assert((N / 2 + 1) * sizeof(double2) + N / 2 * sizeof(double) <= N * sizeof(double2), "tables fit");
-            prop64_tables_kernel<<<(N / 2 + 32) / 32, 32, 0, s>>>(a, h, sf);
-            const cudaError_t e = cudaGetLastError();
+            const cudaError_t e = launch_next(prop64_tables_kernel, dim3((N / 2 + 32) / 32), dim3(32), 0, s, a, h, sf);
             if (e != cudaSuccess) return e;
             a.h = h;
             a.sf = sf;

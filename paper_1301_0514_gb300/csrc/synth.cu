@@ -157,6 +157,7 @@ SCINT_DEV void synth_row32(const SynthArgs& a, int ky, bool live, int t, float2*
 constexpr int kDrawThreads = 32;
 __host__ __device__ constexpr int draw_bins(int n) { return (n / 2 + 1) * (n / 2 + 1); }
 __global__ void __launch_bounds__(kDrawThreads) synth_draw_kernel(SynthArgs a) {
+    begin_after_previous();
     const int n = a.n, half_n = n / 2;
     const int i = blockIdx.x * kDrawThreads + threadIdx.x;
     if (i >= draw_bins(n)) return;
@@ -181,6 +182,7 @@ __global__ void __launch_bounds__(kDrawThreads) synth_draw_kernel(SynthArgs a) {
 template <int N>
 __global__ void __launch_bounds__(synth_threads<N>())
 synth_rows_kernel(SynthArgs a) {
+    begin_pass<N>();
     using Pl = SynthPlan<N>;
     static_assert(synth_cs<N>() == 1, "unsplit rows");
     constexpr int T = Pl::T, E = Pl::E, B = synth_lines<N>();
@@ -220,6 +222,7 @@ synth_rows_kernel(SynthArgs a) {
 template <int N>
 __global__ void __launch_bounds__(synth_col_threads<N>())
 synth_cols_kernel(SynthArgs a) {
+    begin_pass<N>();
     using Pl = SynthPlan<N>;
     static_assert(synth_cs<N>() == 1, "unsplit columns");
     constexpr int T = Pl::T, E = Pl::E, W = synth_col_lines<N>();
@@ -365,16 +368,17 @@ cudaError_t launch_synth_pass(const SynthArgs& a, cudaStream_t s) {
                 if ((e = set_smem(synth_rows_kernel<N>, synth_smem<N>())) != cudaSuccess) return e;
                 if constexpr (N <= kDrawN) {
                     if (!a.drawn) return cudaErrorInvalidValue;
-                    synth_draw_kernel<<<(draw_bins(N) + kDrawThreads - 1) / kDrawThreads, kDrawThreads, 0, s>>>(a);
-                    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+                    e = launch_next(synth_draw_kernel, dim3((draw_bins(N) + kDrawThreads - 1) / kDrawThreads),
+                                    dim3(kDrawThreads), 0, s, a);
+                    if (e != cudaSuccess) return e;
                 }
                 const int rows = N / 2 + 1;
-                return launch_k(synth_rows_kernel<N>, CS, dim3((rows + synth_lines<N>() - 1) / synth_lines<N>() * CS),
-                                dim3(synth_threads<N>()), synth_smem<N>(), s, a);
+                return launch_pass<N>(1, synth_rows_kernel<N>, dim3((rows + synth_lines<N>() - 1) / synth_lines<N>()),
+                                   dim3(synth_threads<N>()), synth_smem<N>(), s, a);
             } else {
                 if ((e = set_smem(synth_cols_kernel<N>, synth_col_smem<N>())) != cudaSuccess) return e;
-                return launch_k(synth_cols_kernel<N>, CS, dim3(N / (2 * synth_col_lines<N>()) * CS),
-                                dim3(synth_col_threads<N>()), synth_col_smem<N>(), s, a);
+                return launch_pass<N>(1, synth_cols_kernel<N>, dim3(N / (2 * synth_col_lines<N>())),
+                                   dim3(synth_col_threads<N>()), synth_col_smem<N>(), s, a);
             }
         }
     });

@@ -107,3 +107,40 @@ def test_least_group_workspace(n):
     want = S.sum_passband(p, phi, lam)
     got = S.sum_passband(p, phi, lam, workspace=ws)
     assert (got - want).abs().max().item() <= 5 * 2.0 ** -23 * want.max().item()
+
+
+@pytest.mark.parametrize("n", [64, 256, 512, 1024, 2048])
+def test_overlapped_launches_keep_their_order(n):
+    """Kernels set up while the one before ends (grids on both sides of the line) read nothing early:
+    chains of screen, propagation and curves through the same buffers, back to back, replayed as a graph
+    and with another library's kernels between them, give the bits of one call at a time."""
+    ps = [S.params(n=n, pixel_km=10.0, r_diff_km=60.0, lambda_nm=550.0, seed=7, screen_id=i) for i in range(4)]
+    tr = np.array([[3.0, 5.0, 0.3, 0.7], [n / 3.0, 1.0, 1.1, 0.5]])
+    ws = torch.empty(S.workspace_bytes(ps[0], 1), dtype=torch.uint8, device="cuda")
+    phi, out = torch.empty((n, n), dtype=torch.float64, device="cuda"), torch.empty((n, n), device="cuda")
+    curves = torch.empty((2, 100), device="cuda")
+
+    def chain(p):
+        S.make_screen(p, out=phi, workspace=ws)
+        S.propagate(p, phi, out=out, workspace=ws)
+        S.lightcurve(p, out, tr, 100, out=curves)
+        return out, curves
+
+    want = []
+    for p in ps:
+        want.append([t.clone() for t in chain(p)])
+        torch.cuda.synchronize()
+    for _ in range(8):
+        got = [[t.clone() for t in chain(p)] for p in ps]
+        assert all(torch.equal(a, b) for g, w in zip(got, want) for a, b in zip(g, w))
+    for p in ps:        # no other kernel between the chains
+        chain(p)
+    assert torch.equal(out, want[-1][0]) and torch.equal(curves, want[-1][1])
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        for p in ps:
+            chain(p)
+    for _ in range(4):
+        out.zero_(), curves.zero_(), phi.zero_()
+        g.replay()
+        assert torch.equal(out, want[-1][0]) and torch.equal(curves, want[-1][1])
