@@ -61,6 +61,14 @@ int scint_phase_fixed(const double* phi, int64_t* P, int64_t n, void* stream);
  */
 void scint_testing_persist(int withhold, int wait_limit);
 
+/*
+ * The parts of the persistent batch kernel's 512-thread block that synchronise through named barriers
+ * in one work item of an n x n screen (pass 0 rows, 1 columns): parts[] takes their sizes in threads, in
+ * order of use (host, room for 2).  Part i of s threads is threads [i s, (i + 1) s) and uses barrier
+ * 1 + i; no block barrier stands between the uses.  Returns the number of sizes (0 where there are none).
+ */
+int scint_testing_persist_parts(int n, int pass, int* parts);
+
 #ifdef __cplusplus
 }
 #endif

@@ -157,6 +157,7 @@ def lib() -> ctypes.CDLL:
         "scint_batch_mode": ([_i], _i),
         "scint_batch_status": ([_vp], _i),
         "scint_testing_persist": ([_i, _i], None),
+        "scint_testing_persist_parts": ([_i, _i, ctypes.POINTER(_i)], _i),
         "scint_tune_batch": ([ctypes.POINTER(BatchItem), _i, _vp, _vp, _i, _vp, _sz, ctypes.POINTER(_i),
                               ctypes.POINTER(ctypes.c_double), ctypes.POINTER(_i), _vp], _i),
         "scint_profile_enable": ([_i], _i),

@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "api_internal.h"
+#include "persist.cuh"
 
 namespace {
 
@@ -354,6 +355,7 @@ int scint_batch_status(void* stream) {
     return scint::clear_error();
 }
 
+int scint_testing_persist_parts(int n, int pass, int* parts) { return scint::persist_barrier_parts(n, pass, parts); }
 void scint_testing_persist(int withhold, int wait_limit) { scint::persist_testing(withhold, wait_limit); }
 
 size_t scint_batch_workspace_bytes(const scint_batch_item* items, int n_items, int n_lambda, int n_lanes) {

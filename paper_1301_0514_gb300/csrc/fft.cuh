@@ -397,6 +397,8 @@ SCINT_DEV void twiddle_powers(const C (&base)[4], C (&w)[R]) {
 // the SUB-thread part of the block that thread threadIdx.x belongs to, through the named
 // barrier 1 + threadIdx.x / SUB (SUB a multiple of 32 dividing the block; barrier 0 stays
 // the block's own; a warp of its own needs none) -- so that two independent teams can share one block.
+// Parts of two sizes share barrier ids (1 + threadIdx.x / SUB in both): between their uses in one block
+// stands a block barrier, or every id belongs to the same threads in both.
 template <int SUB> SCINT_DEV void team_sync() {
     if constexpr (SUB == 0) __syncthreads();
     else if constexpr (SUB == 32) __syncwarp();

@@ -80,6 +80,24 @@ int persist_items(int n, int pass) {
     return k;
 }
 
+// Threads of the named barriers of an item (rows: the start's and the lines' parts are one)
+template <int N> __host__ __device__ constexpr int rows_part() { return rows_subs<N>() > 1 ? prow_threads<N>() : 0; }
+template <int N> __host__ __device__ constexpr int cols_part() { return cols_subs<N>() > 1 ? pcol_threads<N>() : 0; }
+int persist_barrier_parts(int n, int pass, int* parts) {
+    int k = 0;
+    dispatch_n(n, [&](auto nc) -> cudaError_t {
+        constexpr int N = decltype(nc)::value;
+        if constexpr (persist_size<N>()) {
+            const int start = pass == 0 ? rows_part<N>() : cols_start_part<N, false, cols_part<N>()>();
+            const int line = pass == 0 ? rows_part<N>() : cols_line_part<N, false, cols_part<N>()>();
+            for (const int part : {start, line})
+                if (part > 32) parts[k++] = part;    // the whole block and single warps use no named barrier
+        }
+        return cudaSuccess;
+    });
+    return k;
+}
+
 SCINT_DEV unsigned ld_acquire(const unsigned* p) {
     unsigned v;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -107,13 +125,11 @@ SCINT_DEV void run_item(const PropArgs& a, int pass, int item, float2* smem) {
         // two bodies side by side synchronise on their own named barriers
         if (pass == 0) {
             constexpr int SUB = prow_threads<N>();
-            constexpr int BAR = rows_subs<N>() > 1 ? SUB : 0;
-            prop_rows_body<N, false, BAR>(a, item * rows_subs<N>() + tid / SUB, tid % SUB,
+            prop_rows_body<N, false, rows_part<N>()>(a, item * rows_subs<N>() + tid / SUB, tid % SUB,
                                           smem + (tid / SUB) * (prow_smem<N>() / sizeof(float2)));
         } else {
             constexpr int SUB = pcol_threads<N>();
-            constexpr int BAR = cols_subs<N>() > 1 ? SUB : 0;
-            prop_cols_body<N, false, BAR>(a, item * cols_subs<N>() + tid / SUB, tid % SUB,
+            prop_cols_body<N, false, cols_part<N>()>(a, item * cols_subs<N>() + tid / SUB, tid % SUB,
                                           smem + (tid / SUB) * (pcol_smem<N>() / sizeof(float2)));
         }
     }

@@ -26,6 +26,8 @@ constexpr size_t kPersistCounterBytes = sizeof(unsigned) * (1 + 2 * kPersistMaxS
 bool persist_supported(int n);          // grid sizes the persistent kernel runs
 size_t persist_smem(int n);             // its shared memory for grid n
 int persist_items(int n, int pass);     // work items of one screen's pass
+// sizes (threads) of the block's parts whose named barriers an item uses, in order of use, at most 2; returns how many
+int persist_barrier_parts(int n, int pass, int* parts);
 cudaError_t launch_persist_args(const PropArgs& a, PropArgs* dst, cudaStream_t s);
 cudaError_t launch_persist_prop(const PersistPlan& pl, size_t smem, cudaStream_t s);
 

@@ -78,6 +78,14 @@ SCINT_DEV void prop_rows_body(const PropArgs& a, int bid, int tid, float2* smem3
     }
 }
 
+// The parts of a block (threads, 0 the whole block) that a column body synchronises, SUB threads of a block
+// long: at its start, where the twiddle table is shared (-1: nothing is shared, no barrier), and in its line transforms.
+template <int N, bool CONJ> __host__ __device__ constexpr bool cols_by_teams() { return !CONJ && col_teams<N>(); }
+template <int N, bool CONJ, int SUB> __host__ __device__ constexpr int cols_start_part() { return cols_by_teams<N, CONJ>() ? -1 : SUB; }
+template <int N, bool CONJ, int SUB> __host__ __device__ constexpr int cols_line_part() {
+    return cols_by_teams<N, CONJ>() ? FftPlan<N, kColEPT>::T : SUB;
+}
+
 // ---- column pass ---------------------------------------------------------------
 // The fields are read through L2 only (ld.global.cg): in the persistent batch kernel a
 // field slot is rewritten by other blocks between uses, and L1 is not coherent across
@@ -88,8 +96,9 @@ SCINT_DEV void prop_cols_body(const PropArgs& a, int bid, int tid, float2* smem3
     constexpr int TWM = pcol_twm<N, CONJ>();
     constexpr int T = Pl::T, E = Pl::E, W = pcol_lines<N>(), WL = pstrip<N>(), BUFL = Pl::BUF;
     // a team of T threads per column (col_teams), or W lines interleaved: element e of line w at pad16(e) * W + w
-    constexpr bool TEAMS = !CONJ && col_teams<N>();
-    constexpr int LW = TEAMS ? 1 : W, SUBC = TEAMS ? T : SUB;
+    constexpr bool TEAMS = cols_by_teams<N, CONJ>();
+    constexpr int LW = TEAMS ? 1 : W, START = cols_start_part<N, CONJ, SUB>(), SUBC = cols_line_part<N, CONJ, SUB>();
+    static_assert(START >= 0 || TWM == 2, "a shared twiddle table needs the barrier");
     const int w = TEAMS ? tid / T : tid % W, t = TEAMS ? tid % T : tid / W;
     const int x0 = bid * W;    // first column of the block: strip x0 / WL, offset x0 % WL
     const int x = x0 + w;
@@ -104,7 +113,7 @@ SCINT_DEV void prop_cols_body(const PropArgs& a, int bid, int tid, float2* smem3
     else if constexpr (TWM == 1) fill_twiddle_table<float2, N>(tws, a.tw, tid, pcol_threads<N>());
 #pragma unroll
     for (int m = 0; m < E; ++m) acc[m] = 0.0f;
-    team_sync<SUB>();
+    if constexpr (START >= 0) team_sync<START>();
 #pragma unroll 1
     for (int l = 0; l < a.lam.count; ++l) {
         const float2* src = a.work + (size_t)l * N * N + (size_t)(x0 / WL) * N * WL + (x0 % WL);
