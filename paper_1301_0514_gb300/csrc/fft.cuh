@@ -268,7 +268,7 @@ SCINT_DEV void dft16_fused(float2* x, const float2* w) {
 // over the T = N/E threads of the line, E/R butterflies per thread.  The stages
 // are radix 16 (EPT 16 or 32), radix 8 (EPT 8) or radix 4 (EPT 4), then one smaller tail stage.
 // With EPT 8 and 4 every stage after the first must have N/R >= 16 (the padded
-// addressing of the loads below), i.e. N >= 128 and N >= 64.
+// addressing of the loads below; fft_stage asserts it), i.e. N >= 128 (or N <= 16) and N >= 64.
 template <int N, int EPT = 16>
 struct FftPlan {
     static_assert(N >= 2 && (N & (N - 1)) == 0, "N must be a power of two");
@@ -455,6 +455,8 @@ SCINT_DEV void fft_stage(C (&v)[FftPlan<N, EPT>::E], C* buf, int t, const C* __r
     constexpr int R = Pl::radix(S), P = Pl::span(S), BF = E / R;
     constexpr bool FIRST = (S == 0), LAST = (S == Pl::NSTAGE - 1);
     constexpr int HALF = N / 2;
+    // the loads below add pad16's parts: N / R a multiple of 16, or no padding before element N at all
+    static_assert(FIRST || (N / R) % 16 == 0 || N <= 16, "no plan: too few values per thread for this length");
     C u[E];
     if constexpr (FIRST) {
         // butterfly b takes positions t + b T + r N/R = t + (b + r BF) T

@@ -63,9 +63,10 @@ SCINT_DEV double taper_of(const Prop64Args& a, int i) {
 template <int N> __host__ __device__ constexpr size_t p64_smem() { return (size_t)FftPlan<N>::BUF * sizeof(double2); }
 // values per thread: 4 at N = 128 and 256 (a line has two warps or one; with eight values per thread
 // and 256 lines the SMs had one or two warps each, and the FP64 pipe was 33 % busy), 8 up to
-// N = 1024 (four were 4 % slower at 512: more FP64 operations, and the lines fill the SMs)
+// N = 1024 (four were 4 % slower at 512: more FP64 operations, and the lines fill the SMs).  Below 128 what
+// has a plan: 4 at 64, 16 at 32 (eight values of 32- and 64-point lines leave stages that fft_stage refuses), 8 at 16.
 template <int N> __host__ __device__ constexpr int p64_ept() {
-    return N == 128 || N == 256 ? 4 : (N <= 1024 ? 8 : 16);
+    return N >= 64 && N <= 256 ? 4 : (N == 32 || N > 1024 ? 16 : 8);
 }
 
 template <int N, bool TAB>
