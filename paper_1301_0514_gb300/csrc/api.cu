@@ -231,6 +231,16 @@ struct TwCache {
 };
 TwCache g_tw;
 
+// An allocation ends every capture that is open in global mode, another thread's or one of this
+// thread's own on another stream; in relaxed mode it concerns none of them.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    RelaxedCapture(const RelaxedCapture&) = delete;
+    RelaxedCapture& operator=(const RelaxedCapture&) = delete;
+};
+
 int cached_twiddles(int n, int kind, cudaStream_t s, const void** out) {
     *out = nullptr;
     int dev = 0;
@@ -247,6 +257,7 @@ int cached_twiddles(int n, int kind, cudaStream_t s, const void** out) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     SCINT_CUDA(cudaStreamIsCapturing(s, &cs));
     if (cs != cudaStreamCaptureStatusNone) return SCINT_OK;
+    const RelaxedCapture relaxed;
     void* p = nullptr;
     if (cudaMalloc(&p, (size_t)n * (kind == kTw32 ? 8 : 16)) != cudaSuccess) {
         cudaGetLastError();
