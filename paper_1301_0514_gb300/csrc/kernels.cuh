@@ -212,7 +212,7 @@ cudaError_t launch_curve_moments(const float* curves, int n_curves, int n_sample
 // ---- screen check of Sect. 3.1.1 (screen_check.cu) --------------------------------
 constexpr int kRadialThreads = 512;
 constexpr int kCrecThreads = 256;
-constexpr int kCrecSplit = 8;       // blocks (one cluster) per lag
+constexpr int kCrecParts = 8;       // parts of a lag's sum, and the most blocks (one cluster) per lag
 constexpr int kBisectBlocks = 148;  // blocks of a root round, shared between its points (and BisectState within 1280 bytes)
 // Annulus sums of |F|^2 and bin counts (an octant of the spectrum walked by `blocks` persistent
 // blocks, n_hist annuli in shared memory), then S_rec = sum / count * inv_l2.

@@ -225,29 +225,53 @@ SCINT_DEV double block_sum_fixed(double v, double* red) {
     return t;
 }
 
-// A lag's sum over a cluster of kCrecSplit blocks (7000 J0 terms keep one SM's narrow FP64 pipe
-// busy for 0.14 ms, and a call has fewer lags than the GPU has SMs: 48 lags 144 -> 56 us), block
-// partials added in rank order through distributed shared memory.
-__global__ void __launch_bounds__(kCrecThreads) crec_kernel(CrecArgs a, const double* r_km, int n_r, double* d) {
-    __shared__ double red[kCrecThreads];
-    __shared__ double part;
+// A lag's terms in kCrecParts parts: thread t of part k takes j = 1 + 256 k + t, then every 2048th.  The parts'
+// sums are added in the order of k, whichever blocks formed them, so a lag's bits do not depend on the call's
+// other lags.  One block per lag, or a cluster when the lags leave SMs idle (launch_crec).
+__global__ void __launch_bounds__(kCrecThreads) crec_kernel(CrecArgs a, const double* r_km, double* d) {
+    static_assert(kCrecThreads == 32 * kCrecParts, "a warp per part");
+    __shared__ double red[kCrecParts][kCrecThreads];
+    __shared__ double part[kCrecParts];
     auto cl = cooperative_groups::this_cluster();
-    const int rank = (int)cl.block_rank(), i = blockIdx.x / kCrecSplit;
-    const double acc = crec_terms(a.s, a.J, a.dq, r_km[i], 1 + rank * (int)blockDim.x + (int)threadIdx.x,
-                                  kCrecSplit * (int)blockDim.x);
-    const double t = block_sum_fixed(acc, red);
-    if (threadIdx.x == 0) part = t;
-    cl.sync();
-    if (rank == 0 && threadIdx.x == 0) {
+    const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank(), i = (int)blockIdx.x / C;
+    const int t = threadIdx.x;
+    const int parts = min(kCrecParts, (a.J + kCrecThreads - 1) / kCrecThreads);    // the others have no term
+    const double r = r_km[i];
+#pragma unroll 1
+    for (int k = rank; k < parts; k += C)
+        red[k][t] = crec_terms(a.s, a.J, a.dq, r, 1 + k * kCrecThreads + t, kCrecParts * kCrecThreads);
+    __syncthreads();
+    // warp w adds up part w (reducing after every part was 6 % slower with 2048 terms)
+    const int w = t / 32, lane = t % 32;
+    if (w < parts && w % C == rank) {
+        double v = 0.0;
+#pragma unroll
+        for (int k = 0; k < kCrecThreads / 32; ++k) v += red[w][32 * k + lane];
+        for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) part[w] = v;
+    }
+    if (C > 1) cl.sync();
+    else __syncthreads();
+    if (rank == 0 && t == 0) {
         double tot = 0.0;
-        for (int k = 0; k < kCrecSplit; ++k) tot += *cl.map_shared_rank(&part, k);
+        for (int k = 0; k < parts; ++k) tot += C > 1 ? *cl.map_shared_rank(&part[k], k % C) : part[k];
         d[i] = 4.0 * kPi * a.dq * tot;
     }
-    cl.sync();    // no block leaves before its partial is read
+    if (C > 1) cl.sync();    // no block leaves before its parts are read
 }
 
+// Blocks per lag.  7000 J0 terms keep one SM's narrow FP64 pipe busy for 0.14 ms, so up to two lags per three
+// SMs go to a cluster of as many blocks as there are parts with terms (at most 8).  From there on the lags fill
+// the SMs by themselves, and the idle threads and barriers of a cluster cost more than the spread gives.  One block /
+// a cluster of eight, us: 48 lags of 7000 terms 146 / 56, 152 lags 146 / 194; 1000 lags of 128 terms 31 / 140.
 cudaError_t launch_crec(const CrecArgs& a, const double* r_km, int n_r, double* d, cudaStream_t s) {
-    return launch_k(crec_kernel, kCrecSplit, dim3(n_r * kCrecSplit), dim3(kCrecThreads), 0, s, a, r_km, n_r, d);
+    int dev = 0, sms = 0, cs = 1;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    if (n_r <= sms * 2 / 3)
+        while (cs < kCrecParts && cs * kCrecThreads < a.J) cs *= 2;
+    return launch_k(crec_kernel, cs, dim3(n_r * cs), dim3(kCrecThreads), 0, s, a, r_km, d);
 }
 
 // ---- R_diff^rec: bisection of D_rec(R) = 1 on (0, L/2] ------------------------------
