@@ -16,6 +16,7 @@
 // regenerated per bin (spectrum.cuh), never stored.  The root takes a few launches (bisect_kernel);
 // within one the blocks' partial sums are combined in a fixed order by the
 // last block to finish, so the result does not depend on scheduling.
+#include <algorithm>
 #include <cmath>
 
 #include <cooperative_groups.h>
@@ -72,22 +73,25 @@ SCINT_DEV unsigned long long to_fixed(double v, int s) {
 // The bins of one octant, 0 <= ax <= ay <= n/2 (a = |m|), stand for the whole grid: up to eight
 // bins (+-ax, +-ay), (+-ay, +-ax) share |m|^2 and so the annulus, its shift and the amplitude
 // (one index search, one powf and one log2 per eight bins; the noise of each bin stays its own).
-// A warp takes kSeg cells of a spectral row ay, each lane kRun of them in a row, in the
+// A warp takes 32 R cells of a spectral row ay, each lane R of them in a row, in the
 // direction in which the annulus changes slowly (at most 0.71 per cell), and adds a run of
 // cells of one annulus in a register before it goes to the block's shared histogram.  The sums
-// are the same integers as bin by bin.  At n = 14000: sums 2.16 -> 1.17 ms (328 -> 176 warp
+// are the same integers as bin by bin.  At n = 14000: sums 2.16 -> 1.14 ms (328 -> 176 warp
 // instructions per 32 bins; Philox and the two branches of -ln u remain, issue 76 %), counts
-// 0.35 -> 0.07 ms, against whole rows per block and a powf and an annulus search per bin.  The tasks go round the
-// blocks, so that the rows ay <= low_k, drawn in FP64, spread over all SMs.
-constexpr int kRun = 4, kSeg = 32 * kRun;
+// 0.35 -> 0.07 ms, against whole rows per block and a powf and an annulus search per bin.  The rows ay <= low_k,
+// drawn in FP64, go first and cell by cell (radial_square).
+// R = 4, or 1 while that leaves warps without a task (1000^2: 51 -> 38 us).
+constexpr int kRun = 4;
 
 // number of (row, segment) tasks of rows 0..h
-__host__ __device__ constexpr int radial_tasks(int h) {
+template <int R> __host__ __device__ constexpr int radial_tasks(int h) {
+    constexpr int kSeg = 32 * R;
     const int G = h / kSeg;
     return kSeg * (G * (G + 1) / 2) + (h + 1 - G * kSeg) * (G + 1);
 }
-// task -> (row ay, first cell): rows [g kSeg, (g + 1) kSeg) have g + 1 segments each
-SCINT_DEV void radial_task(int task, int& ay, int& ax0) {
+// task -> (row ay, first cell): rows [g kSeg, (g + 1) kSeg), kSeg = 32 R, have g + 1 segments each
+template <int R> SCINT_DEV void radial_task(int task, int& ay, int& ax0) {
+    constexpr int kSeg = 32 * R;
     int g = (int)((sqrtf(8.0f * ((float)task / kSeg) + 1.0f) - 1.0f) * 0.5f);
     while (kSeg * ((g + 1) * (g + 2) / 2) <= task) ++g;
     while (kSeg * (g * (g + 1) / 2) > task) --g;
@@ -96,11 +100,51 @@ SCINT_DEV void radial_task(int task, int& ay, int& ax0) {
     ax0 = (rem % (g + 1)) * kSeg;
 }
 
+// The octant's rows 0..min(low_k, n/2), whose bins are drawn in FP64: a cell per group of G lanes (1, 2, 4 or 8),
+// which share its up to eight draws.  In runs of four cells per lane the chain of 32 logarithms took 50 us, longer
+// than the whole sums of a small grid.
+__host__ __device__ constexpr int square_cells(int rows) { return rows * (rows + 1) / 2; }
+// Lanes per cell: a draw costs about 30 instructions on the FP64 pipe and a cell's amplitude 70, repeated by each
+// of its lanes; so many lanes while latency counts, one when the pipe is full.
+inline int square_lanes(int cells) { return cells <= 4096 ? 8 : (cells <= 12288 ? 4 : (cells <= 16384 ? 2 : 1)); }
+SCINT_DEV void radial_square(const SynthArgs& a, int rows, int n_hist, int G, unsigned long long* hs) {
+    const int n = a.n, h = n / 2, cells = square_cells(rows);
+    const int lane = threadIdx.x & 31, g = lane & (G - 1);
+    const int step = (int)gridDim.x * (kRadialThreads / 32) * (32 / G);
+#pragma unroll 1
+    for (int c0 = ((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * (32 / G); c0 < cells; c0 += step) {
+        const int c = c0 + lane / G;
+        unsigned long long acc = 0ull;
+        int j = n_hist;
+        if (c < cells) {
+            int ay = (int)((sqrtf(8.0f * (float)c + 1.0f) - 1.0f) * 0.5f);
+            while (square_cells(ay + 1) <= c) ++ay;
+            while (square_cells(ay) > c) --ay;
+            const int ax = c - square_cells(ay), m2 = ax * ax + ay * ay;
+            j = annulus_of(m2);
+            if (j < n_hist && m2 > 0) {
+                const int shift = annulus_shift(a, j);
+                const double sig = amplitude_low(a, m2), sig2 = sig * sig;
+#pragma unroll 1
+                for (int d = g; d < 8; d += G) {
+                    // (ax, ay) or (ay, ax), then the mirror bins in y (d & 2) and x (d & 1): 0 and -n/2 have none
+                    const int px = d < 4 ? ax : ay, py = d < 4 ? ay : ax;
+                    if ((d >= 4 && ax == ay) || ((d & 2) && (py == 0 || py == h)) || ((d & 1) && (px == 0 || px == h))) continue;
+                    const u32x4 w = bin_words(a, d & 1 ? n - px : px, d & 2 ? n - py : py);
+                    acc += to_fixed(sig2 * (2.0 * neg_log_ua64(w)), shift);
+                }
+            }
+        }
+        for (int o = 1; o < G; o *= 2) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (g == 0 && j < n_hist) atomicAdd(hs + j, acc);
+    }
+}
+
 // COUNT: bins per annulus.  Otherwise: fixed-point sums of |F|^2 (high bins from
 // their FP32 value, low bins from their FP64 value, as the synthesis draws them).
-template <bool COUNT>
+template <bool COUNT, int R>
 __global__ void __launch_bounds__(kRadialThreads)
-radial_kernel(SynthArgs a, int n_hist, unsigned long long* sums, unsigned long long* counts) {
+radial_kernel(SynthArgs a, int n_hist, int square_group, unsigned long long* sums, unsigned long long* counts) {
     extern __shared__ __align__(16) unsigned char radial_smem[];
     unsigned long long* hs = reinterpret_cast<unsigned long long*>(radial_smem);
     unsigned* hc = reinterpret_cast<unsigned*>(radial_smem);
@@ -110,20 +154,24 @@ radial_kernel(SynthArgs a, int n_hist, unsigned long long* sums, unsigned long l
     }
     __syncthreads();
     const int n = a.n, h = n / 2;
-    const int tasks = radial_tasks(h), lane = threadIdx.x & 31;
+    // row ay has no annulus below ay
+    const int top = min(h, n_hist), square = min(a.low_k, top);
+    const int tasks = radial_tasks<R>(top), lane = threadIdx.x & 31;
     const int warps = gridDim.x * (kRadialThreads / 32);
+    if (!COUNT) radial_square(a, square + 1, n_hist, square_group, hs);
+    const int first = COUNT ? 0 : radial_tasks<R>(square);    // the rows above the square
 #pragma unroll 1
-    for (int task = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; task < tasks; task += warps) {
+    for (int task = first + (threadIdx.x >> 5) * gridDim.x + blockIdx.x; task < tasks; task += warps) {
         int ay, ax0;
-        radial_task(task, ay, ax0);
-        ax0 += lane * kRun;
+        radial_task<R>(task, ay, ax0);
+        ax0 += lane * R;
         int cur = -1, shift = 0;
         unsigned long long acc = 0ull;
         unsigned cnt = 0u;
         // frequency -h and its mirror are one bin, and so is 0
         const bool two_y = ay != 0 && ay != h;
 #pragma unroll 1
-        for (int i = 0; i < kRun; ++i) {
+        for (int i = 0; i < R; ++i) {
             const int ax = ax0 + i;
             if (ax > ay) break;
             const int m2 = ax * ax + ay * ay;
@@ -141,10 +189,8 @@ radial_kernel(SynthArgs a, int n_hist, unsigned long long* sums, unsigned long l
             const bool two_x = ax != 0 && ax != h;
             if (COUNT) {
                 cnt += (two_x ? 2u : 1u) * (two_y ? 2u : 1u) * (ax != ay ? 2u : 1u);
-            } else if (j < n_hist && m2 > 0) {
-                const bool low = ay <= a.low_k;    // ax <= ay
-                const double sig_low = low ? amplitude_low(a, m2) : 0.0, sig2_low = sig_low * sig_low;
-                const float sig = low ? 0.0f : amplitude_high(a, m2), sig2 = sig * sig;
+            } else if (j < n_hist) {
+                const float sig = amplitude_high(a, m2), sig2 = sig * sig;
                 // (ax, ay) and, off the diagonal, (ay, ax); each with both signs of both
 #pragma unroll 1
                 for (int q = 0; q < (ax != ay ? 4 : 2); ++q) {
@@ -154,13 +200,8 @@ radial_kernel(SynthArgs a, int n_hist, unsigned long long* sums, unsigned long l
                     const uint32_t ky = (uint32_t)((q & 1) ? n - py : py);
                     const u32x4 w = philox4x32_10(u32x4{(uint32_t)px, ky, a.screen_id, 0u}, a.key0, a.key1);
                     const u32x4 v = philox4x32_10(u32x4{(uint32_t)(n - px), ky, a.screen_id, 0u}, a.key0, a.key1);
-                    if (low) {
-                        acc += to_fixed(sig2_low * (2.0 * neg_log_ua64(w)), shift);
-                        if (two_px) acc += to_fixed(sig2_low * (2.0 * neg_log_ua64(v)), shift);
-                    } else {
-                        acc += to_fixed(sig2 * (2.0f * neg_log_ua32(w)), shift);
-                        if (two_px) acc += to_fixed(sig2 * (2.0f * neg_log_ua32(v)), shift);
-                    }
+                    acc += to_fixed(sig2 * (2.0f * neg_log_ua32(w)), shift);
+                    if (two_px) acc += to_fixed(sig2 * (2.0f * neg_log_ua32(v)), shift);
                 }
             }
         }
@@ -188,15 +229,25 @@ __global__ void radial_finish_kernel(SynthArgs a, int n_hist, double inv_l2, dou
     s[j] = counts[j] ? ldexp((double)fx, -annulus_shift(a, j)) / (double)counts[j] * inv_l2 : 0.0;
 }
 
-cudaError_t launch_radial_spectrum(const SynthArgs& a, double inv_l2, int n_hist, double* s_rec,
-                                   unsigned long long* counts, int blocks, cudaStream_t s) {
+template <int R>
+static cudaError_t launch_radial(const SynthArgs& a, int n_hist, unsigned long long* sums, unsigned long long* counts,
+                                 int blocks, cudaStream_t s) {
     const size_t bytes_s = (size_t)n_hist * sizeof(unsigned long long), bytes_c = (size_t)n_hist * sizeof(unsigned);
     cudaError_t e;
-    if ((e = set_smem(radial_kernel<false>, bytes_s)) != cudaSuccess) return e;
-    if ((e = set_smem(radial_kernel<true>, bytes_c)) != cudaSuccess) return e;
+    if ((e = set_smem(radial_kernel<false, R>, bytes_s)) != cudaSuccess) return e;
+    if ((e = set_smem(radial_kernel<true, R>, bytes_c)) != cudaSuccess) return e;
+    const int group = square_lanes(square_cells(std::min(a.low_k, std::min(a.n / 2, n_hist)) + 1));
+    radial_kernel<true, R><<<blocks, kRadialThreads, bytes_c, s>>>(a, n_hist, 0, sums, counts);
+    radial_kernel<false, R><<<blocks, kRadialThreads, bytes_s, s>>>(a, n_hist, group, sums, counts);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_radial_spectrum(const SynthArgs& a, double inv_l2, int n_hist, double* s_rec,
+                                   unsigned long long* counts, int blocks, cudaStream_t s) {
     unsigned long long* fx = reinterpret_cast<unsigned long long*>(s_rec);
-    radial_kernel<true><<<blocks, kRadialThreads, bytes_c, s>>>(a, n_hist, fx, counts);
-    radial_kernel<false><<<blocks, kRadialThreads, bytes_s, s>>>(a, n_hist, fx, counts);
+    const bool runs = radial_tasks<kRun>(std::min(a.n / 2, n_hist)) >= blocks * (kRadialThreads / 32);
+    const cudaError_t e = runs ? launch_radial<kRun>(a, n_hist, fx, counts, blocks, s) : launch_radial<1>(a, n_hist, fx, counts, blocks, s);
+    if (e != cudaSuccess) return e;
     radial_finish_kernel<<<(n_hist + 255) / 256, 256, 0, s>>>(a, n_hist, inv_l2, s_rec, counts);
     return cudaGetLastError();
 }

@@ -147,18 +147,4 @@ SCINT_DEV void spectrum_pair_high(const SynthArgs& a, int kx, int ky, float2& f,
     g = shaped_high(w2, sig);
 }
 
-// |F[ky][kx]|^2 = sigma^2 (g_re^2 + g_im^2) / 2 = sigma^2 (-2 ln u_a) / 2 of a
-// bin with Philox words w and m2 = mx^2 + my^2 > 0 (the Box-Muller angle
-// cancels), in the precision spectrum_bin uses for it: FP64 for the low bins
-// (|mx|, |my| <= a.low_k), FP32 for the others.
-SCINT_DEV bool low_bin(const SynthArgs& a, int mx, int my) { return abs(mx) <= a.low_k && abs(my) <= a.low_k; }
-SCINT_DEV double power_low(const SynthArgs& a, const u32x4& w, int m2) {
-    const double sig = amplitude_low(a, m2);
-    return sig * sig * (2.0 * neg_log_ua64(w));
-}
-SCINT_DEV float power_high(const SynthArgs& a, const u32x4& w, int m2) {
-    const float sig = amplitude_high(a, m2);
-    return sig * sig * (2.0f * neg_log_ua32(w));
-}
-
 }  // namespace scint
