@@ -96,15 +96,15 @@ __device__ double block_sum_all(double v) {
     return t;
 }
 
-// U samples of a thread (0 past the end) as doubles, through their bits unless one of them is unusual:
+// U samples of a thread as doubles, through their bits unless one of them is unusual:
 // on GB300's narrow FP64 pipe a conversion costs as much as two additions.
 template <int U>
-SCINT_DEV void load_widened(const float* x, int s, int step, int n, double (&d)[U]) {
+SCINT_DEV void load_widened(const float* x, int step, double (&d)[U]) {
     float v[U];
     bool odd = false;
 #pragma unroll
     for (int k = 0; k < U; ++k) {
-        v[k] = s + k * step < n ? x[s + k * step] : 0.0f;
+        v[k] = x[(size_t)k * step];
         odd |= f2d_unusual(v[k]);
     }
     if (!odd) {
@@ -115,56 +115,66 @@ SCINT_DEV void load_widened(const float* x, int s, int step, int n, double (&d)[
         for (int k = 0; k < U; ++k) d[k] = (double)v[k];
     }
 }
+// f(k, x_s, y_s) for this thread's samples s: U at a time (k = 0..U - 1), the rest one by one (k = 0)
+template <int U, typename F>
+SCINT_DEV void for_samples(const float* x, const float* y, int n, F&& f) {
+    const int step = blockDim.x;
+    int s = threadIdx.x;
+    if constexpr (U > 1) {
+        for (; n - s > (U - 1) * step; s += U * step) {
+            double xv[U], yv[U];
+            load_widened(x + s, step, xv);
+            load_widened(y + s, step, yv);
+#pragma unroll
+            for (int k = 0; k < U; ++k) f(k, xv[k], yv[k]);
+        }
+    }
+#pragma unroll 1
+    for (; s < n; s += step) {
+        double xv[1], yv[1];
+        load_widened(x + s, step, xv);
+        load_widened(y + s, step, yv);
+        f(0, xv[0], yv[0]);
+    }
+}
 
-// The FP64 pipe bounds it (384 pairs of 4096 samples: 61 -> 54 us, 85 % busy before): four samples of a thread at a
-// time, each with sums of its own, so that the additions do not wait for one another.
+// The FP64 pipe bounds it (384 pairs of 4096 samples: 61 -> 54 us, 85 % busy before): U samples of a
+// thread at a time, each with sums of its own, so that the additions do not wait for one another.
+template <int U>
+SCINT_DEV double block_total(const double (&v)[U]) {
+    if constexpr (U == 4) return block_sum_all((v[0] + v[1]) + (v[2] + v[3]));
+    else return block_sum_all(v[0]);
+}
+template <int U>
 __global__ void __launch_bounds__(256) correlation_kernel(const float* a, int group, long long a_stride,
                                                           const float* b, int n, double* r) {
     const int i = blockIdx.x;
     const float* x = a + (size_t)(i / group) * a_stride;
     const float* y = b + (size_t)i * n;
-    constexpr int U = 4;
-    const int step = blockDim.x;
     double ax[U] = {}, ay[U] = {};
-    for (int s = threadIdx.x; s < n; s += U * step) {
-        double xv[U], yv[U];
-        load_widened(x, s, step, n, xv);
-        load_widened(y, s, step, n, yv);
-#pragma unroll
-        for (int k = 0; k < U; ++k) {
-            ax[k] += xv[k];
-            ay[k] += yv[k];
-        }
-    }
-    const double mx = block_sum_all((ax[0] + ax[1]) + (ax[2] + ax[3])) / n;
-    const double my = block_sum_all((ay[0] + ay[1]) + (ay[2] + ay[3])) / n;
+    for_samples<U>(x, y, n, [&](int k, double xv, double yv) {
+        ax[k] += xv;
+        ay[k] += yv;
+    });
+    const double mx = block_total(ax) / n, my = block_total(ay) / n;
     double axy[U] = {}, axx[U] = {}, ayy[U] = {};
-    for (int s = threadIdx.x; s < n; s += U * step) {
-        double xv[U], yv[U];
-        load_widened(x, s, step, n, xv);
-        load_widened(y, s, step, n, yv);
-#pragma unroll
-        for (int k = 0; k < U; ++k) {
-            if (s + k * step < n) {
-                const double dx = xv[k] - mx, dy = yv[k] - my;
-                axy[k] = fma(dx, dy, axy[k]);
-                axx[k] = fma(dx, dx, axx[k]);
-                ayy[k] = fma(dy, dy, ayy[k]);
-            }
-        }
-    }
-    double sxy = (axy[0] + axy[1]) + (axy[2] + axy[3]), sxx = (axx[0] + axx[1]) + (axx[2] + axx[3]),
-           syy = (ayy[0] + ayy[1]) + (ayy[2] + ayy[3]);
-    sxy = block_sum_all(sxy);
-    sxx = block_sum_all(sxx);
-    syy = block_sum_all(syy);
+    for_samples<U>(x, y, n, [&](int k, double xv, double yv) {
+        const double dx = xv - mx, dy = yv - my;
+        axy[k] = fma(dx, dy, axy[k]);
+        axx[k] = fma(dx, dx, axx[k]);
+        ayy[k] = fma(dy, dy, ayy[k]);
+    });
+    const double sxy = block_total(axy), sxx = block_total(axx), syy = block_total(ayy);
     if (threadIdx.x == 0) r[i] = sxy / sqrt(sxx * syy);
 }
 
 cudaError_t launch_correlation(const float* a, int a_rows, long long a_stride, const float* b, int n_pairs, int n,
                                double* r, cudaStream_t s) {
     if (n_pairs <= 0) return cudaSuccess;
-    correlation_kernel<<<n_pairs, 256, 0, s>>>(a, n_pairs / a_rows, a_stride, b, n, r);
+    // four samples at a time from four samples per thread on; below, one by one in fewer registers (10000 pairs of
+    // 256 samples: 620 us with four sums of which three stay zero, 464 without)
+    if (n >= 4 * 256) correlation_kernel<4><<<n_pairs, 256, 0, s>>>(a, n_pairs / a_rows, a_stride, b, n, r);
+    else correlation_kernel<1><<<n_pairs, 256, 0, s>>>(a, n_pairs / a_rows, a_stride, b, n, r);
     return cudaGetLastError();
 }
 
