@@ -923,8 +923,7 @@ cudaError_t launch_rows(const PropArgs& a, cudaStream_t s) {
                 if (e != cudaSuccess) return e;
                 k<<<blocks, LongPlan<N>::T, prow_long_smem<N>(), s>>>(a, reinterpret_cast<uintptr_t>(a.phi) % 16 == 0);
                 return cudaGetLastError();
-            }
-            if constexpr (row_stream<N>()) {
+            } else if constexpr (row_stream<N>()) {
                 static_assert(prow_stream_smem<N>() <= kMaxSmem, "streamed row pass does not fit");
                 auto k = prop_rows_stream_kernel<N, CONJ>;
                 cudaError_t e = set_smem(k, prow_stream_smem<N>());
@@ -935,11 +934,12 @@ cudaError_t launch_rows(const PropArgs& a, cudaStream_t s) {
                 // a bulk copy starts on a 16-byte boundary: phases elsewhere are read by plain loads
                 return launch_pass<N>(a.lam.count, k, dim3(blocks), dim3(prow_threads<N>()), prow_stream_smem<N>(), s, a,
                                       (int)(reinterpret_cast<uintptr_t>(a.phi) % 16 == 0));
+            } else {
+                cudaError_t e = set_smem(prop_rows_kernel<N, CONJ>, prow_smem<N>());
+                if (e != cudaSuccess) return e;
+                return launch_pass<N>(a.lam.count, prop_rows_kernel<N, CONJ>, dim3(N / prow_lines<N>()),
+                                      dim3(prow_threads<N>()), prow_smem<N>(), s, a);
             }
-            cudaError_t e = set_smem(prop_rows_kernel<N, CONJ>, prow_smem<N>());
-            if (e != cudaSuccess) return e;
-            return launch_pass<N>(a.lam.count, prop_rows_kernel<N, CONJ>, dim3(N / prow_lines<N>()), dim3(prow_threads<N>()),
-                                  prow_smem<N>(), s, a);
         }
     });
 }
@@ -973,27 +973,28 @@ cudaError_t launch_cols(const PropArgs& a, cudaStream_t s) {
                 if (e != cudaSuccess) return e;
                 return launch_k(k, kLongCluster, dim3(N), dim3(LongPlan<N>::T), pcol_long_smem<N>(), s, a,
                                 (int)(reinterpret_cast<uintptr_t>(a.intensity) % 16 == 0));
-            }
-            if constexpr (!CONJ && col_stream<N>()) {
-                static_assert(pcol_stream_smem<N>() <= kMaxSmem, "streamed column pass does not fit");
-                CUtensorMap tm;
-                if (a.h && field_map(&tm, a.work, N, a.lam.count, pstrip<N>())) {
-                    auto k = prop_cols_stream_kernel<N>;
-                    cudaError_t e = set_smem(k, pcol_stream_smem<N>());
-                    int blocks = 0;
-                    if (e == cudaSuccess)
-                        e = walk_blocks(k, pcol_threads<N>(), pcol_stream_smem<N>(), N / pcol_lines<N>(), a.lam.count, &blocks);
-                    if (e != cudaSuccess) return e;
-                    constexpr int align = pcol_lines<N>() == 2 ? 8 : 16;
-                    return launch_pass<N>(a.lam.count, k, dim3(blocks), dim3(pcol_threads<N>()), pcol_stream_smem<N>(), s, a, tm,
-                                          (int)(reinterpret_cast<uintptr_t>(a.intensity) % align == 0));
+            } else {
+                if constexpr (!CONJ && col_stream<N>()) {
+                    static_assert(pcol_stream_smem<N>() <= kMaxSmem, "streamed column pass does not fit");
+                    CUtensorMap tm;
+                    if (a.h && field_map(&tm, a.work, N, a.lam.count, pstrip<N>())) {
+                        auto k = prop_cols_stream_kernel<N>;
+                        cudaError_t e = set_smem(k, pcol_stream_smem<N>());
+                        int blocks = 0;
+                        if (e == cudaSuccess)
+                            e = walk_blocks(k, pcol_threads<N>(), pcol_stream_smem<N>(), N / pcol_lines<N>(), a.lam.count, &blocks);
+                        if (e != cudaSuccess) return e;
+                        constexpr int align = pcol_lines<N>() == 2 ? 8 : 16;
+                        return launch_pass<N>(a.lam.count, k, dim3(blocks), dim3(pcol_threads<N>()), pcol_stream_smem<N>(), s, a, tm,
+                                              (int)(reinterpret_cast<uintptr_t>(a.intensity) % align == 0));
+                    }
                 }
+                constexpr size_t smem = pcol_smem<N, CONJ>();
+                cudaError_t e = set_smem(prop_cols_kernel<N, CONJ>, smem);
+                if (e != cudaSuccess) return e;
+                return launch_pass<N>(a.lam.count, prop_cols_kernel<N, CONJ>, dim3(N / pcol_lines<N>()), dim3(pcol_threads<N>()), smem,
+                                      s, a);
             }
-            constexpr size_t smem = pcol_smem<N, CONJ>();
-            cudaError_t e = set_smem(prop_cols_kernel<N, CONJ>, smem);
-            if (e != cudaSuccess) return e;
-            return launch_pass<N>(a.lam.count, prop_cols_kernel<N, CONJ>, dim3(N / pcol_lines<N>()), dim3(pcol_threads<N>()), smem,
-                                  s, a);
         }
     });
 }
