@@ -457,6 +457,7 @@ void fill_lambda(LambdaSet& ls, int i, const scint_params* p, double lam, double
 // evaluate it (a workspace of the least size under a capture that has no kept twiddles).
 void group_tables(TableArgs& ta, PropArgs& pa, const Carver& cg, float2* slot, const float2* tw) {
     const size_t bytes = ws_transfer(ta.n, ta.count);
+    if (bytes == 0) return;
     if (cg.used + bytes <= cg.size) ta.h = reinterpret_cast<float2*>(cg.base + cg.used);
     else if (ta.count == 1 && tw != slot) ta.h = slot;
     for (int i = 0; i < ta.count; ++i) ta.h_fx[i] = pa.lam.h_fx[i];
@@ -818,7 +819,7 @@ int persist_propagate(const scint_params* const* params, const double* const* ph
         }
         ta.sf = reinterpret_cast<float*>(sf_of[i]);
         pa.sf = ta.sf;
-        if (tables) {
+        if (tables && ws_transfer(nn, n_lambda)) {
             ta.h = reinterpret_cast<float2*>(tables);
             tables += ws_transfer(nn, n_lambda);
             for (int l = 0; l < n_lambda; ++l) ta.h_fx[l] = pa.lam.h_fx[l];

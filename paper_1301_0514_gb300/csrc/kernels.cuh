@@ -89,10 +89,10 @@ struct PropArgs {
     float one;               // 1.0f: the multiplier of the packed passes' additions (fft2.cuh)
 };
 // The tables of a wavelength group, per wavelength: the taper SF at the pixel centres and, if h is
-// set, the transfer function H_x.  H_x is even: up to n = 4096 entry i is H_x(i), i = 0..n/2 (and one of
-// padding, for 16-byte rows); at 8192 entry i is frequency i in FFT order; at kSplitN the even
+// set, the transfer function H_x (from n = 512 on).  H_x is even: up to n = 4096 entry i is H_x(i), i = 0..n/2 (and
+// one of padding, for 16-byte rows); at 8192 entry i is frequency i in FFT order; at kSplitN the even
 // frequencies in order, then the odd ones.
-__host__ __device__ constexpr int transfer_entries(int n) { return n <= 4096 ? n / 2 + 2 : n; }
+__host__ __device__ constexpr int transfer_entries(int n) { return n < 512 ? 0 : (n <= 4096 ? n / 2 + 2 : n); }
 struct TableArgs {
     int n, count;
     double margin_px[kMaxLambda];     // taper margin in pixels (0 = no taper)

@@ -6,18 +6,6 @@
 
 namespace scint {
 
-// v times H_x, from a half table h or evaluated here
-template <int N, int E>
-SCINT_DEV void apply_transfer(float2 (&v)[E], const float2* h, unsigned long long hc, int t) {
-    if (h) {
-#pragma unroll
-        for (int m = 0; m < E; ++m) v[m] = cmul(v[m], __ldg(h + half_index<N, E>(t, m)));
-    } else {
-#pragma unroll
-        for (int m = 0; m < E; ++m) v[m] = cmul(v[m], transfer_signed(hc, signed_index<N, E>(t, m)));
-    }
-}
-
 // ---- row pass ------------------------------------------------------------------
 // The pass bodies take the block index, the thread index and the block's shared memory
 // as arguments, so that the persistent batch kernel (persist.cu) runs the same code as
@@ -97,6 +85,8 @@ SCINT_DEV void prop_cols_body(const PropArgs& a, int bid, int tid, float2* smem3
     constexpr int T = Pl::T, E = Pl::E, W = pcol_lines<N>(), WL = pstrip<N>(), BUFL = Pl::BUF;
     // a team of T threads per column (col_teams), or W lines interleaved: element e of line w at pad16(e) * W + w
     constexpr bool TEAMS = cols_by_teams<N, CONJ>();
+    // without teams H_x is evaluated once per block and wavelength, into two tables in turn (behind the twiddles)
+    constexpr bool OWN_H = own_transfer<N, CONJ>();
     constexpr int LW = TEAMS ? 1 : W, START = cols_start_part<N, CONJ, SUB>(), SUBC = cols_line_part<N, CONJ, SUB>();
     static_assert(START >= 0 || TWM == 2, "a shared twiddle table needs the barrier");
     const int w = TEAMS ? tid / T : tid % W, t = TEAMS ? tid % T : tid / W;
@@ -108,6 +98,7 @@ SCINT_DEV void prop_cols_body(const PropArgs& a, int bid, int tid, float2* smem3
     float acc[E];
     float2* tws = smem32 + W * BUFL;   // shared twiddle table (after the line buffers)
     const float2* twp = TWM == 1 ? tws : a.tw;
+    float2* own_h = tws + (TWM == 1 ? Pl::TWS : 0);
     TwiddleRegs<float2, N, kColEPT> tr;
     if constexpr (TWM == 2) tr.load(a.tw, t);
     else if constexpr (TWM == 1) fill_twiddle_table<float2, N>(tws, a.tw, tid, pcol_threads<N>());
@@ -117,6 +108,10 @@ SCINT_DEV void prop_cols_body(const PropArgs& a, int bid, int tid, float2* smem3
 #pragma unroll 1
     for (int l = 0; l < a.lam.count; ++l) {
         const float2* src = a.work + (size_t)l * N * N + (size_t)(x0 / WL) * N * WL + (x0 % WL);
+        float2* h = own_h + (l & 1) * own_entries<N>();
+        if constexpr (OWN_H) {
+            for (int i = tid; i < own_entries<N>(); i += pcol_threads<N>()) h[i] = transfer_signed(a.lam.h_fx[l], i);
+        }
         float2 v[E];
 #pragma unroll
         for (int m = 0; m < E; ++m) v[m] = __ldcg(src + (size_t)(t + m * T) * WL + w);
@@ -137,8 +132,19 @@ SCINT_DEV void prop_cols_body(const PropArgs& a, int bid, int tid, float2* smem3
             }
             continue;
         } else {
-            const unsigned long long hc = a.lam.h_fx[l];
-            apply_transfer<N, E>(v, N <= 4096 && a.h ? a.h + (size_t)l * transfer_entries(N) : nullptr, hc, t);
+            if constexpr (OWN_H) {
+                // written before the forward transform's barriers; this table's turn comes again after the next one's
+                if constexpr (Pl::NSTAGE == 1) team_sync<SUB>();
+#pragma unroll
+                for (int m = 0; m < E; ++m) v[m] = cmul(v[m], h[half_index<N, E>(t, m)]);
+            } else if (a.h) {
+                const float2* ht = a.h + (size_t)l * transfer_entries(N);
+#pragma unroll
+                for (int m = 0; m < E; ++m) v[m] = cmul(v[m], __ldg(ht + half_index<N, E>(t, m)));
+            } else {
+#pragma unroll
+                for (int m = 0; m < E; ++m) v[m] = cmul(v[m], transfer_signed(a.lam.h_fx[l], signed_index<N, E>(t, m)));
+            }
             if constexpr (TWM == 2) fft_line_tr<float2, N, +1, kColEPT, LW, 1, SUBC>(v, buf, t, tr);
             else fft_line<float2, N, +1, kColEPT, LW, TWM, 1, 1, SUBC>(v, buf, t, twp);
         }

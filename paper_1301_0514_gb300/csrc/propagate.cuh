@@ -65,8 +65,15 @@ template <int N, bool CONJ> __host__ __device__ constexpr int pcol_twm() {
     return !CONJ && col_teams<N>() ? 2 : (kColTw == 1 && pcol_base_bytes<N>() + (size_t)FftPlan<N>::TWS * sizeof(float2) > kMaxSmem
                 ? 2 : kColTw);
 }
+// Below 512 a block's columns evaluate H_x once per block and wavelength into shared memory: with two tables there,
+// and no barrier of their own, that is less than the latency of a table's loads behind the forward transform, which few
+// blocks and warps hide (32 wavelengths at 64^2, the whole call: 145 us with tables in memory, 143 when each element
+// took its own hardware sine, 133 so; at 256^2 149, 148 and 140).
+template <int N, bool CONJ> __host__ __device__ constexpr bool own_transfer() { return !CONJ && N < 512; }
+template <int N> __host__ __device__ constexpr int own_entries() { return N / 2 + 1; }
 template <int N, bool CONJ = false> constexpr size_t pcol_smem() {
-    return pcol_base_bytes<N>() + ptws_bytes<N>(pcol_twm<N, CONJ>());
+    return pcol_base_bytes<N>() + ptws_bytes<N>(pcol_twm<N, CONJ>()) +
+           (own_transfer<N, CONJ>() ? 2 * own_entries<N>() * sizeof(float2) : 0);
 }
 
 // signed FFT frequency index of bin i
