@@ -139,10 +139,10 @@ size_t ws_prop(int n, int g) {
 // the transfer function's tables of a group: part of every workspace size given out, taken where
 // there is room (group_tables), so that a workspace of ws_prop alone still does
 size_t ws_transfer(int n, int g) { return up((size_t)g * transfer_entries(n) * 8); }
-// the largest group of up to g wavelengths that a workspace of `bytes` holds besides `rest`; one smaller,
-// rather than without its tables
+// the largest group of up to g wavelengths that a workspace of `bytes` holds besides `rest`, with or without
+// its tables: another group costs more than the passes' own evaluation
 int group_size(int n, int g, size_t bytes, size_t rest) {
-    while (g > 1 && rest + ws_prop(n, g) + ws_transfer(n, g) > bytes) --g;
+    while (g > 1 && rest + ws_prop(n, g) > bytes) --g;
     return g;
 }
 size_t ws_prop64(int n) { return n <= kMax64N ? up((size_t)n * 16) + up((size_t)n * n * 16) : 0; }

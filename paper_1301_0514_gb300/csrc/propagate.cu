@@ -227,11 +227,15 @@ SCINT_DEV void store_row(float* o, float (&r)[W], int wide, int accumulate) {
     }
 }
 
-template <int N> constexpr size_t pcol_stream_smem() {
-    return col_stage_bytes<N>() + (size_t)(pcol_lines<N>() * FftPlan<N>::BUF + transfer_entries(N)) * sizeof(float2) + 24;
+// TAB: H_x by a copy from the group's tables.  A workspace without room for them has the block evaluate the
+// half table itself, two tables in turn, one barrier between its making and its use (32 wavelengths in one group, with
+// tables / so / with an evaluation per element: 1075 / 1144 / 1281 us at 2048^2, 4.91 / 5.12 / 5.36 ms at 4096^2).
+template <int N, bool TAB> __host__ __device__ constexpr int stream_entries() { return TAB ? transfer_entries(N) : 2 * own_entries<N>(); }
+template <int N, bool TAB> constexpr size_t pcol_stream_smem() {
+    return col_stage_bytes<N>() + (size_t)(pcol_lines<N>() * FftPlan<N>::BUF + stream_entries<N, TAB>()) * sizeof(float2) + 24;
 }
 
-template <int N>
+template <int N, bool TAB>
 __global__ void __launch_bounds__(pcol_threads<N>(), (pcol_threads<N>() <= 256 ? 2 : 1))
 prop_cols_stream_kernel(PropArgs a, const __grid_constant__ CUtensorMap tm, int wide) {
     using Pl = FftPlan<N, kColEPT>;
@@ -244,7 +248,7 @@ prop_cols_stream_kernel(PropArgs a, const __grid_constant__ CUtensorMap tm, int 
     float2* buf = bufs + w * Pl::BUF;
     constexpr int HT = transfer_entries(N);
     float2* hs = bufs + W * Pl::BUF;
-    unsigned long long* bar = reinterpret_cast<unsigned long long*>(hs + HT);    // stage, H
+    unsigned long long* bar = reinterpret_cast<unsigned long long*>(hs + stream_entries<N, TAB>());    // stage, H
     unsigned* reads = reinterpret_cast<unsigned*>(bar + 2);    // teams that have read the stage, H
     const int count = a.lam.count;
     auto load_h = [&](int l) {
@@ -257,7 +261,7 @@ prop_cols_stream_kernel(PropArgs a, const __grid_constant__ CUtensorMap tm, int 
         reads[0] = reads[1] = 0u;
         tile_init_fence();
         issue_columns<N>(stage, &tm, 0, blockIdx.x * W, bar);
-        load_h(0);
+        if (TAB) load_h(0);
     }
     TwiddleRegs<float2, N, 16> tr;
     tr.load(a.tw, t);
@@ -271,6 +275,11 @@ prop_cols_stream_kernel(PropArgs a, const __grid_constant__ CUtensorMap tm, int 
         for (int m = 0; m < E; ++m) acc[m] = 0.0f;
 #pragma unroll 1
         for (int l = 0; l < count; ++l) {
+            const bool new_h = count > 1 || x0 == (int)blockIdx.x * W;
+            float2* h = TAB ? hs : hs + (l & 1) * own_entries<N>();
+            if (!TAB && new_h) {
+                for (int i = threadIdx.x; i < own_entries<N>(); i += pcol_threads<N>()) h[i] = transfer_signed(a.lam.h_fx[l], i);
+            }
             ok = ok && wait_tile(bar, parity & 1);
             parity ^= 1;
             float2 v[E];
@@ -289,14 +298,16 @@ prop_cols_stream_kernel(PropArgs a, const __grid_constant__ CUtensorMap tm, int 
                 }
             }
             const bool more = x0 + (int)gridDim.x * W < N;
-            if (count > 1 || x0 == (int)blockIdx.x * W) {
+            if (TAB && new_h) {
                 ok = ok && wait_tile(bar + 1, parity >> 1);
                 parity ^= 2;
+            } else if (!TAB && new_h) {
+                __syncthreads();    // this table is whole; the other one's readers are past it
             }
 #pragma unroll
-            for (int m = 0; m < E; ++m) v[m] = cmul(v[m], hs[half_index<N, E>(t, m)]);
+            for (int m = 0; m < E; ++m) v[m] = cmul(v[m], h[half_index<N, E>(t, m)]);
             fft_line_tr<float2, N, +1, kColEPT, 1, 1, T>(v, buf, t, tr);
-            if (count > 1 && t == 0) {    // the same for H
+            if (TAB && count > 1 && t == 0) {    // the same for H
                 __threadfence_block();
                 if (atomicAdd(reads + 1, 1u) % W == W - 1 && (l + 1 < count || more)) load_h(l + 1 < count ? l + 1 : 0);
             }
@@ -321,8 +332,21 @@ prop_cols_stream_kernel(PropArgs a, const __grid_constant__ CUtensorMap tm, int 
         __syncthreads();
     }
     if (!ok) {
-        for (int k = 0; k < 4; ++k) wait_tile(bar + (k >> 1), k & 1);
+        for (int k = 0; k < (TAB ? 4 : 2); ++k) wait_tile(bar + (k >> 1), k & 1);
     }
+}
+template <int N, bool TAB>
+cudaError_t launch_cols_stream(const PropArgs& a, const CUtensorMap& tm, cudaStream_t s) {
+    constexpr size_t smem = pcol_stream_smem<N, TAB>();
+    static_assert(smem <= kMaxSmem, "streamed column pass does not fit");
+    auto k = prop_cols_stream_kernel<N, TAB>;
+    cudaError_t e = set_smem(k, smem);
+    int blocks = 0;
+    if (e == cudaSuccess) e = walk_blocks(k, pcol_threads<N>(), smem, N / pcol_lines<N>(), a.lam.count, &blocks);
+    if (e != cudaSuccess) return e;
+    constexpr int align = pcol_lines<N>() == 2 ? 8 : 16;
+    return launch_pass<N>(a.lam.count, k, dim3(blocks), dim3(pcol_threads<N>()), smem, s, a, tm,
+                          (int)(reinterpret_cast<uintptr_t>(a.intensity) % align == 0));
 }
 
 // ---- lines of 8192 points: two half lines per team (fft_long) ----------------------------
@@ -975,19 +999,9 @@ cudaError_t launch_cols(const PropArgs& a, cudaStream_t s) {
                                 (int)(reinterpret_cast<uintptr_t>(a.intensity) % 16 == 0));
             } else {
                 if constexpr (!CONJ && col_stream<N>()) {
-                    static_assert(pcol_stream_smem<N>() <= kMaxSmem, "streamed column pass does not fit");
                     CUtensorMap tm;
-                    if (a.h && field_map(&tm, a.work, N, a.lam.count, pstrip<N>())) {
-                        auto k = prop_cols_stream_kernel<N>;
-                        cudaError_t e = set_smem(k, pcol_stream_smem<N>());
-                        int blocks = 0;
-                        if (e == cudaSuccess)
-                            e = walk_blocks(k, pcol_threads<N>(), pcol_stream_smem<N>(), N / pcol_lines<N>(), a.lam.count, &blocks);
-                        if (e != cudaSuccess) return e;
-                        constexpr int align = pcol_lines<N>() == 2 ? 8 : 16;
-                        return launch_pass<N>(a.lam.count, k, dim3(blocks), dim3(pcol_threads<N>()), pcol_stream_smem<N>(), s, a, tm,
-                                              (int)(reinterpret_cast<uintptr_t>(a.intensity) % align == 0));
-                    }
+                    if (field_map(&tm, a.work, N, a.lam.count, pstrip<N>()))
+                        return a.h ? launch_cols_stream<N, true>(a, tm, s) : launch_cols_stream<N, false>(a, tm, s);
                 }
                 constexpr size_t smem = pcol_smem<N, CONJ>();
                 cudaError_t e = set_smem(prop_cols_kernel<N, CONJ>, smem);
