@@ -464,6 +464,8 @@ void group_tables(TableArgs& ta, PropArgs& pa, const Carver& cg, float2* slot, c
     pa.h = ta.h;
 }
 
+double table_bytes(const TableArgs& ta) { return ta.count * (4.0 * ta.n + (ta.h ? 8.0 * transfer_entries(ta.n) : 0.0)); }
+
 // Propagate one wavelength group [l0, l0 + g) into the intensity map.
 int run_group(const scint_params* p, const double* phi, const double* lam, const double* wts,
               int l0, int g, float* intensity, int accumulate, Carver& c, float2* slot, const float2* tw,
@@ -488,7 +490,6 @@ int run_group(const scint_params* p, const double* phi, const double* lam, const
     pa.sf = ta.sf;
     pa.work = cg.take<float2>((size_t)field_slots(g) * n * n * 8);
     pa.scratch = n >= kSplitN ? cg.take<float>((size_t)n * n * 4) : nullptr;
-    group_tables(ta, pa, cg, slot, tw);
     pa.intensity = intensity;
     pa.accumulate = accumulate;
     pa.one = 1.0f;
@@ -496,8 +497,9 @@ int run_group(const scint_params* p, const double* phi, const double* lam, const
     int rc = plan_for(n, &pl);
     if (rc) return rc;
     const bool packed = pl.packed && g > 1 && packed_prop_supported(n, pl.points, pl.row_twiddles, pl.col_twiddles);
+    if (!packed) group_tables(ta, pa, cg, slot, tw);    // the packed passes evaluate H_x themselves
     const double nn = (double)n * n;
-    SCINT_LAUNCH(K_PROP_TABLES, 4.0 * g * n, 0.0, s, launch_prop_tables(ta, s));
+    SCINT_LAUNCH(K_PROP_TABLES, table_bytes(ta), 0.0, s, launch_prop_tables(ta, s));
     // rows: phi read once, one complex64 field written per wavelength; FFT_x + IFFT_x per row
     SCINT_LAUNCH(K_PROP_ROWS, 8.0 * nn + 8.0 * g * nn, 2.0 * g * n * fft_flops(n), s,
                  packed ? launch_prop_rows2(pa, pl.points, pl.row_twiddles, s) : launch_prop_rows(pa, false, s));
@@ -603,7 +605,7 @@ int conj_impl(const scint_params* p, const double* phi, const double* lambdas, c
         pa.conj.direct = direct ? 1 : 0;
         pa.conj.pattern = direct ? nullptr : cg.take<float>((size_t)gg * n * n * 4);
         ra.pattern = pa.conj.pattern;
-        SCINT_LAUNCH(K_PROP_TABLES, 4.0 * gg * n, 0.0, s, launch_prop_tables(ta, s));
+        SCINT_LAUNCH(K_PROP_TABLES, table_bytes(ta), 0.0, s, launch_prop_tables(ta, s));
         // one FFT per row and per column and wavelength
         SCINT_LAUNCH(K_CONJ_ROWS, 8.0 * nn + 8.0 * gg * nn, 1.0 * gg * n * fft_flops(n), s,
                      launch_prop_rows(pa, true, s));
@@ -830,7 +832,7 @@ int persist_propagate(const scint_params* const* params, const double* const* ph
         pa.intensity = intensities[i];
         pa.accumulate = 0;
         pa.one = 1.0f;
-        SCINT_LAUNCH(K_PROP_TABLES, 4.0 * n_lambda * nn, 0.0, s, launch_prop_tables(ta, s));
+        SCINT_LAUNCH(K_PROP_TABLES, table_bytes(ta), 0.0, s, launch_prop_tables(ta, s));
         SCINT_CUDA(launch_persist_args(pa, reinterpret_cast<PropArgs*>(ws + L.args) + i, s));
     }
     // phases: R(o0), R(o1), C(o0), R(o2), C(o1), ..., C(o_last)
@@ -1406,7 +1408,7 @@ int scint_lightcurve_adjoint(const scint_params* p, const double* phi, const dou
         pa.sf = ta.sf;
         pa.work = cg.take<float2>((size_t)field_slots(gg) * n * n * 8);
         if (n >= kSplitN) cg.take<float>((size_t)n * n * 4);    // the forward columns' scratch: not used here
-        group_tables(ta, pa, cg, slot, tw);
+        if (n >= kSplitN) group_tables(ta, pa, cg, slot, tw);    // the rows of smaller grids and the adjoint passes read none
         AdjArgs aa{};
         aa.n = n;
         aa.phi = phi;
@@ -1417,7 +1419,7 @@ int scint_lightcurve_adjoint(const scint_params* p, const double* phi, const dou
         aa.grad_phi = grad_phi;
         aa.accumulate = accumulate || l0 > 0;
         aa.lam = pa.lam;
-        SCINT_LAUNCH(K_PROP_TABLES, 4.0 * gg * n, 0.0, s, launch_prop_tables(ta, s));
+        SCINT_LAUNCH(K_PROP_TABLES, table_bytes(ta), 0.0, s, launch_prop_tables(ta, s));
         SCINT_LAUNCH(K_PROP_ROWS, 8.0 * nn + 8.0 * gg * nn, 2.0 * gg * n * fft_flops(n), s, launch_prop_rows(pa, false, s));
         SCINT_LAUNCH(K_ADJ_COLS, 16.0 * gg * nn + 4.0 * nn, 4.0 * gg * n * fft_flops(n), s, launch_adj_cols(aa, s));
         SCINT_LAUNCH(K_ADJ_ROWS, 8.0 * gg * nn + 8.0 * nn + (aa.accumulate ? 16.0 : 8.0) * nn,
