@@ -132,7 +132,7 @@ inline cudaError_t launch_next(void (*k)(KArgs...), dim3 grid, dim3 block, size_
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...);
 }
-// Passes that are launched so: grids of at most 65536 threads, a fifth of what the chip holds (N lines of
+// Passes that are launched so (the synthesis' above 512^2 are not, synth.cu): grids of at most 65536 threads, a fifth of what the chip holds (N lines of
 // N / 16 threads: to 1024^2), and at most eight times as many thread-wavelengths.  A longer pass hides its
 // own launch, and its waiting blocks take room from the one that works, this stream's or another's: with
 // every pass let in, 4096^2 at one wavelength went from 668 to 677 us, and with 1024^2 at 32 wavelengths
