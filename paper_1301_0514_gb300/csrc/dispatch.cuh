@@ -111,6 +111,9 @@ inline cudaError_t resident_blocks(K kernel, int threads, size_t smem, int* out)
 // before touching anything, then let the next one of the stream be set up.  In this order one kernel at
 // most waits on the chip; the other way round a whole chain of them piles up beside the one that works
 // (256^2 in 64-bit, 20 passes as a graph: 59 us a pass in this order, 165 in the other).
+// What the kernel before wrote is read by plain loads (or __ldcg, or TMA): the read-only path (__ldg) is for
+// memory that stands still from the reading kernel's start, which here lies before the wait.  What an
+// earlier kernel of the stream wrote stands still by then: the one before has waited for it.
 __device__ __forceinline__ void begin_after_previous() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -33,8 +33,8 @@ __global__ void __launch_bounds__(256) lightcurve_kernel(const __grid_constant__
     track_sample(a.tr[c], s, n, ix, iy, tx, ty);
     const int ix1 = (ix + 1) & (n - 1), iy1 = (iy + 1) & (n - 1);
     const float* I = a.intensity;
-    const float i00 = __ldg(I + (size_t)iy * n + ix), i01 = __ldg(I + (size_t)iy * n + ix1);
-    const float i10 = __ldg(I + (size_t)iy1 * n + ix), i11 = __ldg(I + (size_t)iy1 * n + ix1);
+    const float i00 = I[(size_t)iy * n + ix], i01 = I[(size_t)iy * n + ix1];
+    const float i10 = I[(size_t)iy1 * n + ix], i11 = I[(size_t)iy1 * n + ix1];
     const float top = fmaf(tx, i01 - i00, i00);
     const float bot = fmaf(tx, i11 - i10, i10);
     a.curves[(size_t)c * a.n_samples + s] = fmaf(ty, bot - top, top);

@@ -46,10 +46,10 @@ SCINT_DEV void prop_rows_body(const PropArgs& a, int bid, int tid, float2* smem3
             const unsigned long long cy = chirp_turns(C, y, N);
 #pragma unroll
             for (int m = 0; m < E; ++m)
-                v[m] = unit_phasor(P[m * T], S, cy + chirp_turns(C, t + m * T, N)) * (sfy * __ldg(sf + t + m * T));
+                v[m] = unit_phasor(P[m * T], S, cy + chirp_turns(C, t + m * T, N)) * (sfy * sf[t + m * T]);
         } else {
 #pragma unroll
-            for (int m = 0; m < E; ++m) v[m] = unit_phasor(P[m * T], S) * (sfy * __ldg(sf + t + m * T));
+            for (int m = 0; m < E; ++m) v[m] = unit_phasor(P[m * T], S) * (sfy * sf[t + m * T]);
         }
         if constexpr (TWM == 2) fft_line_tr<float2, N, -1, 16, 1, 1, SUB>(v, buf, t, tr);
         else fft_line<float2, N, -1, 16, 1, TWM, 1, 1, SUB>(v, buf, t, twp);

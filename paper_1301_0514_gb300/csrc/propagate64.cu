@@ -51,12 +51,12 @@ __global__ void prop64_tables_kernel(Prop64Args a, double2* h, double* sf) {
 }
 template <int N, bool TAB>
 SCINT_DEV double2 transfer_of(const Prop64Args& a, int i) {
-    if constexpr (TAB) return __ldg(a.h + (i <= N / 2 ? i : N - i));
+    if constexpr (TAB) return a.h[i <= N / 2 ? i : N - i];
     else return transfer64(a, i);
 }
 template <int N, bool TAB>
 SCINT_DEV double taper_of(const Prop64Args& a, int i) {
-    if constexpr (TAB) return __ldg(a.sf + (i < N / 2 ? i : N - 1 - i));
+    if constexpr (TAB) return a.sf[i < N / 2 ? i : N - 1 - i];
     else return taper64(i, N, a.margin_px);
 }
 
@@ -120,7 +120,13 @@ cudaError_t launch_passes64(const Prop64Args& a, cudaStream_t s) {
     if (e == cudaSuccess) e = set_smem(prop64_cols_kernel<N, TAB>, p64_smem<N>());
     if (e != cudaSuccess) return e;
     constexpr int T = FftPlan<N, p64_ept<N>()>::T;
-    if ((e = launch_pass<N>(1, prop64_rows_kernel<N, TAB>, dim3(N), dim3(T), p64_smem<N>(), s, a)) != cudaSuccess) return e;
+    if constexpr (TAB) {
+        e = launch_pass<N>(1, prop64_rows_kernel<N, TAB>, dim3(N), dim3(T), p64_smem<N>(), s, a);
+    } else {    // the kernel before may be the one that fills the twiddles (begin_after_previous)
+        prop64_rows_kernel<N, TAB><<<N, T, p64_smem<N>(), s>>>(a);
+        e = cudaGetLastError();
+    }
+    if (e != cudaSuccess) return e;
     return launch_pass<N>(1, prop64_cols_kernel<N, TAB>, dim3(N), dim3(T), p64_smem<N>(), s, a);
 }
 
