@@ -33,6 +33,10 @@ def decorrelation(p: _lib.ScintParams, intensity: torch.Tensor, tracks, separati
     each separation: a (n_tracks, n_separations) float64 device tensor."""
     base = np.asarray(tracks, dtype=np.float64).reshape(-1, 4)
     sep = np.asarray(separations_px, dtype=np.float64)
+    if len(base) == 0:
+        raise ValueError("tracks must hold at least one track")
+    if sep.ndim != 1:
+        raise ValueError("separations_px must be a list of separations, the same for every track")
     # parallel_tracks of every base track at once
     sin, cos = (np.array([f(th) for th in base[:, 2]])[:, None] for f in (math.sin, math.cos))
     all_tracks = np.empty((len(base), len(sep), 4))
