@@ -209,8 +209,12 @@ def _stream(stream) -> int:
     if stream is None:
         if not torch.cuda.is_initialized():
             torch.cuda.init()
-        # the handle of the current device's current stream, without building a Stream object around it
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        # the handle of the current device's current stream, without building a Stream object around it where
+        # PyTorch has the (internal) call for that
+        try:
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        except AttributeError:
+            stream = torch.cuda.current_stream()
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
