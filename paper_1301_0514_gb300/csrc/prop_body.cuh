@@ -15,7 +15,6 @@ namespace scint {
 template <int N, bool CONJ, int SUB = 0>
 SCINT_DEV void prop_rows_body(const PropArgs& a, int bid, int tid, float2* smem32) {
     using Pl = FftPlan<N>;
-    constexpr int TWM = prow_twm<N>();
     constexpr int T = Pl::T, E = Pl::E, B = prow_lines<N>(), W = pstrip<N>(), BUFL = Pl::BUF;
     const int team = tid / T, t = tid % T;    // line of the block, index in its team
     const int y = bid * B + team;
@@ -23,11 +22,8 @@ SCINT_DEV void prop_rows_body(const PropArgs& a, int bid, int tid, float2* smem3
     // fixed-point phase of this thread's pixels, kept in shared memory across the
     // wavelength loop (each thread reads back only the entries it wrote)
     long long* P = reinterpret_cast<long long*>(smem32 + B * BUFL) + team * N + t;
-    float2* tws = smem32 + B * BUFL + B * N;    // shared twiddle table (after P, 8 B per entry)
-    const float2* twp = TWM == 1 ? tws : a.tw;
     TwiddleRegs<float2, N, 16> tr;
-    if constexpr (TWM == 2) tr.load(a.tw, t);
-    else if constexpr (TWM == 1) fill_twiddle_table<float2, N>(tws, a.tw, tid, prow_threads<N>());
+    tr.load(a.tw, t);
     phases_fixed<E>([&](int m) { return a.phi[(size_t)y * N + t + m * T]; }, [&](int m, long long p) { P[m * T] = p; });
     team_sync<SUB>();
 
@@ -51,14 +47,12 @@ SCINT_DEV void prop_rows_body(const PropArgs& a, int bid, int tid, float2* smem3
 #pragma unroll
             for (int m = 0; m < E; ++m) v[m] = unit_phasor(P[m * T], S) * (sfy * sf[t + m * T]);
         }
-        if constexpr (TWM == 2) fft_line_tr<float2, N, -1, 16, 1, 1, SUB>(v, buf, t, tr);
-        else fft_line<float2, N, -1, 16, 1, TWM, 1, 1, SUB>(v, buf, t, twp);
+        fft_line_tr<float2, N, -1, 16, 1, 1, SUB>(v, buf, t, tr);
         if constexpr (!CONJ) {
             const unsigned long long hc = a.lam.h_fx[l];
 #pragma unroll
             for (int m = 0; m < E; ++m) v[m] = cmul(v[m], transfer_fast(hc, signed_index<N, E>(t, m)));
-            if constexpr (TWM == 2) fft_line_tr<float2, N, +1, 16, 1, 1, SUB>(v, buf, t, tr);
-            else fft_line<float2, N, +1, 16, 1, TWM, 1, 1, SUB>(v, buf, t, twp);
+            fft_line_tr<float2, N, +1, 16, 1, 1, SUB>(v, buf, t, tr);
         }
         float2* dst = a.work + (size_t)l * N * N;
 #pragma unroll

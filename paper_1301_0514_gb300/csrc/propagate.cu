@@ -60,13 +60,8 @@ cudaError_t launch_prop_tables(const TableArgs& a, cudaStream_t s) {
     return launch_next(prop_tables_kernel, grid, dim3(256), 0, s, a);
 }
 
-// Resident row blocks per SM the register budget is set for (build-time choice, 2 by default;
-// 3 caps the pass at 80 registers).
-#ifndef SCINT_ROW_MIN_BLOCKS
-#define SCINT_ROW_MIN_BLOCKS 2
-#endif
 template <int N, bool CONJ>
-__global__ void __launch_bounds__(prow_threads<N>(), (prow_threads<N>() <= 256 ? SCINT_ROW_MIN_BLOCKS : 1))
+__global__ void __launch_bounds__(prow_threads<N>(), (prow_threads<N>() <= 256 ? 2 : 1))
 prop_rows_kernel(PropArgs a) {
     extern __shared__ float2 smem32[];
     begin_pass<N>();
@@ -115,7 +110,6 @@ __global__ void __launch_bounds__(prow_threads<N>(), (prow_threads<N>() <= 256 ?
 prop_rows_stream_kernel(PropArgs a, int bulk) {
     using Pl = FftPlan<N>;
     constexpr int T = Pl::T, E = Pl::E, B = prow_lines<N>(), W = pstrip<N>(), BUFL = Pl::BUF;
-    static_assert(prow_twm<N>() == 2, "register twiddle bases");
     extern __shared__ float2 smem32[];
     begin_pass<N>();
     const int team = threadIdx.x / T, t = threadIdx.x % T;

@@ -4,22 +4,8 @@
 #include "fft.cuh"
 #include "kernels.cuh"
 
-// Twiddle source of the propagation FFTs (build-time tuning choices, measured on
-// GB300 at 1024^2-4096^2 x 32 wavelengths): 1 = per-block shared table,
-// 2 = per-thread register bases + products.  The row pass is faster with
-// register bases (its 2 blocks/SM keep the shared-memory pipe busy), the column
-// pass with the shared table (its single block/SM has registers to spare).
-#ifndef SCINT_ROW_TWIDDLES
-#define SCINT_ROW_TWIDDLES 2
-#endif
-#ifndef SCINT_COL_TWIDDLES
-#define SCINT_COL_TWIDDLES 1
-#endif
-
 namespace scint {
 
-constexpr int kRowTw = SCINT_ROW_TWIDDLES;
-constexpr int kColTw = SCINT_COL_TWIDDLES;
 constexpr int kColEPT = 16;   // values per thread in the column passes
 constexpr size_t kMaxSmem = 227 * 1024;
 
@@ -28,7 +14,6 @@ constexpr size_t kMaxSmem = 227 * 1024;
 // propagate.cu, adj_*_split_kernel in adjoint.cu): each block transforms one parity
 // as a whole N/2-point line.  The kernels below are the unsplit passes.
 template <int N> __host__ __device__ constexpr int pcs() { return N >= kSplitN ? 2 : 1; }
-template <int N> __host__ __device__ constexpr int prow_twm() { return kRowTw; }
 
 // rows per row-pass block, columns per column-pass block (all lines of a block
 // are transformed together); threads are per block
@@ -49,8 +34,7 @@ template <int N> __host__ __device__ constexpr int pstrip() { return pcol_lines<
 
 template <int N> constexpr size_t ptws_bytes(int twm) { return twm == 1 ? (size_t)FftPlan<N>::TWS * sizeof(float2) : 0; }
 template <int N> constexpr size_t prow_smem() {
-    return (size_t)prow_lines<N>() * (FftPlan<N>::BUF * sizeof(float2) + N * sizeof(long long)) +
-           ptws_bytes<N>(prow_twm<N>());
+    return (size_t)prow_lines<N>() * (FftPlan<N>::BUF * sizeof(float2) + N * sizeof(long long));
 }
 // Transfer-function column blocks of these sizes give each column a team of threads with a barrier and a line buffer
 // of its own, so that one column's line exchanges run beside another's butterflies; in smaller
@@ -61,9 +45,10 @@ template <int N> __host__ __device__ constexpr bool col_teams() { return N >= 51
 template <int N> __host__ __device__ constexpr size_t pcol_base_bytes() {
     return (size_t)pcol_lines<N>() * FftPlan<N>::BUF * sizeof(float2);
 }
+// Twiddles of the column passes (fft.cuh): register bases and their products (2) in the teams, which share no barrier
+// that a table's making could use, and where the table does not fit; else the block's shared table (1).  The row passes take bases.
 template <int N, bool CONJ> __host__ __device__ constexpr int pcol_twm() {
-    return !CONJ && col_teams<N>() ? 2 : (kColTw == 1 && pcol_base_bytes<N>() + (size_t)FftPlan<N>::TWS * sizeof(float2) > kMaxSmem
-                ? 2 : kColTw);
+    return (!CONJ && col_teams<N>()) || pcol_base_bytes<N>() + (size_t)FftPlan<N>::TWS * sizeof(float2) > kMaxSmem ? 2 : 1;
 }
 // Below 512 a block's columns evaluate H_x once per block and wavelength into shared memory: with two tables there,
 // and no barrier of their own, that is less than the latency of a table's loads behind the forward transform, which few
