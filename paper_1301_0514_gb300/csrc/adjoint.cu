@@ -48,9 +48,17 @@ cudaError_t launch_lightcurve_adjoint(const CurveAdjArgs& a, cudaStream_t s) {
 }
 
 // ---- adjoint column pass ----------------------------------------------------------
-// buffers, the g_I columns (in place of the accumulator) and the twiddle table
+// H_y takes the values that the forward columns take (transfer_signed), so that this is the adjoint of that pass: from a
+// half table per wavelength, evaluated by the block into shared memory, two tables in turn (as in prop_cols_body);
+// at 8192 element by element, since the load/store pipe of its one column per block has no room for the table
+// (one wavelength 1.58 ms with it, 1.25 without; 4096^2 0.913 and 0.909 ms for five, 2048^2 0.211 and 0.221).
+// From 2048 on as many blocks as are resident walk the columns, so that the twiddle table is filled once per block
+// (one wavelength: 4096^2 0.241 -> 0.216 ms, 8192^2 1.48 -> 1.25).
+template <int N> __host__ __device__ constexpr bool acol_tables() { return N < 8192; }
+// line buffers, the twiddle table and the two tables of H_y/N (the g_I columns live in registers)
 template <int N> constexpr size_t acol_smem() {
-    return (size_t)pcol_lines<N>() * FftPlan<N, kColEPT>::BUF * sizeof(float2) + (size_t)FftPlan<N>::TWS * sizeof(float2);
+    return ((size_t)pcol_lines<N>() * FftPlan<N, kColEPT>::BUF + FftPlan<N>::TWS + (acol_tables<N>() ? 2 * own_entries<N>() : 0)) *
+           sizeof(float2);
 }
 
 template <int N>
@@ -61,40 +69,55 @@ adj_cols_kernel(AdjArgs a) {
     constexpr int T = Pl::T, E = Pl::E, W = pcol_lines<N>(), WL = pstrip<N>(), BUFL = Pl::BUF;
     extern __shared__ float2 smem32[];
     const int w = threadIdx.x % W, t = threadIdx.x / W;
-    const int x0 = blockIdx.x * W;
-    const int x = x0 + w;
     float2* buf = smem32 + w;
     float gi[E];                                  // g_I of this column (own entries), in registers
     float2* tws = smem32 + W * BUFL;
-    const float2* twp = TWM == 1 ? tws : a.tw;
-    if constexpr (TWM == 1) fill_twiddle_table<float2, N>(tws, a.tw, threadIdx.x, blockDim.x);
-#pragma unroll
-    for (int m = 0; m < E; ++m) gi[m] = a.grad_map[(size_t)(t + m * T) * N + x];
+    float2* own_h = tws + FftPlan<N>::TWS;
+    fill_twiddle_table<float2, N>(tws, a.tw, threadIdx.x, blockDim.x);
     __syncthreads();
+    int turn = 0;    // which of the two tables
 #pragma unroll 1
-    for (int l = 0; l < a.lam.count; ++l) {
-        float2* f = a.work + (size_t)l * N * N + (size_t)(x0 / WL) * N * WL + (x0 % WL);
-        const unsigned long long hc = a.lam.h_fx[l];    // H_y from its fixed-point phase
-        float2 v[E];
+    for (int x0 = blockIdx.x * W; x0 < N; x0 += gridDim.x * W) {
 #pragma unroll
-        for (int m = 0; m < E; ++m) v[m] = f[(size_t)(t + m * T) * WL + w];
-        fft_line<float2, N, -1, kColEPT, W, TWM>(v, buf, t, twp);
+        for (int m = 0; m < E; ++m) gi[m] = a.grad_map[(size_t)(t + m * T) * N + x0 + w];
+#pragma unroll 1
+        for (int l = 0; l < a.lam.count; ++l) {
+            float2* f = a.work + (size_t)l * N * N + (size_t)(x0 / WL) * N * WL + (x0 % WL);
+            if (acol_tables<N>() && (a.lam.count > 1 || x0 == (int)blockIdx.x * W)) {
+                turn ^= 1;
+                for (int i = threadIdx.x; i < own_entries<N>(); i += pcol_threads<N>())
+                    own_h[turn * own_entries<N>() + i] = transfer_signed(a.lam.h_fx[l], i) * (1.0f / N);
+            }
+            const float2* h = own_h + turn * own_entries<N>();
+            const unsigned long long hc = a.lam.h_fx[l];
+            auto transfer = [&](int m) {
+                if constexpr (acol_tables<N>()) return h[half_index<N, E>(t, m)];
+                else return transfer_signed(hc, signed_index<N, E>(t, m)) * (1.0f / N);
+            };
+            float2 v[E];
 #pragma unroll
-        for (int m = 0; m < E; ++m) v[m] = cmul(v[m], transfer_at(hc, t + m * T, N));
-        fft_line<float2, N, +1, kColEPT, W, TWM>(v, buf, t, twp);          // A_out of this column
-        const float c2w = 2.0f * a.lam.weight[l];
+            for (int m = 0; m < E; ++m) v[m] = f[(size_t)(t + m * T) * WL + w];
+            fft_line<float2, N, -1, kColEPT, W, TWM>(v, buf, t, tws);
+            // the table was written before the transform's barriers; its turn comes again after the next one's
+            if constexpr (Pl::NSTAGE == 1) __syncthreads();
 #pragma unroll
-        for (int m = 0; m < E; ++m) v[m] = v[m] * (c2w * gi[m]);          // G_out
-        fft_line<float2, N, -1, kColEPT, W, TWM>(v, buf, t, twp);
+            for (int m = 0; m < E; ++m) v[m] = cmul(v[m], transfer(m));
+            fft_line<float2, N, +1, kColEPT, W, TWM>(v, buf, t, tws);          // A_out of this column
+            const float c2w = 2.0f * a.lam.weight[l];
 #pragma unroll
-        for (int m = 0; m < E; ++m) v[m] = cmulc(v[m], transfer_at(hc, t + m * T, N));
-        fft_line<float2, N, +1, kColEPT, W, TWM>(v, buf, t, twp);          // P_y^H G_out
+            for (int m = 0; m < E; ++m) v[m] = v[m] * (c2w * gi[m]);          // G_out
+            fft_line<float2, N, -1, kColEPT, W, TWM>(v, buf, t, tws);
 #pragma unroll
-        for (int m = 0; m < E; ++m) f[(size_t)(t + m * T) * WL + w] = v[m];
+            for (int m = 0; m < E; ++m) v[m] = cmulc(v[m], transfer(m));
+            fft_line<float2, N, +1, kColEPT, W, TWM>(v, buf, t, tws);          // P_y^H G_out
+#pragma unroll
+            for (int m = 0; m < E; ++m) f[(size_t)(t + m * T) * WL + w] = v[m];
+        }
     }
 }
 
 // ---- adjoint row pass --------------------------------------------------------------
+// H_x as the forward rows evaluate it (transfer_fast's bits).
 // buffers and fixed-point phases (the g_phi sums and the twiddle bases live in registers)
 template <int N> constexpr size_t arow_smem() {
     return (size_t)prow_lines<N>() * (FftPlan<N>::BUF * sizeof(float2) + N * sizeof(long long));
@@ -147,14 +170,22 @@ adj_rows_kernel(AdjArgs a) {
 
 // ---- N = 16384: the adjoint passes on the radix-2 cluster split --------------------
 // Block r of a cluster transforms the parity-r half of every line as a whole 8192-point
-// line in its own shared memory (fft.cuh: split_dif, split_combine), as the forward
-// passes do.  The column pass chains two transform pairs per wavelength: after the first
+// line in its own shared memory (fft.cuh: split_dif, split_combine; the forward passes hold it as two
+// half lines instead, the values of H are theirs).  The column pass chains two transform pairs per wavelength: after the first
 // (A_out) each block holds G_out at its quarter of the outputs, n and n + N/2, i.e. both
 // halves of the decimation-in-frequency pairs for those n; it keeps its parity's a_n or
 // b_n and hands the other to its partner through shared memory.  Grids are persistent.
 template <int N> __host__ __device__ constexpr int asplit_threads() { return FftPlan<N / 2>::T; }
+// H/N of the column pass at the frequencies 2j + r, j = 0..N/4, in shared memory (one wavelength 6.42 ms, 7.12 evaluated
+// element by element; with the hardware sine of a whole turn 6.94): the other half of a parity mirrors them (f = 2k + r with k >= N/4 is
+// 2 (k - N/2) + r, whose magnitude is 2 (N/2 - k) - r)
+template <int N> __host__ __device__ constexpr int asplit_entries() { return N / 4 + 1; }
+template <int N> SCINT_DEV int asplit_index(int t, int m, int r) {
+    const int k = t + m * FftPlan<N / 2>::T;
+    return 2 * m >= FftPlan<N / 2>::E ? N / 2 - k - r : k;
+}
 template <int N> constexpr size_t asplit_col_smem() {
-    return (size_t)(FftPlan<N / 2>::BUF + FftPlan<N / 2>::TWS) * sizeof(float2);
+    return (size_t)(FftPlan<N / 2>::BUF + FftPlan<N / 2>::TWS + asplit_entries<N>()) * sizeof(float2);
 }
 template <int N> constexpr size_t asplit_row_smem() {
     return (size_t)FftPlan<N / 2>::BUF * sizeof(float2) + (size_t)N * sizeof(long long);
@@ -170,6 +201,7 @@ __global__ void __launch_bounds__(asplit_threads<N>(), 1) adj_cols_split_kernel(
     const int t = threadIdx.x;
     float2* buf = smem32;
     float2* tws = smem32 + Pl::BUF;
+    float2* h = tws + Pl::TWS;
     fill_twiddle_table<float2, H2>(tws, a.tw, t, T, 2);
     cluster_arrive();    // the first wait also publishes the twiddle table to the block
 #pragma unroll 1
@@ -184,7 +216,6 @@ __global__ void __launch_bounds__(asplit_threads<N>(), 1) adj_cols_split_kernel(
 #pragma unroll 1
         for (int l = 0; l < a.lam.count; ++l) {
             float2* f = a.work + (size_t)l * N * N + (size_t)(x / WL) * N * WL + (x % WL);
-            const unsigned long long hc = a.lam.h_fx[l];    // H_y from its fixed-point phase
             float2 v[E];
 #pragma unroll
             for (int m = 0; m < E; ++m) {
@@ -192,9 +223,13 @@ __global__ void __launch_bounds__(asplit_threads<N>(), 1) adj_cols_split_kernel(
                 v[m] = split_dif(f[(size_t)e * WL], f[(size_t)(e + H2) * WL], r, e, a.tw);
             }
             cluster_wait();
+            // the block is past its last use of the former table: a barrier stands after every one (split_combine)
+            if (a.lam.count > 1 || x == (int)blockIdx.x / 2) {
+                for (int i = t; i < asplit_entries<N>(); i += T) h[i] = transfer_signed(a.lam.h_fx[l], 2 * i + r) * (1.0f / N);
+            }
             fft_line<float2, H2, -1, 16, 1, 1, 1>(v, buf, t, tws);
 #pragma unroll
-            for (int m = 0; m < E; ++m) v[m] = cmul(v[m], transfer_at(hc, 2 * (t + m * T) + r, N));
+            for (int m = 0; m < E; ++m) v[m] = cmul(v[m], h[asplit_index<N>(t, m, r)]);
             fft_line<float2, H2, +1, 16, 1, 1, 1>(v, buf, t, tws);
             const float c2w = 2.0f * a.lam.weight[l];
             float2 gq[E];                                    // G_out at n and n + N/2
@@ -224,7 +259,7 @@ __global__ void __launch_bounds__(asplit_threads<N>(), 1) adj_cols_split_kernel(
             line_sync<2>();                                  // the partner is done with this block's buffer
             fft_line<float2, H2, -1, 16, 1, 1, 1>(v, buf, t, tws);
 #pragma unroll
-            for (int m = 0; m < E; ++m) v[m] = cmulc(v[m], transfer_at(hc, 2 * (t + m * T) + r, N));
+            for (int m = 0; m < E; ++m) v[m] = cmulc(v[m], h[asplit_index<N>(t, m, r)]);
             fft_line<float2, H2, +1, 16, 1, 1, 1>(v, buf, t, tws);
             // P_y^H G_out over the field (the partner read this column before its first exchange)
             split_combine<float2, H2>(v, buf, t, r, a.tw, [&](int, int n, float2 y0, float2 y1) {
@@ -265,7 +300,7 @@ __global__ void __launch_bounds__(asplit_threads<N>(), 1) adj_rows_split_kernel(
 #pragma unroll 1
         for (int l = 0; l < a.lam.count; ++l) {
             const float2* f = a.work + (size_t)l * N * N;
-            const unsigned long long hc = a.lam.h_fx[l];    // H_x from its fixed-point phase
+            const unsigned long long hc = a.lam.h_fx[l];    // H_x, evaluated (2-4 % slower from the group's table)
             float2 v[E];
 #pragma unroll
             for (int m = 0; m < E; ++m) {
@@ -275,7 +310,7 @@ __global__ void __launch_bounds__(asplit_threads<N>(), 1) adj_rows_split_kernel(
             cluster_wait();
             fft_line_tr<float2, H2, -1, 16, 1>(v, buf, t, tr);
 #pragma unroll
-            for (int m = 0; m < E; ++m) v[m] = cmulc(v[m], transfer_at(hc, 2 * (t + m * T) + r, N));
+            for (int m = 0; m < E; ++m) v[m] = cmulc(v[m], transfer_signed(hc, 2 * signed_index<H2, E>(t, m) + r) * (1.0f / N));
             fft_line_tr<float2, H2, +1, 16, 1>(v, buf, t, tr);     // G_in of this row
             const unsigned long long S = a.lam.scale_fx[l];
             const float s_l = a.lam.scale[l];
@@ -313,12 +348,17 @@ cudaError_t launch_adj_cols(const AdjArgs& a, cudaStream_t s) {
             if (e != cudaSuccess) return e;
             return launch_k(adj_cols_split_kernel<N>, 2, dim3(2 * std::min(nc, N)), dim3(asplit_threads<N>()),
                             asplit_col_smem<N>(), s, a);
-        } else if constexpr (acol_smem<N>() > kMaxSmem || arow_smem<N>() > kMaxSmem) {
-            return cudaErrorNotSupported;
         } else {
+            static_assert(acol_smem<N>() <= kMaxSmem, "adjoint column pass does not fit");
             cudaError_t e = set_smem(adj_cols_kernel<N>, acol_smem<N>());
             if (e != cudaSuccess) return e;
-            adj_cols_kernel<N><<<N / pcol_lines<N>(), pcol_threads<N>(), acol_smem<N>(), s>>>(a);
+            int blocks = N / pcol_lines<N>();
+            if constexpr (N >= 2048) {
+                int resident = 0;
+                if ((e = resident_blocks(adj_cols_kernel<N>, pcol_threads<N>(), acol_smem<N>(), &resident)) != cudaSuccess) return e;
+                blocks = std::min(blocks, resident);
+            }
+            adj_cols_kernel<N><<<blocks, pcol_threads<N>(), acol_smem<N>(), s>>>(a);
             return cudaGetLastError();
         }
     });
@@ -336,9 +376,8 @@ cudaError_t launch_adj_rows(const AdjArgs& a, cudaStream_t s) {
             if (e != cudaSuccess) return e;
             return launch_k(adj_rows_split_kernel<N>, 2, dim3(2 * std::min(nc, N)), dim3(asplit_threads<N>()),
                             asplit_row_smem<N>(), s, a);
-        } else if constexpr (acol_smem<N>() > kMaxSmem || arow_smem<N>() > kMaxSmem) {
-            return cudaErrorNotSupported;
         } else {
+            static_assert(arow_smem<N>() <= kMaxSmem, "adjoint row pass does not fit");
             cudaError_t e = set_smem(adj_rows_kernel<N>, arow_smem<N>());
             if (e != cudaSuccess) return e;
             adj_rows_kernel<N><<<N / prow_lines<N>(), prow_threads<N>(), arow_smem<N>(), s>>>(a);
