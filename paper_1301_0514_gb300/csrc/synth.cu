@@ -68,8 +68,7 @@ cudaError_t launch_twiddles64(double2* tw, int n, cudaStream_t s) {
 }
 
 // Lines per block (all transformed together); N = 16384 lines (256 KB in
-// double-float) go to a cluster of two blocks (the split kernels below).
-template <int N> __host__ __device__ constexpr int synth_cs() { return N >= kSplitN ? 2 : 1; }
+// double-float) go to a cluster of two blocks (the split kernels below), for which none of the unsplit shapes hold.
 template <int N> __host__ __device__ constexpr int synth_tile_lines() { return N >= kTile64 ? 1 : (kTile64 / N < N ? kTile64 / N : N); }
 // Rows per row-pass block: the tile, but no more than leaves about two blocks per SM (the
 // N/2 + 1 rows over 304 blocks).  Up to N = 512 every bin is drawn in FP64, whose pipe is
@@ -84,7 +83,7 @@ template <int N> __host__ __device__ constexpr int synth_lines() {
 // (by events: draw and rows 38 -> 28 us, columns 16 -> 8 us; at 512^2 95 -> 64 and 19 -> 9 us).
 template <int N> __host__ __device__ constexpr int synth_ept() { return N >= 64 && N <= kDrawN ? 4 : 16; }
 template <int N> using SynthPlan = FftPlan<N, synth_ept<N>()>;
-template <int N> __host__ __device__ constexpr int synth_threads() { return synth_lines<N>() * SynthPlan<N>::T / synth_cs<N>(); }
+template <int N> __host__ __device__ constexpr int synth_threads() { return synth_lines<N>() * SynthPlan<N>::T; }
 // column pass: complex lines (each two real output columns) per block, the tile but no more than
 // leaves 128 blocks (two at N = 4096, 139 KB of shared memory: 0.236 -> 0.201 ms per 4096^2 pass
 // against one)
@@ -92,9 +91,9 @@ template <int N> __host__ __device__ constexpr int synth_col_lines() {
     constexpr int spread = N / 256 > 1 ? N / 256 : 1;
     return N == 4096 ? 2 : (synth_tile_lines<N>() < spread ? synth_tile_lines<N>() : spread);
 }
-template <int N> __host__ __device__ constexpr int synth_col_threads() { return synth_col_lines<N>() * SynthPlan<N>::T / synth_cs<N>(); }
-template <int N> constexpr size_t synth_smem() { return (size_t)synth_lines<N>() * FftPlan<N>::BUF * sizeof(dfc) / synth_cs<N>(); }
-template <int N> constexpr size_t synth_col_smem() { return (size_t)synth_col_lines<N>() * FftPlan<N>::BUF * sizeof(dfc) / synth_cs<N>(); }
+template <int N> __host__ __device__ constexpr int synth_col_threads() { return synth_col_lines<N>() * SynthPlan<N>::T; }
+template <int N> constexpr size_t synth_smem() { return (size_t)synth_lines<N>() * FftPlan<N>::BUF * sizeof(dfc); }
+template <int N> constexpr size_t synth_col_smem() { return (size_t)synth_col_lines<N>() * FftPlan<N>::BUF * sizeof(dfc); }
 
 // The intermediate G(ky, x), ky = 0..N/2, is stored in strips of one column pair
 // p = x/2 (synth_strip<N>() values each), so that a column pass reads contiguous memory:
@@ -184,7 +183,7 @@ __global__ void __launch_bounds__(synth_threads<N>())
 synth_rows_kernel(SynthArgs a) {
     begin_pass<N>();
     using Pl = SynthPlan<N>;
-    static_assert(synth_cs<N>() == 1, "unsplit rows");
+    static_assert(N < kSplitN, "unsplit rows");
     constexpr int T = Pl::T, E = Pl::E, B = synth_lines<N>();
     extern __shared__ dfc smem_df[];
     const int team = threadIdx.x / T, t = threadIdx.x % T;
@@ -224,7 +223,7 @@ __global__ void __launch_bounds__(synth_col_threads<N>())
 synth_cols_kernel(SynthArgs a) {
     begin_pass<N>();
     using Pl = SynthPlan<N>;
-    static_assert(synth_cs<N>() == 1, "unsplit columns");
+    static_assert(N < kSplitN, "unsplit columns");
     constexpr int T = Pl::T, E = Pl::E, W = synth_col_lines<N>();
     extern __shared__ dfc smem_df[];
     const int w = threadIdx.x % W;
@@ -357,40 +356,36 @@ template <bool ROWS>
 cudaError_t launch_synth_pass(const SynthArgs& a, cudaStream_t s) {
     return dispatch_n(a.n, [&](auto nc) -> cudaError_t {
         constexpr int N = decltype(nc)::value;
-        if constexpr (synth_smem<N>() > 227 * 1024) {
-            return cudaErrorNotSupported;
-        } else {
-            constexpr int CS = synth_cs<N>();
-            cudaError_t e;
-            if constexpr (CS == 2) {
-                static_assert(synth_split_smem<N>() <= 227 * 1024, "split synthesis pass does not fit");
-                auto k = ROWS ? synth_rows_split_kernel<N> : synth_cols_split_kernel<N>;
-                int nc = 0;
-                if ((e = set_smem(k, synth_split_smem<N>())) != cudaSuccess) return e;
-                if ((e = active_clusters(k, 2, synth_split_threads<N>(), synth_split_smem<N>(), &nc)) != cudaSuccess)
-                    return e;
-                const int lines = ROWS ? N / 2 + 1 : N / 2;
-                if (!ROWS && !a.pairs) return cudaErrorInvalidValue;
-                e = launch_k(k, 2, dim3(2 * std::min(nc, lines)), dim3(synth_split_threads<N>()),
-                             synth_split_smem<N>(), s, a);
-                if (e != cudaSuccess || ROWS) return e;
-                return launch_pairs_to_rows(a.pairs, a.phi, N, s);
-            } else if (ROWS) {
-                if ((e = set_smem(synth_rows_kernel<N>, synth_smem<N>())) != cudaSuccess) return e;
-                if constexpr (N <= kDrawN) {
-                    if (!a.drawn) return cudaErrorInvalidValue;
-                    e = launch_next(synth_draw_kernel, dim3((draw_bins(N) + kDrawThreads - 1) / kDrawThreads),
-                                    dim3(kDrawThreads), 0, s, a);
-                    if (e != cudaSuccess) return e;
-                }
-                const int rows = N / 2 + 1;
-                return launch_synth<N>(synth_rows_kernel<N>, dim3((rows + synth_lines<N>() - 1) / synth_lines<N>()),
-                                   dim3(synth_threads<N>()), synth_smem<N>(), s, a);
-            } else {
-                if ((e = set_smem(synth_cols_kernel<N>, synth_col_smem<N>())) != cudaSuccess) return e;
-                return launch_synth<N>(synth_cols_kernel<N>, dim3(N / (2 * synth_col_lines<N>())),
-                                   dim3(synth_col_threads<N>()), synth_col_smem<N>(), s, a);
+        cudaError_t e;
+        if constexpr (N >= kSplitN) {
+            static_assert(synth_split_smem<N>() <= 227 * 1024, "split synthesis pass does not fit");
+            auto k = ROWS ? synth_rows_split_kernel<N> : synth_cols_split_kernel<N>;
+            int nc = 0;
+            if ((e = set_smem(k, synth_split_smem<N>())) != cudaSuccess) return e;
+            if ((e = active_clusters(k, 2, synth_split_threads<N>(), synth_split_smem<N>(), &nc)) != cudaSuccess)
+                return e;
+            const int lines = ROWS ? N / 2 + 1 : N / 2;
+            if (!ROWS && !a.pairs) return cudaErrorInvalidValue;
+            e = launch_k(k, 2, dim3(2 * std::min(nc, lines)), dim3(synth_split_threads<N>()),
+                         synth_split_smem<N>(), s, a);
+            if (e != cudaSuccess || ROWS) return e;
+            return launch_pairs_to_rows(a.pairs, a.phi, N, s);
+        } else if (ROWS) {
+            static_assert(synth_smem<N>() <= 227 * 1024 && synth_col_smem<N>() <= 227 * 1024, "unsplit synthesis pass does not fit");
+            if ((e = set_smem(synth_rows_kernel<N>, synth_smem<N>())) != cudaSuccess) return e;
+            if constexpr (N <= kDrawN) {
+                if (!a.drawn) return cudaErrorInvalidValue;
+                e = launch_next(synth_draw_kernel, dim3((draw_bins(N) + kDrawThreads - 1) / kDrawThreads),
+                                dim3(kDrawThreads), 0, s, a);
+                if (e != cudaSuccess) return e;
             }
+            const int rows = N / 2 + 1;
+            return launch_synth<N>(synth_rows_kernel<N>, dim3((rows + synth_lines<N>() - 1) / synth_lines<N>()),
+                               dim3(synth_threads<N>()), synth_smem<N>(), s, a);
+        } else {
+            if ((e = set_smem(synth_cols_kernel<N>, synth_col_smem<N>())) != cudaSuccess) return e;
+            return launch_synth<N>(synth_cols_kernel<N>, dim3(N / (2 * synth_col_lines<N>())),
+                               dim3(synth_col_threads<N>()), synth_col_smem<N>(), s, a);
         }
     });
 }
