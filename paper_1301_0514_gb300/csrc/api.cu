@@ -381,12 +381,12 @@ int check_passband(const scint_params* p, const double* lambdas, const double* w
 }
 
 // ---- propagation plans (variants of the transfer-function passes) ----------------
-// Default: the one-wavelength passes.  Measured on GB300 (1024^2-8192^2, 8 and 32
-// wavelengths), the packed passes with 16 values per thread and register twiddle bases in
-// both passes are 1-4 % faster when a screen runs alone, but 2.5 % slower when eight
-// screens share the GPU on the batch executor's lanes (their blocks need more shared
-// memory), and the persistent batch kernel runs the one-wavelength passes only.  scint_tune
-// picks a size's fastest variant alone, scint_tune_batch the fastest set for a batch.
+// Default: the one-wavelength passes.  Since these are streamed they are the faster ones at every size: one passband
+// alone against the best packed variant (16 values per thread, register twiddle bases) 0.296 / 0.334 ms (1024^2, 32
+// wavelengths), 1.068 / 1.185 (2048^2), 4.85 / 5.02 (4096^2), 6.03 / 7.63 (8192^2, 8 wavelengths); 48 screens on
+// eight lanes 105.8 / 116.9 ms.  The persistent batch kernel runs the one-wavelength passes only.  The packed
+// passes stay as plans that a caller sets, and as candidates of scint_tune (a size's fastest variant alone) and of
+// scint_tune_batch (the fastest set for a batch).
 std::mutex g_plan_mu;
 std::map<std::pair<int, int>, scint_plan> g_plans;   // (device, n) -> plan
 

@@ -163,7 +163,7 @@ cudaError_t launch_smooth_pass(const SmoothArgs& a, int which, cudaStream_t s);
 struct Track { uint64_t x0, y0, dx, dy; };
 Track make_track(int n, const double* t);    // t = (x0, y0, theta, ds) in pixels
 constexpr int kTracksPerLaunch = 64, kManyTracks = 512;
-// K: the tracks an argument holds (kTracksPerLaunch, or kManyTracks for more: 20 KB of arguments)
+// K: the tracks an argument holds (kTracksPerLaunch, or kManyTracks for more: 16 KB of arguments)
 template <int K>
 struct CurveArgs {
     int n, n_tracks, n_samples;

@@ -25,8 +25,9 @@
 //
 // Block shape: 512 threads, one block per SM; an item is the work of one 512-thread
 // block of the ordinary pass or of two 256-thread blocks, run side by side on the two
-// halves of the block on disjoint shared memory, each half synchronising on its own
-// named barrier (with one block-wide barrier the halves stalled together: 22 % slower).
+// halves of the block on disjoint shared memory, each half (in the columns: each column's
+// team) synchronising on its own named barrier (with one block-wide barrier the halves
+// stalled together: 22 % slower).
 #include <algorithm>
 #include <vector>
 

@@ -76,19 +76,22 @@ prop_cols_kernel(PropArgs a) {
     prop_cols_body<N, CONJ>(a, blockIdx.x, threadIdx.x, smem32);
 }
 
-// ---- streamed passes (rows 512 to 8192, columns of the transfer function 512 to 4096) ------
+// ---- streamed passes (rows, and columns of the transfer function, 512 to 4096) -------------
 // The same arithmetic with the inputs of the next wavelength or line on their way while this one is
 // transformed: without it every warp of a block waited for its loads at the same time, at the
 // head of each wavelength.  The copies need neither registers nor load instructions (a copy by
 // cp.async had cost more than it hid, on the load/store pipe that the line exchanges keep
 // 60 % busy).  The passes are bound by issue slots (105-120 instructions per pixel and wavelength)
-// and by the load/store pipe of the exchanges; per-launch times before and after, ms:
+// and by the load/store pipe of the exchanges; per-launch times before and after (event pairs, which keep the launches
+// apart), ms:
 //                  32 wavelengths                          one wavelength
 //          rows           columns               rows             columns
-//   512    0.102 -> 0.079   0.085 -> 0.078      0.0118 -> 0.0106   0.0098 -> 0.0100
-//   1024   0.176 -> 0.152   0.160 -> 0.140      0.0171 -> 0.0145   0.0131 -> 0.0140
-//   2048   0.625 -> 0.571   0.573 -> 0.490      0.0458 -> 0.0307   0.0414 -> 0.0350
-//   4096   2.501 -> 2.371   2.562 -> 2.463      0.1657 -> 0.1075   0.1637 -> 0.1312
+//   512    0.102 -> 0.080   0.084 -> 0.078      0.0112 -> 0.0111  0.0097 -> 0.0097
+//   1024   0.176 -> 0.155   0.159 -> 0.139      0.0172 -> 0.0152  0.0139 -> 0.0142
+//   2048   0.625 -> 0.573   0.573 -> 0.491      0.0449 -> 0.0317  0.0405 -> 0.0351
+//   4096   2.504 -> 2.382   2.563 -> 2.519      0.1657 -> 0.1075  0.1619 -> 0.1308
+// A whole call at one wavelength in a graph: 512^2 14.5 -> 13.2 us, 1024^2 24.6 -> 22.3.  There the former columns
+// (interleaved lines, a shared twiddle table) with early launches take 13.4 and 22.1 us: no rule for that.
 // The one-FFT columns keep plain loads: with half the transforms per value the copies of 16-byte
 // rows became their bound (4096^2, 8 wavelengths: 0.493 ms, streamed 0.531).
 //   Row pass: the block's phases by one bulk copy into the array that keeps their fixed-point
@@ -344,8 +347,8 @@ cudaError_t launch_cols_stream(const PropArgs& a, const CUtensorMap& tm, cudaStr
 }
 
 // ---- lines of 8192 points: two half lines per team (fft_long) ----------------------------
-// Per launch against 512 threads with sixteen values each: rows 3.70 -> 3.0 ms (8 wavelengths), 0.795 ->
-// 0.495 (one); columns 3.95 -> 2.9 and 1.09 -> 0.56.
+// Per launch against 512 threads with sixteen values each: rows 3.70 -> 3.06 ms (8 wavelengths), 0.797 ->
+// 0.496 (one); columns 3.95 -> 2.9 to 3.2 and 1.08 -> 0.56.
 // Row pass: 256 threads per row, two rows per SM; the phases by bulk copy as above, the taper
 // from its table (no room beside two rows' phases).
 // Column pass: 256 threads and one column per block, two blocks per SM, so that one column's
@@ -567,7 +570,7 @@ bool field_map(CUtensorMap* tm, const float2* work, int n, int count, int strip)
 // Block 1's quarter is the upper half of its half-problem, so it runs fft_long with the halves
 // swapped: W_{N/2}^n changes sign, and array a is always the part the block keeps.
 // Measured per 16384^2 pass at one wavelength, against 512 threads with sixteen values each, one
-// block per SM, whole lines read by both blocks: rows 4.2 -> 3.1 ms, columns 3.1 -> 2.7 ms (with the transpose).
+// block per SM, whole lines read by both blocks: rows 4.24 -> 3.07 ms, columns 3.09 -> 2.75 ms (with the transpose).
 template <int N> __host__ __device__ constexpr int psplit_threads() { return FftPlan<N / 2>::T; }
 template <int N> constexpr size_t conj_row_split_smem() {
     return (size_t)FftPlan<N / 2>::BUF * sizeof(float2) + (size_t)N * sizeof(long long);
@@ -1098,7 +1101,7 @@ __global__ void __launch_bounds__(256) resample_tiled_kernel(const __grid_consta
     }
 }
 
-// Plain form for grids below one tile and scale factors beyond the patch.
+// Plain form for grids below one tile.
 __global__ void resample_kernel(ResampleArgs a) {
     const int n = a.n;
     const size_t total = (size_t)n * n;

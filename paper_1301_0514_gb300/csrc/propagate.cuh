@@ -10,9 +10,9 @@ constexpr int kColEPT = 16;   // values per thread in the column passes
 constexpr size_t kMaxSmem = 227 * 1024;
 
 // Lines longer than one block's shared memory (N = 16384) go to a cluster of two
-// blocks, split by one radix-2 step (prop_*_split_kernel and conj_*_split_kernel in
-// propagate.cu, adj_*_split_kernel in adjoint.cu): each block transforms one parity
-// as a whole N/2-point line.  The kernels below are the unsplit passes.
+// blocks, split by one radix-2 step: each block transforms one parity, as two half lines (prop_*_split_kernel in
+// propagate.cu) or as a whole N/2-point line (conj_*_split_kernel there, adj_*_split_kernel in adjoint.cu).
+// The kernels below are the unsplit passes.
 template <int N> __host__ __device__ constexpr int pcs() { return N >= kSplitN ? 2 : 1; }
 
 // rows per row-pass block, columns per column-pass block (all lines of a block
