@@ -597,6 +597,21 @@ SCINT_DEV void long_split(float2* a, float2* b, float2 w0) {
         long_split<N, M + 1>(a, b, w0);
     }
 }
+// The same with the factors from the table, tw[j] = W_N^j: each rounded once, where W_N^t W_32^m is three times.  Eight
+// loads serve sixteen factors: W_N^(t + (m + 8) T) = -i W_N^(t + m T).
+template <int N>
+SCINT_DEV void long_split_table(float2* a, float2* b, const float2* __restrict__ tw, int t) {
+    constexpr int Q = LongPlan<N>::H / 2;
+#pragma unroll
+    for (int m = 0; m < Q; ++m) {
+        const float2 w = __ldg(tw + t + m * LongPlan<N>::T);
+        const float2 d = a[m] - b[m], e = a[m + Q] - b[m + Q];
+        a[m] = a[m] + b[m];
+        a[m + Q] = a[m + Q] + b[m + Q];
+        b[m] = cmul(d, w);
+        b[m + Q] = cmul(e, make_float2(w.y, -w.x));
+    }
+}
 template <int N, int M = 0>
 SCINT_DEV void long_join(float2* a, float2* b, float2 w0) {
     if constexpr (M < LongPlan<N>::H) {
@@ -606,10 +621,14 @@ SCINT_DEV void long_join(float2* a, float2* b, float2 w0) {
         long_join<N, M + 1>(a, b, w0);
     }
 }
+// w0 = W_N^t; table: tw of long_split_table for the forward step, or NULL
 template <int N, int DIR, int SUB = 0>
 SCINT_DEV void fft_long(float2 (&a)[16], float2 (&b)[16], float2* buf, int t, const TwiddleRegs<float2, N / 2, 16, 4>& tr,
-                        float2 w0) {
-    if constexpr (DIR < 0) long_split<N>(a, b, w0);
+                        float2 w0, const float2* __restrict__ table = nullptr) {
+    if constexpr (DIR < 0) {
+        if (table) long_split_table<N>(a, b, table, t);
+        else long_split<N>(a, b, w0);
+    }
     fft_line_tr<float2, N / 2, DIR, 16, 1, 1, SUB>(a, buf, t, tr);
     fft_line_tr<float2, N / 2, DIR, 16, 1, 1, SUB>(b, buf, t, tr);
     if constexpr (DIR > 0) long_join<N>(a, b, w0);
