@@ -621,16 +621,14 @@ SCINT_DEV void long_join(float2* a, float2* b, float2 w0) {
         long_join<N, M + 1>(a, b, w0);
     }
 }
-// w0 = W_N^t; table: tw of long_split_table for the forward step, or NULL
-template <int N, int DIR, int SUB = 0>
+// w0 = W_N^t; TABLE: the forward step's factors from tw instead (long_split_table)
+template <int N, int DIR, bool TABLE = false>
 SCINT_DEV void fft_long(float2 (&a)[16], float2 (&b)[16], float2* buf, int t, const TwiddleRegs<float2, N / 2, 16, 4>& tr,
-                        float2 w0, const float2* __restrict__ table = nullptr) {
-    if constexpr (DIR < 0) {
-        if (table) long_split_table<N>(a, b, table, t);
-        else long_split<N>(a, b, w0);
-    }
-    fft_line_tr<float2, N / 2, DIR, 16, 1, 1, SUB>(a, buf, t, tr);
-    fft_line_tr<float2, N / 2, DIR, 16, 1, 1, SUB>(b, buf, t, tr);
+                        float2 w0, const float2* __restrict__ tw = nullptr) {
+    if constexpr (DIR < 0 && TABLE) long_split_table<N>(a, b, tw, t);
+    else if constexpr (DIR < 0) long_split<N>(a, b, w0);
+    fft_line_tr<float2, N / 2, DIR, 16>(a, buf, t, tr);
+    fft_line_tr<float2, N / 2, DIR, 16>(b, buf, t, tr);
     if constexpr (DIR > 0) long_join<N>(a, b, w0);
 }
 

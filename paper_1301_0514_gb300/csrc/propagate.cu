@@ -443,7 +443,7 @@ __global__ void __launch_bounds__(LongPlan<N>::T, 2) prop_rows_long_kernel(PropA
             }
             // the one-FFT method has no accurate H to make up for the products' rounding: its factors come from the table
             // (rms error of 3 wavelengths at 8192^2: 3.41e-7 with products, 3.30e-7 before there were half lines)
-            fft_long<N, -1>(va, vb, buf, t, tr, w0, CONJ ? a.tw : nullptr);
+            fft_long<N, -1, CONJ>(va, vb, buf, t, tr, w0, a.tw);
             // every thread is past an exchange, hence done with the phases at the last wavelength
             if (bulk && t == 0 && l + 1 == a.lam.count && y + (int)gridDim.x < N) load_phi(y + gridDim.x);
             float2* dst = a.work + (size_t)l * N * N + strip_index<W>(y, CONJ ? 2 * t : t, N);
